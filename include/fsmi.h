@@ -85,10 +85,10 @@ typedef struct {
     int flags;          /* FSMI_FLAG_* bits, 0 by default */
 } fsmi_params;
 
-/* Exact 2D FSMI evaluates, for each first-hit cell j, the boundary terms of Theorem 1's pair sum
- * within about 5.7 sigma of the cell's centre: every term beyond weighs less than 2^-27 of its
- * factor |C_m - C_{m-1}|, so the MI differs from the full n(n+1) sweep by about one FP32 rounding
- * at most (not bit for bit).
+/* Exact 2D FSMI evaluates, for each first-hit cell j, the terms of Theorem 1's pair sum within about
+ * 5.7 sigma of the cell's centre: what lies beyond on one side weighs less than 2^-24 of the largest
+ * C_k, so the MI differs from the full n(n+1) sweep by about one FP32 rounding at most (not bit for
+ * bit).
  * FSMI_FLAG_FULL_WINDOW widens the window to every term whose Gaussian tail is non-zero in FP32
  * (about 13.3 sigma; the tail underflows to exactly 0 beyond), which gives the full sweep's result
  * bit for bit; FSMI_FLAG_FULL_SWEEP evaluates all n(n+1) terms (both for verification and timing

@@ -22,6 +22,7 @@
 #include "dda2d.cuh"
 #include "fsmi_internal.h"
 #include "gauss_tail.cuh"
+#include "cell_mass.cuh"
 
 namespace fsmi {
 
@@ -48,8 +49,24 @@ __device__ __forceinline__ void carve_2d(float *base, int stride, float *&sl, fl
     sc = sx + stride;
     sp = sc + stride;
 }
-// internal variant id of the full n(n+1) exact sweep (FSMI_FLAG_FULL_SWEEP)
-constexpr int kExactFullSweep = 3;
+// Internal variant ids beside FSMI_EXACT (boundary form), FSMI_APPROX and FSMI_UNIFORM: the full
+// n(n+1) sweep of the boundary form (FSMI_FLAG_FULL_SWEEP), and the exact sum in the mass form of
+// degree 3 and 4.
+constexpr int kExactFullSweep = 3, kExactMass3 = 4, kExactMass4 = 5;
+__host__ __device__ constexpr bool mass_variant(int v) { return v == kExactMass3 || v == kExactMass4; }
+
+// The kernel variant of a call whose cells come from the grid (every width at most sqrt 2 cells).
+// The exact sum takes the mass form (cell_mass.cuh) from sigma = 1 cell on; below that, and for
+// explicit beams, whose cells may be any width, the boundary form. Approx-FSMI stays in boundary form:
+// its band is too short to pay for the sources' polynomials (Delta = 3, 517 poses x 181 beams, R = 181.5:
+// 274 us in mass form, 250 us in boundary form). The exact sum of the 2048x2048 office batch (1024
+// poses x 360 beams, R = 256, sigma = 2) takes 1.69 ms in mass form, 1.86 ms in boundary form.
+inline int grid_variant(const DevParams &p)
+{
+    if (p.variant != FSMI_EXACT) return p.variant;
+    if (p.sigma < kMassSigma4) return p.flags & FSMI_FLAG_FULL_SWEEP ? kExactFullSweep : FSMI_EXACT;
+    return p.sigma >= kMassSigma3 ? kExactMass3 : kExactMass4;
+}
 
 enum { kSrcMap = 0, kSrcBeams = 1, kSrcSets = 2, kSrcTraj = 3 };
 
@@ -370,6 +387,140 @@ __device__ __forceinline__ float approx_pairs_sum(const float2 *LW, const float 
     return r;
 }
 
+// ---- the exact pair sum in mass form ---------------------------------------------------------
+//
+// I = sum_k C_k sum_j P(e_j) G_{k,j}, the lanes holding source cells k (their mass polynomials in
+// registers, cell_mass.cuh) and running over the targets j, which shared memory gives in pairs:
+// Tg[p] = (x_2p, x_2p+1, P_2p, P_2p+1) with x the scaled cell centres, one 16-byte load per pair of
+// targets and two sources. Every term is a product of non-negative factors (C_k of known cells may
+// round below zero), so nothing cancels. Target -1 is the no-return event (P = 0 unless e0 is set);
+// a slot past the last cell has P = 0.
+//
+// A pair of terms costs 7 packed FP32 operations and two ex2 (14 FMA-pipe cycles and 8 SFU cycles per
+// warp at D = 3) where the boundary form costs 10 and two ex2 and two rcp (20 and 24).
+//
+// Windows: a cell whose centre lies beyond the cut adds at most its mass beyond that distance less
+// half its width; kMassCut plus half the widest cell leaves out at most 3e-8 on one side, half an
+// FP32 ulp. (FSMI_FLAG_FULL_WINDOW: kTailCut, beyond which 2^(-d^2) is exactly 0;
+// FSMI_FLAG_FULL_SWEEP: no cut. Both add the same non-zero terms in the same order.)
+constexpr float kMassCut = 4.58f;
+
+// Builds Tg in place over sl and the scratch array after it, from the top pair down (writing Tg[p]
+// overwrites l_4p .. l_4p+3, which only Tg[2p - 1], Tg[2p] and Tg[2p + 1] read: they lie higher, or
+// at p <= 1 in the same step of 32 pairs, whose reads all come before its writes), and replaces P
+// in sp by the cells' scaled widths.
+__device__ __forceinline__ void build_targets(float *sl, float *sp, int n, float cs, float pe0, float mu0)
+{
+    const int lane = lane_id();
+    float4 *Tg = reinterpret_cast<float4 *>(sl);
+    const int pend = (n >> 1) + 1;  // pairs 0 .. n / 2
+    for (int top = (pend + 31) & ~31; top > 0; top -= 32) {
+        const int p = top - 32 + lane;
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float2 w = make_float2(0.0f, 0.0f);
+        const int m = 2 * p;
+        if (m < n) {  // l_m, l_{m+1}, l_{m+2}: m + 2 <= n + 1, inside the array
+            const float2 l2 = *reinterpret_cast<const float2 *>(sl + m);
+            const float2 p2 = *reinterpret_cast<const float2 *>(sp + m);
+            const float l0 = l2.x * cs, l1 = l2.y * cs;
+            v.x = 0.5f * (l0 + l1);
+            v.z = p2.x;
+            w.x = l1 - l0;
+            if (m + 1 < n) {
+                const float l3 = sl[m + 2] * cs;
+                v.y = 0.5f * (l1 + l3);
+                v.w = p2.y;
+                w.y = l3 - l1;
+            }
+        }
+        __syncwarp();
+        if (p < pend) {
+            Tg[p] = v;
+            if (m < n) *reinterpret_cast<float2 *>(sp + m) = w;
+        }
+        __syncwarp();
+    }
+    if (lane == 0) Tg[-1] = make_float4(mu0, mu0, 0.0f, pe0);
+    __syncwarp();
+}
+
+// Exact sum. Sources in rounds of 64 while more than 32 remain, lane i the adjacent cells A = 2i and
+// B = A + 1 of the round, then one per lane. In every round all lanes run over the same number of
+// pairs below and above their own (the fewest that cover every window of the round, by coverage
+// trials from the previous round's counts), clamped to the beam.
+template <int D>
+__device__ __forceinline__ float exact_mass_sum(const float4 *Tg, const float *sc, const float *sw, int n, bool e0, float cut)
+{
+    const int lane = lane_id();
+    const float *Tf = reinterpret_cast<const float *>(Tg);
+    auto xq = [&](int m) { return Tf[4 * (m >> 1) + (m & 1)]; };  // x_m (m >> 1 floors m = -1)
+    const int mlo = e0 ? -1 : 0, plast = (n - 1) >> 1;
+    const float span = xq(n - 1) - xq(0);
+    const float per = span > 0.0f ? __fdividef((float)n, span) : 0.0f;
+    int GN = (int)fminf(cut * per, (float)(n + 1)) >> 1, GP = GN;  // first trial
+    float r = 0.0f;
+    int kb = 0;
+    for (; kb < n; kb += 64) {
+        const bool two = n - kb > 32;  // one source per lane in the last round of at most 32
+        const int k = kb + (two ? 2 * lane : lane);
+        const bool act = k < n, actB = two && k + 1 < n;
+        const int a = act ? k : kb;  // an idle lane shadows the round's first source with weight 0
+        const int b = actB ? a + 1 : a;
+        const int pa = a >> 1;
+        const float xa = xq(a), xb = xq(b);
+        const float below = xa - cut, above = xb + cut;
+        auto neg_ok = [&](int G) {
+            const int m = 2 * (pa - G) - 1;
+            return !act || m < mlo || xq(m) < below;
+        };
+        auto pos_ok = [&](int G) {
+            const int m = 2 * (pa + G) + 2;
+            return !act || m >= n || xq(m) >= above;
+        };
+        if (__all_sync(kFull, neg_ok(GN))) {
+            while (GN > 0 && __all_sync(kFull, neg_ok(GN - 1))) --GN;
+        } else {
+            do ++GN;
+            while (!__all_sync(kFull, neg_ok(GN)));
+        }
+        if (__all_sync(kFull, pos_ok(GP))) {
+            while (GP > 0 && __all_sync(kFull, pos_ok(GP - 1))) --GP;
+        } else {
+            do ++GP;
+            while (!__all_sync(kFull, pos_ok(GP)));
+        }
+        int p = max(pa - GN, -1);
+        const int end = min(pa + GP, plast);
+        const MassSource<D> A = mass_source<D>(xa, sw[a]);
+        f32x2 accA = pack2(0.0f, 0.0f);
+        float a0, a1;
+        if (two) {
+            const MassSource<D> B = mass_source<D>(xb, sw[b]);
+            f32x2 accB = pack2(0.0f, 0.0f);
+#pragma unroll kPair2Unroll
+            for (; p <= end; ++p) {
+                const float4 q = Tg[p];
+                const f32x2 X = pack2(q.x, q.y), P = pack2(q.z, q.w);
+                accA = mass_term<D>(A, X, P, accA);
+                accB = mass_term<D>(B, X, P, accB);
+            }
+            float b0, b1;
+            unpack2(accB, b0, b1);
+            r = fmaf(actB ? sc[b] : 0.0f, b0 + b1, r);
+        } else {
+#pragma unroll kPairUnroll
+            for (; p <= end; ++p) {
+                const float4 q = Tg[p];
+                accA = mass_term<D>(A, pack2(q.x, q.y), pack2(q.z, q.w), accA);
+            }
+        }
+        unpack2(accA, a0, a1);
+        r = fmaf(act ? sc[a] : 0.0f, a0 + a1, r);
+        if (!two) break;
+    }
+    return r;
+}
+
 // Uniform-FSMI (Algorithm 4) from D = inclusive prefix of C (sd), with Algorithm 4's clamps.
 __device__ __forceinline__ float uniform_sum(const float *sd, const float *sp, int n, bool e0, float pe0, int H,
                                              float inv_2h1)
@@ -512,6 +663,15 @@ __device__ __forceinline__ float beam_sum(const DevParams &p, int n, float *sl, 
             const float2 *LW = reinterpret_cast<const float2 *>(sl);
             I = D < kPad2D ? approx_pairs_sum<false>(LW, sc, sp, n, e0, pe0, mu0, D)
                            : approx_pairs_sum<true>(LW, sc, sp, n, e0, pe0, mu0, D);
+        }
+        if (mass_variant(VAR)) {
+            const float mu0 = sl[0] * cs - 0.5f * cs;  // e_0 centre, l_1 - 1/2 (scaled)
+            build_targets(sl, sp, n, cs, e0 ? pe0 : 0.0f, mu0);
+            const float4 *Tg = reinterpret_cast<const float4 *>(sl);
+            float cut = fmaf(0.70710678f, cs, kMassCut);
+            if (p.flags & FSMI_FLAG_FULL_WINDOW) cut = kTailCut;
+            if (p.flags & FSMI_FLAG_FULL_SWEEP) cut = __int_as_float(0x7f800000);
+            I = exact_mass_sum<VAR == kExactMass3 ? 3 : 4>(Tg, sc, sp, n, e0, cut);
         }
         if (VAR == FSMI_UNIFORM) I = uniform_sum(sx, sp, n, e0, pe0, p.H, p.inv_2h1);
         I = warp_sum(I);

@@ -92,10 +92,18 @@ static cudaError_t dispatch(const Src2D &src, const DevParams &p, long long nbea
                             unsigned long long *queue, cudaStream_t s)
 {
     if (nbeams <= 0) return cudaSuccess;
-    switch (p.variant) {
-        case FSMI_EXACT:
-            if (p.flags & FSMI_FLAG_FULL_SWEEP) return launch_variant<kExactFullSweep, SRC>(src, p, nbeams, out, status, queue, s);
-            return launch_variant<FSMI_EXACT, SRC>(src, p, nbeams, out, status, queue, s);
+    int var = p.variant == FSMI_EXACT && (p.flags & FSMI_FLAG_FULL_SWEEP) ? kExactFullSweep : p.variant;
+    if constexpr (SRC != kSrcBeams) {
+        var = grid_variant(p);
+        switch (var) {
+            case kExactMass3: return launch_variant<kExactMass3, SRC>(src, p, nbeams, out, status, queue, s);
+            case kExactMass4: return launch_variant<kExactMass4, SRC>(src, p, nbeams, out, status, queue, s);
+            default: break;
+        }
+    }
+    switch (var) {
+        case FSMI_EXACT: return launch_variant<FSMI_EXACT, SRC>(src, p, nbeams, out, status, queue, s);
+        case kExactFullSweep: return launch_variant<kExactFullSweep, SRC>(src, p, nbeams, out, status, queue, s);
         case FSMI_APPROX: return launch_variant<FSMI_APPROX, SRC>(src, p, nbeams, out, status, queue, s);
         default: return launch_variant<FSMI_UNIFORM, SRC>(src, p, nbeams, out, status, queue, s);
     }
@@ -163,6 +171,10 @@ static cudaError_t prepare_src()
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_2d<kExactFullSweep, SRC>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_2d<FSMI_APPROX, SRC>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_2d<FSMI_UNIFORM, SRC>);
+    if constexpr (SRC != kSrcBeams) {
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_2d<kExactMass3, SRC>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_2d<kExactMass4, SRC>);
+    }
     return e;
 }
 

@@ -3,6 +3,8 @@
 // The sets form one ordered list of work items (a 2D beam or a 3D ray each); warps take items in
 // that order from the work queue, so each set finishes roughly in arrival order, and the kernel can
 // record when every item completed (from which per-set latencies follow).
+#include <type_traits>
+
 #include "eval2d.cuh"
 #include "evalrle.cuh"
 
@@ -448,10 +450,11 @@ cudaError_t launch_mixed_planned(const MixedSrc &src, const DevParams &d2, const
             p.nmax = min(mix_bound(c), d3.nmax);
             MixedSrc sc3 = src;
             sc3.has2d = false;
-            e = thm5_of(p) ? launch_mixed_variant<VAR, kMix3DThm5>(sc3, n2, p, nitems, out, times, status, queue, s,
-                                                                  plan, kMixClasses + c)
-                           : launch_mixed_variant<VAR, kMix3DOther>(sc3, n2, p, nitems, out, times, status, queue, s,
-                                                                   plan, kMixClasses + c);
+            // (a 3D class holds no 2D path: one instantiation whatever the 2D variant)
+            e = thm5_of(p) ? launch_mixed_variant<FSMI_EXACT, kMix3DThm5>(sc3, n2, p, nitems, out, times, status, queue,
+                                                                         s, plan, kMixClasses + c)
+                           : launch_mixed_variant<FSMI_EXACT, kMix3DOther>(sc3, n2, p, nitems, out, times, status, queue,
+                                                                          s, plan, kMixClasses + c);
             if (e != cudaSuccess) return e;
         }
     }
@@ -479,24 +482,18 @@ cudaError_t launch_eval_mixed(const float *map, int W, int H, const float4 *gain
     if (p3) d3 = *p3;
     MixedSrc src{map, W, H, gains, poses2, P2, dirs2, B2, p2 != nullptr, vols, nvol, poses3, P3, dirs3, R3,
                  p3 != nullptr, sets, nsets};
-    if (plan) {
-        switch (d2.variant) {
-            case FSMI_EXACT:
-                if (d2.flags & FSMI_FLAG_FULL_SWEEP)
-                    return launch_mixed_planned<kExactFullSweep>(src, d2, d3, nitems, out, times, status, queue, plan, s);
-                return launch_mixed_planned<FSMI_EXACT>(src, d2, d3, nitems, out, times, status, queue, plan, s);
-            case FSMI_APPROX:
-                return launch_mixed_planned<FSMI_APPROX>(src, d2, d3, nitems, out, times, status, queue, plan, s);
-            default: return launch_mixed_planned<FSMI_UNIFORM>(src, d2, d3, nitems, out, times, status, queue, plan, s);
-        }
-    }
-    switch (d2.variant) {
-        case FSMI_EXACT:
-            if (d2.flags & FSMI_FLAG_FULL_SWEEP)
-                return launch_mixed_variant<kExactFullSweep>(src, d2, d3, nitems, out, times, status, queue, s);
-            return launch_mixed_variant<FSMI_EXACT>(src, d2, d3, nitems, out, times, status, queue, s);
-        case FSMI_APPROX: return launch_mixed_variant<FSMI_APPROX>(src, d2, d3, nitems, out, times, status, queue, s);
-        default: return launch_mixed_variant<FSMI_UNIFORM>(src, d2, d3, nitems, out, times, status, queue, s);
+    auto go = [&](auto var) {
+        constexpr int VAR = decltype(var)::value;
+        return plan ? launch_mixed_planned<VAR>(src, d2, d3, nitems, out, times, status, queue, plan, s)
+                    : launch_mixed_variant<VAR>(src, d2, d3, nitems, out, times, status, queue, s);
+    };
+    switch (grid_variant(d2)) {
+        case kExactMass3: return go(std::integral_constant<int, kExactMass3>{});
+        case kExactMass4: return go(std::integral_constant<int, kExactMass4>{});
+        case FSMI_EXACT: return go(std::integral_constant<int, FSMI_EXACT>{});
+        case kExactFullSweep: return go(std::integral_constant<int, kExactFullSweep>{});
+        case FSMI_APPROX: return go(std::integral_constant<int, FSMI_APPROX>{});
+        default: return go(std::integral_constant<int, FSMI_UNIFORM>{});
     }
 }
 
@@ -506,8 +503,6 @@ static cudaError_t prepare_mixed_var()
     cudaFuncAttributes a;
     cudaError_t e = cudaFuncGetAttributes(&a, k_eval_mixed<VAR, kMixAny>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_mixed<VAR, kMix2D>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_mixed<VAR, kMix3DOther>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_mixed<VAR, kMix3DThm5>);
     return e;
 }
 
@@ -520,6 +515,10 @@ cudaError_t prepare_mixed()
 {
     cudaFuncAttributes a;
     cudaError_t e = cudaFuncGetAttributes(&a, k_mixed_plan);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_mixed<FSMI_EXACT, kMix3DOther>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_mixed<FSMI_EXACT, kMix3DThm5>);
+    if (e == cudaSuccess) e = prepare_mixed_var<kExactMass3>();
+    if (e == cudaSuccess) e = prepare_mixed_var<kExactMass4>();
     if (e == cudaSuccess) e = prepare_mixed_var<FSMI_EXACT>();
     if (e == cudaSuccess) e = prepare_mixed_var<kExactFullSweep>();
     if (e == cudaSuccess) e = prepare_mixed_var<FSMI_APPROX>();
