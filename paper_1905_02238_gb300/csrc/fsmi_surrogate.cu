@@ -490,10 +490,6 @@ __device__ __forceinline__ unsigned pack_bf16x2(float lo, float hi)
     return *reinterpret_cast<const unsigned *>(&v);
 }
 
-__device__ __forceinline__ void ldsm_x2(unsigned addr, unsigned &r0, unsigned &r1)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
-}
 
 __device__ __forceinline__ void mma_bf16_k8(float (&c)[4], unsigned a0, unsigned a1, unsigned b0)
 {
@@ -734,179 +730,223 @@ cudaError_t dgrad_conv(int N, int Lin, const float *dz, const bf16 *w, const flo
     return cudaGetLastError();
 }
 
-// Conv activations [rows][32 channels] (64 B per row) are kept in 128-byte lines of two rows;
-// the 16-byte chunk (row parity, channel quarter) of line L sits at chunk ((parity << 2) | q) ^
-// (L & 7). The eight rows 2t + k - 1 (t = t0 .. t0 + 7) that one ldmatrix phase reads for a conv
-// tap then land in eight different bank groups, and so do the eight rows one accumulator store
-// writes. Implicit GEMM: the im2col operand is addressed row by row, never materialised.
-__device__ __forceinline__ int act_chunk(int r, int q)
+// ---- the conv stack in registers ------------------------------------------------------------------
+//
+// One warp per beam. An accumulator tile of mma.m16n8k16 holds (row g, columns 2w, 2w + 1) and
+// (row g + 8, the same), g = lane / 4, w = lane % 4; packed to BF16 pairs that is the A operand
+// of the next layer's MMA for the same rows. A stride-2 conv's row t reads its input at positions
+// 2t - 1, 2t, 2t + 1, so the layers are computed for strips of 16 positions t with equal residues:
+// for conv3's positions u = u0 .. u0 + 15, conv2 at 2u and 2u + 1, conv1 at 4u .. 4u + 3. Each strip is
+// then the next layer's operand for one tap as it stands; the remaining tap, position 4u - 1 (2u - 1), is
+// the strip of 4u + 3 (2u + 1) one row down, two shuffles per pair of registers. No activation
+// goes through shared memory: a beam writes its profile there (1 KB) and reads it as conv1's operand.
+//
+// What bounds it: the kernel with the activations in shared memory moved about 700 wavefronts of
+// shared memory per beam (its pipe 78 % busy, the tensor pipe 39 %) and 1,835 warp instructions; this one
+// moves 185 and issues 1,000, and the tensor pipe (62 % busy) is the bound. 4096 x 360 beams: 2.65 ms
+// against 4.27 ms. Three blocks of four warps per SM leave 168 registers, which hold conv2's weight
+// fragments. Measured on the same batch, conv and fc together: 3.29 ms so; 3.32 ms with four blocks and
+// conv2's weights read per strip, 3.38 - 3.61 ms with the next beam's samples fetched ahead (registers),
+// 3.78 ms with both strips of a beam unrolled.
+constexpr int kConvWarps = 4;
+constexpr int kS2 = 104;  // W2 / W3 row stride (bf16): 208 B, eight rows in eight bank groups
+constexpr int kXWords = 4 + kL;  // a beam's profile, with zeros before it
+// block: W1 [32][8], W2 / W3 [32][104] bf16, kL zero words, then each warp's profile
+constexpr int kConvSmem = kCh * 8 * 2 + 2 * kCh * kS2 * 2 + kL * 4 + kConvWarps * kXWords * 4;
+
+// relu(acc + b) as bf16 pairs: P[nt][h] = columns 8 nt + 2w, + 1 of row g + 8 h
+__device__ __forceinline__ void relu_pack(const float (&acc)[4][4], const float2 (&b)[4], unsigned (&P)[4][2])
 {
-    const int line = r >> 1;
-    return line * 8 + ((((r & 1) << 2) | q) ^ (line & 7));  // in 16-byte units
+    const __nv_bfloat162 zero = __floats2bfloat162_rn(0.0f, 0.0f);
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const __nv_bfloat162 v = __hmax2(__floats2bfloat162_rn(acc[nt][2 * h] + b[nt].x, acc[nt][2 * h + 1] + b[nt].y), zero);
+            P[nt][h] = *reinterpret_cast<const unsigned *>(&v);
+        }
 }
 
-constexpr int kConvWarps = 8;
-constexpr int kS2 = 104;  // W2 / W3 row stride (bf16): 208 B, eight rows in eight bank groups
-// per-warp buffers in 16-byte units: act1 (128 rows), then a 4 KB region that holds first the
-// profile x (64 units) and conv1's operand A1 (128 rows of 16 B), later act2 (64 rows)
-constexpr int kAct1Units = 128 * 4, kRegUnits = 256;
-constexpr int kConvWarpUnits = kAct1Units + kRegUnits;
-// block: W1 [32][8], W2 / W3 [32][104] bf16, biases, one zero chunk
-constexpr int kConvWBytes = kCh * 8 * 2 + 2 * kCh * kS2 * 2 + 3 * kCh * 4 + 16;
-
-// relu(acc + b) as bf16 pairs into a swizzled activation buffer (rows mt * 16 + g, + 8)
-__device__ __forceinline__ void store_act_swz(uint4 *act, const float *b, int mt, const float (&acc)[4][4])
+// The strip one row down: row g takes row g - 1, row 0 the last row of the strip before (carry, which
+// then holds this strip's last row).
+__device__ __forceinline__ void shift_rows(const unsigned (&P)[4][2], unsigned (&carry)[4], unsigned (&S)[4][2])
 {
-    const int lane = lane_id(), g = lane >> 2, w = lane & 3;
+    const int lane = lane_id();
+    const bool first = lane < 4;
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
-        const int c = nt * 8 + 2 * w;
-        const int r0 = mt * 16 + g;
-        unsigned *p0 = reinterpret_cast<unsigned *>(act + act_chunk(r0, nt)) + w;
-        unsigned *p1 = reinterpret_cast<unsigned *>(act + act_chunk(r0 + 8, nt)) + w;
-        *p0 = pack_bf16x2(relu(acc[nt][0] + b[c]), relu(acc[nt][1] + b[c + 1]));
-        *p1 = pack_bf16x2(relu(acc[nt][2] + b[c]), relu(acc[nt][3] + b[c + 1]));
+        const unsigned lo = __shfl_sync(kFull, P[nt][0], lane + 28), hi = __shfl_sync(kFull, P[nt][1], lane + 28);
+        S[nt][0] = first ? carry[nt] : lo;
+        S[nt][1] = first ? lo : hi;
+        carry[nt] = hi;
     }
 }
 
-// Weight fragments of a K = 96 conv layer for all 6 k-steps and 4 n8 tiles.
-__device__ __forceinline__ void load_wfrag(const bf16 *Wt, unsigned (&bw)[6][4][2])
+// Weight fragments of k-step ks (16 of the K = 96 inputs) of a conv layer for the four n8 tiles
+__device__ __forceinline__ void load_wfrag(const bf16 *Wt, int ks, unsigned (&bw)[4][2])
 {
     const int lane = lane_id();
 #pragma unroll
-    for (int ks = 0; ks < 6; ++ks)
-#pragma unroll
-        for (int np = 0; np < 2; ++np) {
-            const int row = np * 16 + (lane & 7) + 8 * (lane >> 4);
-            ldsm_x4(smem_u32(Wt + row * kS2 + ks * 16 + 8 * ((lane >> 3) & 1)), bw[ks][2 * np][0], bw[ks][2 * np][1],
-                    bw[ks][2 * np + 1][0], bw[ks][2 * np + 1][1]);
-        }
-}
-
-// One m16 x n32 strip of a stride-2, K = 96 conv from the swizzled activations `in` (Lin rows):
-// im2col row t, k-step ks (tap ks / 2, channel half ks % 2) is input row 2t + ks / 2 - 1.
-__device__ __forceinline__ void conv_strip_k96(const uint4 *in, const uint4 *zero, int mt, const unsigned (&bw)[6][4][2],
-                                               float (&acc)[4][4])
-{
-    const int lane = lane_id();
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.0f;
-    const int t = mt * 16 + (lane & 15);
-#pragma unroll
-    for (int ks = 0; ks < 6; ++ks) {
-        const int r = 2 * t + (ks >> 1) - 1;
-        const int q = ((ks & 1) << 1) | (lane >> 4);
-        const uint4 *src = r >= 0 ? in + act_chunk(r, q) : zero;
-        unsigned a0, a1, a2, a3;
-        ldsm_x4(smem_u32(src), a0, a1, a2, a3);
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) mma_bf16(acc[nt], a0, a1, a2, a3, bw[ks][nt][0], bw[ks][nt][1]);
+    for (int np = 0; np < 2; ++np) {
+        const int row = np * 16 + (lane & 7) + 8 * (lane >> 4);
+        ldsm_x4(smem_u32(Wt + row * kS2 + ks * 16 + 8 * ((lane >> 3) & 1)), bw[2 * np][0], bw[2 * np][1],
+                bw[2 * np + 1][0], bw[2 * np + 1][1]);
     }
 }
 
-// The conv stack of one beam. x: profile as 256 words (bf16 pairs) in the warp's region; h0 row
-// (1024 bf16, index t * 32 + c) to global memory.
-__device__ void conv_stack(uint4 *act1, uint4 *reg, const uint4 *zero, const bf16 *sW1, const bf16 *sW2,
-                           const bf16 *sW3, const float *sb, bf16 *__restrict__ h0)
+// acc += (channels 16 hh .. of one tap's strip P) W
+__device__ __forceinline__ void tap_mma(float (&acc)[4][4], const unsigned (&P)[4][2], int hh, const unsigned (&bw)[4][2])
 {
-    const int lane = lane_id();
-    const unsigned *x = reinterpret_cast<const unsigned *>(reg);  // x[i] = (o, inside) of sample i
-    uint4 *A1 = reg + 64;                                          // 128 rows x 16 B
-    // conv1 operand: A1[t] = {x[2t-1], x[2t], x[2t+1], 0} (k * 2 + ci order, K padded to 8)
-    for (int t = lane; t < 128; t += 32)
-        A1[t] = make_uint4(t > 0 ? x[2 * t - 1] : 0u, x[2 * t], x[2 * t + 1], 0u);
-    __syncwarp();
-    float acc[4][4];
-    {
-        unsigned b[4];  // W1 fragments of the four n8 tiles (K = 8)
-        ldsm_x4(smem_u32(sW1 + lane * 8), b[0], b[1], b[2], b[3]);
-        for (int mt = 0; mt < 8; ++mt) {
-            unsigned a0, a1;
-            ldsm_x2(smem_u32(A1 + mt * 16 + (lane & 15)), a0, a1);
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.0f;
-                mma_bf16_k8(acc[nt], a0, a1, b[nt]);
-            }
-            store_act_swz(act1, sb, mt, acc);
-        }
-    }
-    __syncwarp();
-    unsigned bw[6][4][2];
-    load_wfrag(sW2, bw);
-    uint4 *act2 = reg;  // x and A1 are dead
-    for (int mt = 0; mt < 4; ++mt) {
-        conv_strip_k96(act1, zero, mt, bw, acc);
-        store_act_swz(act2, sb + kCh, mt, acc);
-    }
-    __syncwarp();
-    load_wfrag(sW3, bw);
-    const int g = lane >> 2, c2 = 2 * (lane & 3);
-    const float *b3 = sb + 2 * kCh;
-    for (int mt = 0; mt < 2; ++mt) {
-        conv_strip_k96(act2, zero, mt, bw, acc);
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int c = nt * 8 + c2, t0 = mt * 16 + g;
-            *reinterpret_cast<unsigned *>(h0 + t0 * kCh + c) =
-                pack_bf16x2(relu(acc[nt][0] + b3[c]), relu(acc[nt][1] + b3[c + 1]));
-            *reinterpret_cast<unsigned *>(h0 + (t0 + 8) * kCh + c) =
-                pack_bf16x2(relu(acc[nt][2] + b3[c]), relu(acc[nt][3] + b3[c + 1]));
-        }
-    }
-    __syncwarp();
+    for (int nt = 0; nt < 4; ++nt)
+        mma_bf16(acc[nt], P[2 * hh][0], P[2 * hh][1], P[2 * hh + 1][0], P[2 * hh + 1][1], bw[nt][0], bw[nt][1]);
 }
 
 // Conv stack for N beams: profiles from the map (map != nullptr; beam n = pose n / B, direction
-// n % B) or given (x [N][256] bf16 pairs). h0 [N][1024] bf16.
-__global__ void __launch_bounds__(kConvWarps * 32)
+// n % B) or given (x [N][256] bf16 pairs). h0 [N][1024] bf16 (index t * 32 + c).
+__global__ void __launch_bounds__(kConvWarps * 32, 3)
     k_conv_infer(const float *__restrict__ map, int W, int H, const int32_t *__restrict__ poses,
                  const int32_t *__restrict__ dirs, int B, int keep, const __nv_bfloat162 *__restrict__ xg, long long N,
                  const bf16 *__restrict__ w, const float *__restrict__ params, bf16 *__restrict__ h0,
-                 unsigned long long *queue)
+                 unsigned long long *queue, int chunk)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    bf16 *sW1 = (bf16 *)smem_raw;        // [32][8]
-    bf16 *sW2 = sW1 + kCh * 8;           // [32][104]
-    bf16 *sW3 = sW2 + kCh * kS2;         // [32][104]
-    float *sb = (float *)(sW3 + kCh * kS2);  // b1, b2, b3
-    uint4 *zero = (uint4 *)(sb + 3 * kCh);
-    uint4 *wbase = zero + 1 + (size_t)(threadIdx.x >> 5) * kConvWarpUnits;
-    uint4 *act1 = wbase, *reg = wbase + kAct1Units;
+    bf16 *sW1 = (bf16 *)smem_raw;  // [32][8]
+    bf16 *sW2 = sW1 + kCh * 8;     // [32][104]
+    bf16 *sW3 = sW2 + kCh * kS2;   // [32][104], row 8 nt + n = output channel 8 (n / 2) + 2 nt + n % 2
+    unsigned *zero = (unsigned *)(sW3 + kCh * kS2);
+    unsigned *xs = zero + kL + (threadIdx.x >> 5) * kXWords + 4;
     for (int e = threadIdx.x; e < kCh * 8; e += blockDim.x) {
         const int c = e / 8, kk = e % 8;
         sW1[e] = kk < kK * kCin ? w[oW1 + c * kK * kCin + kk] : __float2bfloat16_rn(0.0f);
     }
     for (int e = threadIdx.x; e < kCh * kS2; e += blockDim.x) {
-        const int c = e / kS2, kk = e % kS2;
-        sW2[e] = kk < kK * kCh ? w[oW2 + c * kK * kCh + kk] : __float2bfloat16_rn(0.0f);
-        sW3[e] = kk < kK * kCh ? w[oW3 + c * kK * kCh + kk] : __float2bfloat16_rn(0.0f);
+        const int r = e / kS2, kk = e % kS2, c3 = 8 * ((r & 7) >> 1) + 2 * (r >> 3) + (r & 1);
+        sW2[e] = kk < kK * kCh ? w[oW2 + r * kK * kCh + kk] : __float2bfloat16_rn(0.0f);
+        sW3[e] = kk < kK * kCh ? w[oW3 + c3 * kK * kCh + kk] : __float2bfloat16_rn(0.0f);
     }
-    for (int e = threadIdx.x; e < kCh; e += blockDim.x) {
-        sb[e] = params[oB1 + e];
-        sb[kCh + e] = params[oB2 + e];
-        sb[2 * kCh + e] = params[oB3 + e];
-    }
-    if (threadIdx.x == 0) *zero = make_uint4(0u, 0u, 0u, 0u);
+    for (int e = threadIdx.x; e < kL; e += blockDim.x) zero[e] = 0u;
+    const int lane = lane_id(), g = lane >> 2, wq = lane & 3;
+    if (lane < 4) xs[lane - 4] = 0u;  // position -1
     __syncthreads();
-    const int lane = lane_id();
-    __nv_bfloat162 *xs = reinterpret_cast<__nv_bfloat162 *>(reg);
-    for_each_item(N, queue, 4, [&](long long n) {
-        if (map) {
-            const int32_t *pose = poses + 4 * (n / B);
-            int dx, dy;
-            beam_dir_2d(pose, dirs + 2 * (n % B), dx, dy);
-            for (int i = lane; i < kL; i += 32) {
-                float o, in;
-                sample_2d(map, W, H, pose[0], pose[1], dx, dy, i, keep, o, in);
-                xs[i] = __floats2bfloat162_rn(o, in);
+    // biases of this lane's columns (conv3: channels 8 w + 2 nt, + 1), W1's fragments
+    float2 b1[4], b2[4], b3[4];
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+        const int c = 8 * nt + 2 * wq, c3 = 8 * wq + 2 * nt;
+        b1[nt] = make_float2(params[oB1 + c], params[oB1 + c + 1]);
+        b2[nt] = make_float2(params[oB2 + c], params[oB2 + c + 1]);
+        b3[nt] = make_float2(params[oB3 + c3], params[oB3 + c3 + 1]);
+    }
+    unsigned bw1[4], bw2[6][4][2];
+    ldsm_x4(smem_u32(sW1 + lane * 8), bw1[0], bw1[1], bw1[2], bw1[3]);
+#pragma unroll
+    for (int ks = 0; ks < 6; ++ks) load_wfrag(sW2, ks, bw2[ks]);
+    // conv1's operand for position p: taps 0 .. 2 are the words x[2p - 1 + w], the fourth is zero
+    const unsigned *xa = wq < 3 ? xs + 8 * g + wq - 1 : zero;
+    // a warp takes `chunk` (<= 32) consecutive beams per queue grab, lane j the j-th's origin and direction
+    for (;;) {
+        unsigned long long b0 = 0;
+        if (lane == 0) b0 = atomicAdd(queue, (unsigned long long)chunk);
+        b0 = __shfl_sync(kFull, b0, 0);
+        if ((long long)b0 >= N) break;
+        const int nb = (int)min((long long)chunk, N - (long long)b0);
+        int ox = 0, oy = 0, dx = 0, dy = 0;
+        if (map && lane < nb) {
+            const long long n = (long long)b0 + lane;
+            int pi, bi;
+            if (n <= 0x7fffffffLL) {  // 32-bit division, the common case
+                pi = (int)((unsigned)n / (unsigned)B);
+                bi = (int)((unsigned)n - (unsigned)pi * (unsigned)B);
+            } else {
+                pi = (int)(n / B);
+                bi = (int)(n % B);
             }
-        } else {
-            for (int i = lane; i < kL; i += 32) xs[i] = xg[n * kL + i];
+            const int32_t *pose = poses + 4 * (size_t)pi;
+            ox = pose[0];
+            oy = pose[1];
+            beam_dir_2d(pose, dirs + 2 * (size_t)bi, dx, dy);
         }
-        __syncwarp();
-        conv_stack(act1, reg, zero, sW1, sW2, sW3, sb, h0 + n * kFlat);
-    });
+        for (int j = 0; j < nb; ++j) {
+            const long long n = (long long)b0 + j;
+            if (map) {
+                // sample i lies in the cell floor of the Q31 position (o << 15) + (2 i + 1) d; the low 32
+                // bits of the shifted position are the cell inside the map and at least its extent outside
+                const int sx = __shfl_sync(kFull, ox, j), sy = __shfl_sync(kFull, oy, j);
+                const int ex = __shfl_sync(kFull, dx, j), ey = __shfl_sync(kFull, dy, j);
+                long long px = ((long long)sx << 15) + (2LL * lane + 1) * ex;
+                long long py = ((long long)sy << 15) + (2LL * lane + 1) * ey;
+                float o[kL / 32];
+                bool in[kL / 32];
+#pragma unroll
+                for (int k = 0; k < kL / 32; ++k) {
+                    const unsigned cx = (unsigned)(px >> 31), cy = (unsigned)(py >> 31);
+                    in[k] = lane + 32 * k < keep && cx < (unsigned)W && cy < (unsigned)H;
+                    o[k] = in[k] ? __ldg(map + ((size_t)cy * W + cx)) : 0.0f;
+                    px += 64LL * ex;
+                    py += 64LL * ey;
+                }
+#pragma unroll
+                for (int k = 0; k < kL / 32; ++k) xs[lane + 32 * k] = pack_bf16x2(o[k], in[k] ? 1.0f : 0.0f);
+            } else {
+                const unsigned *xr = reinterpret_cast<const unsigned *>(xg) + n * kL;
+#pragma unroll
+                for (int k = 0; k < kL / 32; ++k) xs[lane + 32 * k] = xr[lane + 32 * k];
+            }
+            __syncwarp();
+            unsigned carry1[4] = {0u, 0u, 0u, 0u}, carry2[4] = {0u, 0u, 0u, 0u};
+#pragma unroll 1
+            for (int s = 0; s < 2; ++s) {  // u = 16 s + row
+                unsigned P[4][4][2], S[4][2];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const unsigned *x = xa + 128 * s + 2 * r;
+                    const unsigned a0 = x[0], a1 = x[wq < 3 ? 64 : 0];
+                    float acc[4][4];
+#pragma unroll
+                    for (int nt = 0; nt < 4; ++nt) {
+                        acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.0f;
+                        mma_bf16_k8(acc[nt], a0, a1, bw1[nt]);
+                    }
+                    relu_pack(acc, b1, P[r]);
+                }
+                shift_rows(P[3], carry1, S);
+                float ev[4][4] = {}, od[4][4] = {};
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    tap_mma(ev, S, hh, bw2[hh]);
+                    tap_mma(od, P[1], hh, bw2[hh]);
+                }
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    tap_mma(ev, P[0], hh, bw2[2 + hh]);
+                    tap_mma(od, P[2], hh, bw2[2 + hh]);
+                }
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    tap_mma(ev, P[1], hh, bw2[4 + hh]);
+                    tap_mma(od, P[3], hh, bw2[4 + hh]);
+                }
+                unsigned E[4][2], O[4][2];
+                relu_pack(ev, b2, E);
+                relu_pack(od, b2, O);
+                shift_rows(O, carry2, S);
+                float acc[4][4] = {};
+#pragma unroll
+                for (int ks = 0; ks < 6; ++ks) {
+                    unsigned bw[4][2];
+                    load_wfrag(sW3, ks, bw);
+                    tap_mma(acc, ks < 2 ? S : ks < 4 ? E : O, ks & 1, bw);
+                }
+                unsigned Q[4][2];
+                relu_pack(acc, b3, Q);  // lane w: channels 8 w .. 8 w + 7 of rows g and g + 8
+                uint4 *dst = reinterpret_cast<uint4 *>(h0 + n * kFlat + (16 * s + g) * kCh + 8 * wq);
+                dst[0] = make_uint4(Q[0][0], Q[1][0], Q[2][0], Q[3][0]);
+                dst[kCh] = make_uint4(Q[0][1], Q[1][1], Q[2][1], Q[3][1]);  // 8 rows of 32 bf16 further
+            }
+            __syncwarp();
+        }
+    }
 }
 
 // ---- fc1 + ReLU + fc2 on the 5th-generation tensor cores (tcgen05, accumulators in TMEM) ------------
@@ -1387,7 +1427,7 @@ cudaError_t launch_surrogate_infer(const float *map, int W, int H, const int32_t
     const bf16 *w = (const bf16 *)wbf16;
     unsigned long long *queue = (unsigned long long *)ws;
     bf16 *h0 = (bf16 *)((char *)ws + kQueueBytes);
-    const size_t smem_conv = (size_t)kConvWBytes + (size_t)kConvWarps * kConvWarpUnits * 16;
+    const size_t smem_conv = kConvSmem;
     cudaError_t e = cudaFuncSetAttribute(k_conv_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_conv);
     if (e != cudaSuccess) return e;
     int occ = 0;
@@ -1398,8 +1438,10 @@ cudaError_t launch_surrogate_infer(const float *map, int W, int H, const int32_t
     if (e != cudaSuccess) return e;
     long long grid = (long long)sm_count() * occ;
     if (grid > (N + kConvWarps - 1) / kConvWarps) grid = (N + kConvWarps - 1) / kConvWarps;
+    const long long chunk = N / (grid * kConvWarps * 8);  // eight grabs per warp at least, up to 8 beams each
     k_conv_infer<<<(unsigned)grid, kConvWarps * 32, smem_conv, s>>>(map, W, H, poses, dirs, B, keep,
-                                                                     (const __nv_bfloat162 *)x, N, w, params, h0, queue);
+                                                                     (const __nv_bfloat162 *)x, N, w, params, h0, queue,
+                                                                     (int)std::max(1LL, std::min(8LL, chunk)));
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const long long tiles = (N + kTcRows - 1) / kTcRows;
