@@ -589,51 +589,97 @@ __device__ __forceinline__ int beam_cells(const float *__restrict__ map, int W, 
     const int lane = lane_id();
     int dx, dy;
     beam_dir(pose, ux, uy, dx, dy);
-    const int n = dda_warp(W, H, pose[0], pose[1], dx, dy, rfix, rend, cap, (int *)sx, sl);
-    if (n < 0) return -1;
     const unsigned ncell = (unsigned)W * (unsigned)H;
-    bool bad = false;
-    if (gains) {
-        // four cells per lane in flight: all ids, then all gathers, then all stores
-        constexpr int kG = 4;
-        for (int i0 = lane; i0 < n; i0 += 32 * kG) {
-            unsigned id[kG];
-            float4 v[kG];
+    Geo g;
+    int K;
+    if (!beam_geo(W, H, pose[0], pose[1], dx, dy, rfix, rend, g, K)) return 0;
+    float lend = 0.0f;
+    bool by_range, bad = false;
+    int n = -1;
+    Fixed f;
+    const bool fixed = fixed_setup(g, f) && fixed_cells(f, K) <= cap;
+    if (gains && fixed) {
+        // traversal and gather in one pass, two chunks of intervals (up to four cells per lane) in
+        // flight: the gathers go out before any of their results is stored
+        const int stepm = g.xmaj ? g.sm * g.W : g.sm;
+        n = fixed_run<2>(g, f, K,
+                         [&](const Interval(&v)[2]) {
+                             float4 a[2], b[2];
 #pragma unroll
-            for (int k = 0; k < kG; ++k) {
-                const int i = i0 + 32 * k;
-                id[k] = i < n ? (unsigned)((const int *)sx)[i] : ncell;
-                bad |= i < n && id[k] >= ncell;  // cannot happen for a consistent traversal; never read out of bounds
-            }
+                             for (int u = 0; u < 2; ++u) {
+                                 const unsigned i1 = v[u].ok1 ? (unsigned)v[u].id : ncell;
+                                 const unsigned i2 = v[u].ok2 ? (unsigned)(v[u].id + stepm) : ncell;
+                                 bad |= (v[u].ok1 && i1 >= ncell) || (v[u].ok2 && i2 >= ncell);
+                                 a[u] = b[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                                 if (i1 < ncell) a[u] = __ldg(gains + i1);
+                                 if (i2 < ncell) b[u] = __ldg(gains + i2);
+                                 if (TRAJ && i1 < ncell && __ldg(stamps + i1) < state) a[u].y = a[u].z = 0.0f;
+                                 if (TRAJ && i2 < ncell && __ldg(stamps + i2) < state) b[u].y = b[u].z = 0.0f;
+                             }
 #pragma unroll
-            for (int k = 0; k < kG; ++k) {
-                v[k] = id[k] < ncell ? __ldg(gains + id[k]) : make_float4(0.f, 0.f, 0.f, 0.f);
-                if (TRAJ && id[k] < ncell && __ldg(stamps + id[k]) < state) v[k].y = v[k].z = 0.0f;
-            }
-#pragma unroll
-            for (int k = 0; k < kG; ++k) {
-                const int i = i0 + 32 * k;
-                if (i < n) {
-                    sp[i] = v[k].x;
-                    sc[i] = v[k].y;
-                    sx[i] = v[k].z;
-                }
-            }
+                             for (int u = 0; u < 2; ++u) {
+                                 if (v[u].ok1) {
+                                     const int i = v[u].pos;
+                                     sl[i] = v[u].lam1;
+                                     sp[i] = a[u].x;
+                                     sc[i] = a[u].y;
+                                     sx[i] = a[u].z;
+                                 }
+                                 if (v[u].ok2) {
+                                     const int i = v[u].pos + 1;
+                                     sl[i] = v[u].lam2;
+                                     sp[i] = b[u].x;
+                                     sc[i] = b[u].y;
+                                     sx[i] = b[u].z;
+                                 }
+                             }
+                         },
+                         lend, by_range);
+        __syncwarp();
+    }
+    if (n < 0) {  // ids first, then per cell
+        bad = false;
+        int *ids = (int *)sx;
+        if (fixed && !gains) {
+            const int stepm = g.xmaj ? g.sm * g.W : g.sm;
+            n = fixed_run<1>(g, f, K,
+                             [&](const Interval(&v)[1]) {
+                                 if (v[0].ok1) {
+                                     ids[v[0].pos] = v[0].id;
+                                     sl[v[0].pos] = v[0].lam1;
+                                 }
+                                 if (v[0].ok2) {
+                                     ids[v[0].pos + 1] = v[0].id + stepm;
+                                     sl[v[0].pos + 1] = v[0].lam2;
+                                 }
+                             },
+                             lend, by_range);
+            __syncwarp();
         }
-    } else {
+        if (n < 0) n = dda_walk(g, K, cap, ids, sl, lend, by_range);
+        if (n < 0) return -1;
         for (int i = lane; i < n; i += 32) {
-            const unsigned id = (unsigned)((const int *)sx)[i];
-            bad |= id >= ncell;
-            const float o = id < ncell ? __ldg(map + id) : 0.0f;
-            // a cell already counted by an earlier state of the trajectory (Section 2.4) still
-            // stops the beam with probability o but adds no information
-            const bool counted = TRAJ && id < ncell && __ldg(stamps + id) < state;
-            sp[i] = o;
-            sc[i] = counted ? 0.0f : cell_gain(p.docc, o);
-            sx[i] = counted ? 0.0f : cell_gain(p.demp, o);
+            const unsigned id = (unsigned)ids[i];
+            bad |= id >= ncell;  // cannot happen for a consistent traversal; never read out of bounds
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (id < ncell) {
+                if (gains) {
+                    v = __ldg(gains + id);
+                } else {
+                    const float o = __ldg(map + id);
+                    v = make_float4(o, cell_gain(p.docc, o), cell_gain(p.demp, o), 0.0f);
+                }
+                // a cell already counted by an earlier state of the trajectory (Section 2.4) still
+                // stops the beam with probability o but adds no information
+                if (TRAJ && __ldg(stamps + id) < state) v.y = v.z = 0.0f;
+            }
+            sp[i] = v.x;
+            sc[i] = v.y;
+            sx[i] = v.z;
         }
     }
     if (__any_sync(kFull, bad) && lane == 0) set_status(status, FSMI_STATUS_INTERNAL);
+    if (lane == 0) sl[n] = lend;
     __syncwarp();
     return n;
 }
@@ -648,7 +694,7 @@ __device__ __forceinline__ float beam_sum(const DevParams &p, int n, float *sl, 
     const float cs = p.inv_s2 * (float)kSqrtLog2e;  // distance -> tail variable
     float I = 0.0f;
     if (n > 0) {
-        const float pe0 = cell_prefixes(sp, sc, sx, n, VAR == FSMI_UNIFORM);
+        const float pe0 = cell_prefixes4(sp, sc, sx, n, VAR == FSMI_UNIFORM);
         if (VAR == FSMI_EXACT || VAR == kExactFullSweep) {
             const float mu0 = sl[0] * cs - 0.5f * cs;  // e_0 centre, l_1 - 1/2 (scaled)
             build_pairs(sl, sc, n, cs);
