@@ -11,13 +11,9 @@
 //   conv:  z[t][c] = b[c] + sum_{k<3} sum_ci W[c][k][ci] a[2t + k - 1][ci]
 //
 // Parameters are one flat FP32 vector (master copy, layout below); the weights are used as a BF16
-// copy of the same vector, accumulation is FP32. Training keeps FP32 activations: the layers'
-// products run on the tensor cores with each FP32 operand split into BF16 terms (k_gemm_tc, whose
-// operands are read through index functions, convolutions gathering their im2col entries on the
-// fly; k_dgrad_conv for the convolutions' data gradients), the weight and bias gradients of the
-// convolutions as two-pass reductions over the batch rows (k_wgrad_part, k_colsum_part,
-// k_part_final); every sum is taken in a fixed order, so a training step gives the same floats
-// on every run.
+// copy of the same vector, accumulation is FP32. Training keeps FP32 activations and splits them into
+// BF16 terms for the tensor cores; every sum is taken in a fixed order, so a training step gives
+// the same floats on every run.
 #include <cuda.h>  // CUtensorMap and its enums (the encoder is fetched through the runtime, no -lcuda)
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
@@ -94,351 +90,13 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// ---- split-K partial sums --------------------------------------------------------------------------
-//
-// The training GEMMs (k_gemm_tc, below) may split K over blocks: block z writes its partial tile to
-// part[z][m][n] and k_split_reduce adds the splits in order and applies the epilogue.
-
-template <class FE>
-__global__ void k_split_reduce(int M, int N, int splits, const float *__restrict__ part, FE fe)
-{
-    const long long MN = (long long)M * N;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < MN; e += (long long)gridDim.x * blockDim.x) {
-        float s = 0.0f;
-        for (int z = 0; z < splits; ++z) s += part[z * MN + e];
-        fe((int)(e / N), (int)(e % N), s);
-    }
-}
-
 int grid_cap(long long want)
 {
     const long long cap = (long long)sm_count() * 32;
     return (int)(want < 1 ? 1 : (want > cap ? cap : want));
 }
 
-// ---- training: forward -------------------------------------------------------------------------
-//
-// Activations (FP32, pre-ReLU) per batch of N beams: z1 [N][128][32], z2 [N][64][32],
-// z3 [N][32][32], z4 [N][256]; pred, dpred [N]. Gradients of the same shapes reuse two buffers.
-
-struct TrainBufs {
-    float *z1, *z2, *z3, *z4, *pred, *dpred, *lossp, *g1, *g2, *part;
-    size_t part_floats;
-};
-
 __device__ __forceinline__ float relu(float v) { return v > 0.0f ? v : 0.0f; }
-
-// conv of layer input `in` (x as BF16 pairs for layer 1, relu(z_prev) otherwise): row m = n * Lout + t,
-// column c, k-index kk = k * Cin + ci
-struct ConvA1 {  // im2col of the profile (layer 1)
-    const __nv_bfloat162 *x;
-    __device__ float operator()(int m, int kk) const
-    {
-        const int n = m / 128, t = m % 128, k = kk / kCin, ci = kk % kCin;
-        const int s = 2 * t + k - 1;
-        if (s < 0 || s >= kL) return 0.0f;
-        const __nv_bfloat162 v = x[(long long)n * kL + s];
-        return ci == 0 ? __low2float(v) : __high2float(v);
-    }
-};
-struct ConvA {  // im2col of relu(z_prev) [N][Lin][32]
-    const float *z;
-    int Lin;
-    __device__ float operator()(int m, int kk) const
-    {
-        const int Lout = Lin >> 1;
-        const int n = m / Lout, t = m % Lout, k = kk / kCh, ci = kk % kCh;
-        const int s = 2 * t + k - 1;
-        if (s < 0 || s >= Lin) return 0.0f;
-        return relu(z[((long long)n * Lin + s) * kCh + ci]);
-    }
-};
-struct WConv {  // B(kk, c) = W[c][k][ci] (BF16), kk = k * Cin + ci
-    const bf16 *w;
-    int cin;
-    __device__ float operator()(int kk, int c) const { return bf(w, (long long)c * kK * cin + kk); }
-};
-struct StoreBias {  // out[m][n] = acc + b[n]
-    float *out;
-    const float *b;
-    int ld;
-    __device__ void operator()(int m, int n, float acc) const { out[(long long)m * ld + n] = acc + b[n]; }
-};
-struct ReluRow {  // A(m, k) = relu(z[m][k])
-    const float *z;
-    int ld;
-    __device__ float operator()(int m, int k) const { return relu(z[(long long)m * ld + k]); }
-};
-struct WT {  // B(k, n) = W[n][k] (BF16 row-major [N][K])
-    const bf16 *w;
-    int ld;
-    __device__ float operator()(int k, int n) const { return bf(w, (long long)n * ld + k); }
-};
-
-// pred[n] = b5 + sum_j W5[j] relu(z4[n][j]); lossp[n] = (pred - y)^2; dpred[n] = 2 (pred - y) / N
-__global__ void k_head(const float *__restrict__ z4, const bf16 *__restrict__ w, const float *__restrict__ params,
-                       const float *__restrict__ y, int N, float *pred, float *dpred, float *lossp)
-{
-    const int lane = lane_id();
-    const int wpb = blockDim.x >> 5;
-    for (int n = blockIdx.x * wpb + (threadIdx.x >> 5); n < N; n += gridDim.x * wpb) {
-        float a = 0.0f;
-        for (int j = lane; j < kHid; j += 32) a = fmaf(bf(w, oW5 + j), relu(z4[(long long)n * kHid + j]), a);
-        a = warp_sum(a) + params[oB5];
-        if (lane == 0) {
-            pred[n] = a;
-            if (y) {
-                const float d = a - y[n];
-                dpred[n] = 2.0f * d / (float)N;
-                lossp[n] = d * d;
-            }
-        }
-    }
-}
-
-// loss = sum(lossp) / N (one block, fixed order)
-__global__ void __launch_bounds__(1024) k_loss(const float *__restrict__ lossp, int N, float *loss)
-{
-    __shared__ float sh[32];
-    float a = 0.0f;
-    for (int n = threadIdx.x; n < N; n += blockDim.x) a += lossp[n];
-    a = warp_sum(a);
-    if (lane_id() == 0) sh[threadIdx.x >> 5] = a;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float v = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0f;
-        v = warp_sum(v);
-        if (threadIdx.x == 0) *loss = v / (float)N;
-    }
-}
-
-// ---- training: backward ------------------------------------------------------------------------
-
-// dz4[n][j] = dpred[n] W5[j] [z4 > 0]
-__global__ void k_dz4(const float *__restrict__ z4, const float *__restrict__ dpred, const bf16 *__restrict__ w, int N,
-                      float *__restrict__ dz4)
-{
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < (long long)N * kHid;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int j = (int)(e % kHid);
-        dz4[e] = z4[e] > 0.0f ? dpred[e / kHid] * bf(w, oW5 + j) : 0.0f;
-    }
-}
-
-// ---- reductions over the batch rows, in a fixed order -------------------------------------------
-//
-// Sums over the R rows of a batch (bias gradients, conv weight gradients) run in two passes: block
-// b adds rows [b * rows, (b + 1) * rows) into part[b][...], then one thread per output adds the
-// blocks' partials in block order. The row split depends only on R, so a step's gradients are the
-// same floats on every run (and every GPU).
-constexpr int kRedMaxBlocks = 2048;  // blocks per reduction, at most (bounds the partials)
-
-// rows per block: at least min_rows, a multiple of 32, and few enough blocks
-int red_rows(long long R, int min_rows)
-{
-    const long long per = (R + kRedMaxBlocks - 1) / kRedMaxBlocks;
-    return (int)std::max<long long>(min_rows, (per + 31) / 32 * 32);
-}
-
-// part[b][c] = sum over the block's rows r of f(r, c), for C columns (C divides 256): the block's
-// 256 / C row lanes take every (256 / C)-th row, then their sums are added in lane order. A warp
-// reads consecutive columns of one row.
-template <class F>
-__global__ void __launch_bounds__(256) k_colsum_part(int R, int C, int rows, F f, float *__restrict__ part)
-{
-    __shared__ float sh[256];
-    const int rl = 256 / C;
-    const int c = threadIdx.x % C, rsub = threadIdx.x / C;
-    const int r0 = blockIdx.x * rows, r1 = min(R, r0 + rows);
-    float a = 0.0f;
-    if (rsub < rl)
-        for (int r = r0 + rsub; r < r1; r += rl) a += f(r, c);
-    sh[threadIdx.x] = a;
-    __syncthreads();
-    if (threadIdx.x < C) {
-        float t = 0.0f;
-        for (int k = 0; k < rl; ++k) t += sh[k * C + threadIdx.x];
-        part[(size_t)blockIdx.x * C + threadIdx.x] = t;
-    }
-}
-
-// out[o] = sum over blocks b of part[b][o], in a fixed order: a block takes 32 outputs (one per lane),
-// its 8 warps the 8 contiguous eighths of the blocks, and the eighths' sums are added in order.
-__global__ void __launch_bounds__(256) k_part_final(int nblk, int O, const float *__restrict__ part,
-                                                    float *__restrict__ out)
-{
-    __shared__ float sh[8][32];
-    const int lane = lane_id(), w = threadIdx.x >> 5;
-    const int o = blockIdx.x * 32 + lane;
-    const int b0 = (int)((long long)nblk * w / 8), b1 = (int)((long long)nblk * (w + 1) / 8);
-    float t = 0.0f;
-    if (o < O) {
-#pragma unroll 8
-        for (int b = b0; b < b1; ++b) t += part[(size_t)b * O + o];
-    }
-    sh[w][lane] = t;
-    __syncthreads();
-    if (w == 0 && o < O) {
-        float u = 0.0f;
-        for (int k = 0; k < 8; ++k) u += sh[k][lane];
-        out[o] = u;
-    }
-}
-
-// Conv weight gradient of a layer with CIN input channels, Lin input and Lout = Lin / 2 output
-// positions: gW[c][k * CIN + ci] = sum over rows r = (n, t) of dz[r][c] in[n][2t + k - 1][ci], with
-// `in` the layer input (relu(z) of the previous layer, or the profile x for the first). A block takes
-// `rows` consecutive rows in tiles of kWgTile (Lout is a multiple of kWgTile, so a tile lies in one
-// beam n, at positions t0 .. t0 + kWgTile - 1) and stages the tile's dz rows and the input positions
-// 2 t0 - 1 .. 2 t0 + 2 kWgTile - 1 that its im2col rows read: row i of the tile's im2col is then the
-// 3 CIN consecutive floats from offset 2 CIN i. Each thread adds its outputs over the block's rows in
-// row order into part[b][...] (k_part_final adds the blocks). CIN = 32: a thread holds 4 output
-// channels x 3 taps (one float4 of dz and three input values per row); CIN = 2: one output.
-constexpr int kWgTile = 32;
-
-template <int CIN>
-__global__ void __launch_bounds__(256) k_wgrad_part(int R, int rows, int Lin, const float *__restrict__ dz,
-                                                    const float *__restrict__ z, const __nv_bfloat162 *__restrict__ x,
-                                                    float *__restrict__ part)
-{
-    constexpr int kNKK = kK * CIN, kO = kCh * kNKK, kPos = 2 * kWgTile + 1;
-    __shared__ __align__(16) float sdz[kWgTile * kCh];
-    __shared__ __align__(16) float sin_[kPos * CIN];
-    const int Lout = Lin >> 1;
-    const int r0 = blockIdx.x * rows, r1 = min(R, r0 + rows);
-    const int tid = threadIdx.x;
-    float acc[4][3] = {};
-    for (int rt = r0; rt < r1; rt += kWgTile) {
-        const int n = rt / Lout, t0 = rt - n * Lout;
-        for (int e = tid; e < kWgTile * kCh / 4; e += 256)
-            reinterpret_cast<float4 *>(sdz)[e] = reinterpret_cast<const float4 *>(dz + (long long)rt * kCh)[e];
-        if (CIN == kCh) {
-            for (int e = tid; e < kPos * kCh / 4; e += 256) {
-                const int p = e / (kCh / 4), q = e % (kCh / 4);
-                const int sidx = 2 * t0 - 1 + p;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (sidx >= 0 && sidx < Lin) {
-                    v = reinterpret_cast<const float4 *>(z + ((long long)n * Lin + sidx) * kCh)[q];
-                    v = make_float4(relu(v.x), relu(v.y), relu(v.z), relu(v.w));
-                }
-                reinterpret_cast<float4 *>(sin_)[e] = v;
-            }
-        } else {
-            for (int p = tid; p < kPos; p += 256) {
-                const int sidx = 2 * t0 - 1 + p;
-                float lo = 0.0f, hi = 0.0f;
-                if (sidx >= 0 && sidx < Lin) {
-                    const __nv_bfloat162 v = x[(long long)n * Lin + sidx];
-                    lo = __low2float(v);
-                    hi = __high2float(v);
-                }
-                sin_[2 * p] = lo;
-                sin_[2 * p + 1] = hi;
-            }
-        }
-        __syncthreads();
-        if (CIN == kCh) {
-            const int cg = tid >> 5, kg = tid & 31;
-            for (int i = 0; i < kWgTile; ++i) {
-                const float4 d = reinterpret_cast<const float4 *>(sdz + i * kCh)[cg];
-                const float *a = sin_ + 2 * CIN * i + kg;
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    const float v = a[32 * j];
-                    acc[0][j] = fmaf(d.x, v, acc[0][j]);
-                    acc[1][j] = fmaf(d.y, v, acc[1][j]);
-                    acc[2][j] = fmaf(d.z, v, acc[2][j]);
-                    acc[3][j] = fmaf(d.w, v, acc[3][j]);
-                }
-            }
-        } else if (tid < kO) {
-            const int c = tid / kNKK, kk = tid % kNKK;
-            for (int i = 0; i < kWgTile; ++i) acc[0][0] = fmaf(sdz[i * kCh + c], sin_[2 * CIN * i + kk], acc[0][0]);
-        }
-        __syncthreads();
-    }
-    float *pb = part + (size_t)blockIdx.x * kO;
-    if (CIN == kCh) {
-        const int cg = tid >> 5, kg = tid & 31;
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) pb[(4 * cg + a) * kNKK + 32 * j + kg] = acc[a][j];
-    } else if (tid < kO) {
-        pb[tid] = acc[0][0];
-    }
-}
-
-// out[c] = sum_r f(r, c) for C columns (C divides 256), in a fixed order (k_colsum_part, k_part_final)
-template <class F>
-cudaError_t colsum(int R, int C, F f, float *out, float *part, cudaStream_t s)
-{
-    const int rows = red_rows(R, 64), nblk = (R + rows - 1) / rows;
-    k_colsum_part<<<nblk, 256, 0, s>>>(R, C, rows, f, part);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_part_final<<<(C + 31) / 32, 256, 0, s>>>(nblk, C, part, out);
-    return cudaGetLastError();
-}
-
-// out[c * 3 CIN + k * CIN + ci] = sum over rows of dz[r][c] in[n][2t + k - 1][ci] (R = N Lout rows),
-// in a fixed order (k_wgrad_part, k_part_final)
-template <int CIN>
-cudaError_t wgrad(int R, int Lin, const float *dz, const float *z, const __nv_bfloat162 *x, float *out, float *part,
-                  cudaStream_t s)
-{
-    const int rows = red_rows(R, 512), nblk = (R + rows - 1) / rows;
-    k_wgrad_part<CIN><<<nblk, 256, 0, s>>>(R, rows, Lin, dz, z, x, part);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const int O = kCh * kK * CIN;
-    k_part_final<<<(O + 31) / 32, 256, 0, s>>>(nblk, O, part, out);
-    return cudaGetLastError();
-}
-
-struct Store {
-    float *out;
-    int ld;
-    __device__ void operator()(int m, int n, float acc) const { out[(long long)m * ld + n] = acc; }
-};
-struct StoreMask {  // out[m][n] = acc [mask[m][n] > 0]
-    float *out;
-    const float *mask;
-    int ld;
-    __device__ void operator()(int m, int n, float acc) const
-    {
-        const long long i = (long long)m * ld + n;
-        out[i] = mask[i] > 0.0f ? acc : 0.0f;
-    }
-};
-struct RowT {  // A(m, k) = g[k][m] (row-major [K][ld])
-    const float *g;
-    int ld;
-    __device__ float operator()(int m, int k) const { return g[(long long)k * ld + m]; }
-};
-struct RowN {  // A(m, k) = g[m][k]
-    const float *g;
-    int ld;
-    __device__ float operator()(int m, int k) const { return g[(long long)m * ld + k]; }
-};
-struct WRow {  // B(k, n) = W[k][n] (BF16 row-major [K][ld])
-    const bf16 *w;
-    int ld;
-    __device__ float operator()(int k, int n) const { return bf(w, (long long)k * ld + n); }
-};
-struct SumDz {  // f(r, c) = dz[r][c]
-    const float *dz;
-    int ld;
-    __device__ float operator()(int r, int c) const { return dz[(long long)r * ld + c]; }
-};
-struct W5Grad {  // f(n, j) = dpred[n] relu(z4[n][j])
-    const float *dpred, *z4;
-    __device__ float operator()(int n, int j) const { return dpred[n] * relu(z4[(long long)n * kHid + j]); }
-};
-struct B5Grad {
-    const float *dpred;
-    __device__ float operator()(int n, int) const { return dpred[n]; }
-};
 
 // ---- Adam --------------------------------------------------------------------------------------
 
@@ -498,236 +156,766 @@ __device__ __forceinline__ void mma_bf16_k8(float (&c)[4], unsigned a0, unsigned
                  : "r"(a0), "r"(a1), "r"(b0));
 }
 
-// ---- training GEMMs on the tensor cores ----------------------------------------------------------
-//
-// C[m][n] = sum_k A(m, k) B(k, n) with FP32 operands given as index functions of (row, k), the
-// products on the tensor cores (mma.sync m16n8k16, BF16 operands, FP32 accumulation). An FP32
-// operand is split into BF16 terms, a_1 = bf16(a), a_2 = bf16(a - a_1), a_3 = bf16(a - a_1 - a_2),
-// whose sum is a (1 + d) with |d| <= 2^-18 for two terms and 2^-27 for three (the split-BF16
-// products of Henry, Tang and Heinecke, "Leveraging the bfloat16 artificial intelligence datatype
-// for higher-precision computations", 2019). AS = 3 (the forward pass, whose outputs feed the loss
-// and its derivative): A B = (A_1 + A_2 + A_3) B for a B of BF16 weights, exact in one term, as
-// accurate as FP32 arithmetic. AS = 2 (the backward pass): A_1 B + A_2 B, plus A_1 B_2 when B is
-// FP32 as well (BSPLIT; the A_2 B_2 term, below 2^-18 of the product, is left out). Block tile
-// TM x TN (TM TN = 4096: 8 warps of 32 x 16 outputs, 2 x 2 MMA tiles each), K in stages of kTrK,
-// staged as BF16 pairs in [row][k] order with a row pitch of kTrPitch elements (20 words: the
-// fragment loads of the eight row groups fall in distinct banks). AKF / BKF: the operand's index
-// function is contiguous in k (stage k-pairs across the threads) or in its row (stage rows across
-// them). With more than one K split, block z writes its partial tile to part[z][m][n] and
-// k_split_reduce adds the splits in order.
-constexpr int kTrK = 32, kTrPitch = kTrK + 8;
+constexpr int kS2 = 104;  // W2 / W3 row stride (bf16): 208 B, eight rows in eight bank groups
 
-// the BF16 terms of v0, v1 (t[0] = bf16(v), t[i] = bf16(v - t[0] - ... - t[i-1])) at `at` of each
-// of the first `terms` arrays
-__device__ __forceinline__ void split_store(bf16 *const *t, int terms, int at, float v0, float v1)
+// Weight fragments of k-step ks (16 of the K = 96 inputs) of a conv layer for the four n8 tiles
+__device__ __forceinline__ void load_wfrag(const bf16 *Wt, int ks, unsigned (&bw)[4][2])
 {
-    for (int i = 0; i < terms; ++i) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
-        *reinterpret_cast<__nv_bfloat162 *>(t[i] + at) = h;
-        v0 -= __low2float(h);
-        v1 -= __high2float(h);
+    const int lane = lane_id();
+#pragma unroll
+    for (int np = 0; np < 2; ++np) {
+        const int row = np * 16 + (lane & 7) + 8 * (lane >> 4);
+        ldsm_x4(smem_u32(Wt + row * kS2 + ks * 16 + 8 * ((lane >> 3) & 1)), bw[2 * np][0], bw[2 * np][1],
+                bw[2 * np + 1][0], bw[2 * np + 1][1]);
     }
 }
 
-__device__ __forceinline__ unsigned lds32(const bf16 *p) { return *reinterpret_cast<const unsigned *>(p); }
+// ---- training ---------------------------------------------------------------------------------------
+//
+// Activations (FP32, pre-ReLU) per batch of N beams: z1 [N][128][32], z2 [N][64][32], z3 [N][32][32],
+// z4 [N][256]. All products run on the tensor cores (mma.sync m16n8k16, BF16 operands, FP32
+// accumulation) with each FP32 operand split into BF16 terms, a_1 = bf16(a), a_2 = bf16(a - a_1),
+// a_3 = bf16(a - a_1 - a_2), whose sum is a (1 + d) with |d| <= 2^-18 for two terms and 2^-27 for three
+// (the split-BF16 products of Henry, Tang and Heinecke, "Leveraging the bfloat16 artificial
+// intelligence datatype for higher-precision computations", 2019). The forward pass, whose outputs feed
+// the loss and its derivative, takes three terms (weights are exact in one); the backward pass two,
+// A_1 B_1 + A_2 B_1 + A_1 B_2 where both operands are FP32 (the A_2 B_2 term is below 2^-18 of the
+// product).
+//
+// The convolutions work on strips of 16 output positions per warp whose MMA fragments are formed in
+// registers: nothing is staged, and the im2col matrix exists nowhere. A step of 4096 beams with its sampling
+// takes 265 us; 754 us with every layer an index-function GEMM (operands gathered element by element through
+// shared memory) and the reductions in 21 launches.
 
-template <int TN, int AS, bool BSPLIT, bool AKF, bool BKF, class FA, class FB, class FE>
-__global__ void __launch_bounds__(256) k_gemm_tc(int M, int N, int K, int kper, FA fa, FB fb, FE fe, float *part)
+// (v.x, v.y) as T BF16 pairs
+template <int T>
+__device__ __forceinline__ void split(float2 v, unsigned (&t)[T])
 {
-    constexpr int TM = 4096 / TN, WN = TN / 16, KP = kTrK / 2;
-    static_assert(AS == 2 || AS == 3, "two or three BF16 terms of A");
-    __shared__ __align__(16) bf16 sA[AS][TM * kTrPitch];
-    __shared__ __align__(16) bf16 sB[BSPLIT ? 2 : 1][TN * kTrPitch];
-    bf16 *const ta[3] = {sA[0], sA[1], sA[AS - 1]};
-    bf16 *const tb[2] = {sB[0], sB[BSPLIT ? 1 : 0]};
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int wm = w / WN, wn = w % WN;  // the warp's outputs: rows 32 wm .., columns 16 wn ..
-    const int g = lane >> 2, tq = lane & 3;
-    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+#pragma unroll
+    for (int i = 0; i < T; ++i) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+        t[i] = *reinterpret_cast<const unsigned *>(&h);
+        v.x -= __low2float(h);
+        v.y -= __high2float(h);
+    }
+}
+
+// Channels and fragment columns: column s = 8 nt + 2w + e of an MMA tile holds channel 16 (nt / 2) + 4w +
+// 2 (nt % 2) + e, so that lane w's pairs of the tiles 0, 1 and 2, 3 are 4 consecutive channels each and a
+// warp's 16-byte access covers whole sectors, 64 bytes of each of 8 rows. (With the columns' own order an
+// access is 8 bytes per lane and meets 8 lines for 256 bytes; the L1 wavefronts of that bound these kernels.)
+// The weights are staged in the same order; as a sum over channels runs over all columns, nothing else changes.
+__device__ __forceinline__ int chan(int s) { return 16 * (s >> 4) + 4 * ((s >> 1) & 3) + 2 * ((s >> 3) & 1) + (s & 1); }
+
+// channels 0 .. 3 and 16 .. 19 from p as the pairs of the four n8 tiles
+__device__ __forceinline__ void load8(const float *p, float2 (&v)[4])
+{
+    const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 16);
+    v[0] = make_float2(a.x, a.y);
+    v[1] = make_float2(a.z, a.w);
+    v[2] = make_float2(b.x, b.y);
+    v[3] = make_float2(b.z, b.w);
+}
+
+__device__ __forceinline__ float2 relu2(float2 v) { return make_float2(relu(v.x), relu(v.y)); }
+__device__ __forceinline__ float2 ld2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
+
+// relu(acc + b) of a strip as three BF16 terms P[nt][h] (row g + 8 h); acc + b goes to out (row g of the
+// strip, channel 4w; `step` floats between the strip's rows). bs: the layer's biases from channel 4w on
+__device__ __forceinline__ void store_split(const float (&acc)[4][4], const float *bs, float *out, int step,
+                                            unsigned (&P)[4][2][3])
+{
+    float2 b[4];
+    load8(bs, b);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        float2 z[4];
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt) {
+            z[nt] = make_float2(acc[nt][2 * e] + b[nt].x, acc[nt][2 * e + 1] + b[nt].y);
+            split<3>(relu2(z[nt]), P[nt][e]);
+        }
+        float4 *o = reinterpret_cast<float4 *>(out + 8 * e * step);
+        o[0] = make_float4(z[0].x, z[0].y, z[1].x, z[1].y);
+        o[4] = make_float4(z[2].x, z[2].y, z[3].x, z[3].y);
+    }
+}
+
+// the strip one row down, as shift_rows of the inference kernel, for each term
+__device__ __forceinline__ void shift_terms(const unsigned (&P)[4][2][3], unsigned (&carry)[4][3], unsigned (&S)[4][2][3])
+{
+    const int lane = lane_id();
+    const bool first = lane < 4;
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const unsigned lo = __shfl_sync(kFull, P[nt][0][i], lane + 28), hi = __shfl_sync(kFull, P[nt][1][i], lane + 28);
+            S[nt][0][i] = first ? carry[nt][i] : lo;
+            S[nt][1][i] = first ? lo : hi;
+            carry[nt][i] = hi;
+        }
+}
+
+// acc += strip P (tap `tap`) of a K = 96 layer
+__device__ __forceinline__ void tap_mma3(float (&acc)[4][4], const unsigned (&P)[4][2][3], const bf16 *sW, int tap)
+{
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+        unsigned bw[4][2];
+        load_wfrag(sW, 2 * tap + hh, bw);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+                mma_bf16(acc[nt], P[2 * hh][0][i], P[2 * hh][1][i], P[2 * hh + 1][0][i], P[2 * hh + 1][1][i], bw[nt][0],
+                         bw[nt][1]);
+    }
+}
+
+// The three convolutions of a batch, one warp per beam: the inference kernel's strips of equal residues (conv1 at
+// 4u + r, conv2 at 2u and 2u + 1, conv3 at u; see k_conv_infer) with three terms per activation, every layer's
+// pre-activations written once and read by nobody here; h receives relu(z3) as three BF16 terms,
+// hstride elements apart (fc1's operand). A batch of 4096 writes 142 MB in 46 us (21 us at the copy
+// rate); 12 warps per SM at 168 registers leave the MMA chains' latency in sight. Layer by layer, each reading
+// the one before: 85 us; as index-function GEMMs 198 us.
+constexpr int kFwdWarps = 4;
+__global__ void __launch_bounds__(kFwdWarps * 32, 3)
+    k_convs_fwd(int N, const unsigned *__restrict__ x, const bf16 *__restrict__ w, const float *__restrict__ params,
+                float *__restrict__ z1, float *__restrict__ z2, float *__restrict__ z3, bf16 *__restrict__ h, size_t hstride)
+{
+    __shared__ __align__(16) bf16 sW1[kCh * 8];
+    __shared__ __align__(16) bf16 sW2[kCh * kS2];
+    __shared__ __align__(16) bf16 sW3[kCh * kS2];
+    __shared__ __align__(16) float sb[3 * kCh];
+    for (int e = threadIdx.x; e < 3 * kCh; e += kFwdWarps * 32)
+        sb[e] = params[(e < kCh ? oB1 : e < 2 * kCh ? oB2 : oB3) + e % kCh];
+    for (int e = threadIdx.x; e < kCh * 8; e += kFwdWarps * 32)
+        sW1[e] = e % 8 < kK * kCin ? w[oW1 + chan(e / 8) * kK * kCin + e % 8] : __float2bfloat16_rn(0.0f);
+    for (int e = threadIdx.x; e < kCh * kS2; e += kFwdWarps * 32) {
+        const int kk = e % kS2, at = chan(e / kS2) * kK * kCh + (kk & ~31) + chan(kk & 31);
+        sW2[e] = kk < kK * kCh ? w[oW2 + at] : __float2bfloat16_rn(0.0f);
+        sW3[e] = kk < kK * kCh ? w[oW3 + at] : __float2bfloat16_rn(0.0f);
+    }
+    __syncthreads();
+    const int lane = lane_id(), g = lane >> 2, wq = lane & 3;
+    const float *b1 = sb + 4 * wq, *b2 = b1 + kCh, *b3 = b2 + kCh;
+    unsigned bw1[4];
+    ldsm_x4(smem_u32(sW1 + lane * 8), bw1[0], bw1[1], bw1[2], bw1[3]);
+    for (int n = blockIdx.x * kFwdWarps + (threadIdx.x >> 5); n < N; n += gridDim.x * kFwdWarps) {
+        const unsigned *xr = x + (size_t)n * kL;
+        unsigned carry1[4][3] = {}, carry2[4][3] = {};
+#pragma unroll 1
+        for (int s = 0; s < 2; ++s) {  // u = 16 s + row
+            const int u = 16 * s + g;
+            auto conv1 = [&](int r, unsigned(&P)[4][2][3]) {  // positions 4u + r
+                const int i = 8 * u + 2 * r - 1 + wq;
+                const unsigned a0 = wq < 3 && i >= 0 ? __ldg(xr + i) : 0u, a1 = wq < 3 ? __ldg(xr + i + 64) : 0u;
+                float acc[4][4] = {};
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) mma_bf16_k8(acc[nt], a0, a1, bw1[nt]);
+                store_split(acc, b1, z1 + ((size_t)n * 128 + 4 * u + r) * kCh + 4 * wq, 4 * kCh, P);
+            };
+            float ev[4][4] = {}, od[4][4] = {}, acc[4][4] = {};
+            unsigned P1[4][2][3], P3[4][2][3], Q[4][2][3];
+            conv1(3, P3);
+            shift_terms(P3, carry1, Q);
+            conv1(1, P1);
+            tap_mma3(ev, Q, sW2, 0);
+            tap_mma3(od, P1, sW2, 0);
+            conv1(0, Q);
+            tap_mma3(ev, Q, sW2, 1);
+            conv1(2, Q);
+            tap_mma3(od, Q, sW2, 1);
+            tap_mma3(ev, P1, sW2, 2);
+            tap_mma3(od, P3, sW2, 2);
+            store_split(ev, b2, z2 + ((size_t)n * 64 + 2 * u) * kCh + 4 * wq, 2 * kCh, P1);
+            store_split(od, b2, z2 + ((size_t)n * 64 + 2 * u + 1) * kCh + 4 * wq, 2 * kCh, P3);
+            shift_terms(P3, carry2, Q);
+            tap_mma3(acc, Q, sW3, 0);
+            tap_mma3(acc, P1, sW3, 1);
+            tap_mma3(acc, P3, sW3, 2);
+            const size_t o = ((size_t)n * 32 + u) * kCh + 4 * wq;
+            store_split(acc, b3, z3 + o, kCh, Q);
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    uint2 *d = reinterpret_cast<uint2 *>(h + i * hstride + o + 8 * e * kCh);
+                    d[0] = make_uint2(Q[0][e][i], Q[1][e][i]);
+                    d[4] = make_uint2(Q[2][e][i], Q[3][e][i]);
+                }
+        }
+    }
+}
+
+// ---- fc1's three products ---------------------------------------------------------------------------
+//
+// C[m][n] = sum over the term products of sum_k A_i(m, k) B_j(k, n), with the operands' BF16 terms in
+// memory (written by their producers), `ta` / `tb` elements apart: TA terms of A, TB of B, the products
+// (i, 0) and, with TB = 2, (0, 1). AT / BT: the operand is stored with k along the rows (A [k][m],
+// B [k][n]), else along the columns (A [m][k], B [n][k]). Blocks of 128 x 64 outputs, 8 warps of
+// 32 x 32; K in stages of 32 through a 3-stage cp.async ring, 16-byte chunks XOR-swizzled so that
+// ldmatrix (.trans for k-row storage) meets every bank once. Block z takes k in [z kper, (z + 1) kper).
+// Rows past M and k past K read as zero; lda, ldb and the starts are multiples of 8 elements, N of 64.
+//
+// A batch of 4096: 26 us forward (three products, 6.4 GFLOP of MMAs each here and in the weight gradient, the
+// tensor pipe 55 % busy), 24 us weight gradient, 28 us data gradient; 79, 83 and 75 us when the blocks
+// gathered and split FP32 operands element by element.
+constexpr int kGmM = 128, kGmN = 64, kGmK = 32, kGmStages = 3;
+template <int TA, int TB>
+constexpr int kGmSmem = kGmStages * (TA * kGmM + TB * kGmN) * kGmK * 2;
+
+__device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool ok)
+{
+    const int bytes = ok ? 16 : 0;  // 0: the 16 bytes are zero-filled and src is not read
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void ldsm_x4t(unsigned addr, unsigned &r0, unsigned &r1, unsigned &r2, unsigned &r3)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+                 : "r"(addr));
+}
+
+// one operand's tile of a stage: R rows (of m or n) x 32 k into shared memory at s
+template <int R, bool T>
+__device__ __forceinline__ void stage_tile(unsigned s, const bf16 *src, int ld, int r0, int rmax, int k0, int kend)
+{
+#pragma unroll
+    for (int c = threadIdx.x; c < R * 4; c += 256) {
+        if (T) {  // [k][row]: R / 8 chunks per k
+            const int k = c / (R / 8), q = c % (R / 8);
+            const bool ok = k0 + k < kend && r0 + 8 * q < rmax;
+            cp_async16(s + k * R * 2 + ((q ^ (k & 7)) << 4), ok ? src + (size_t)(k0 + k) * ld + r0 + 8 * q : src, ok);
+        } else {  // [row][k]: 4 chunks per row
+            const int r = c >> 2, q = c & 3;
+            const bool ok = r0 + r < rmax && k0 + 8 * q < kend;
+            cp_async16(s + r * 64 + ((q ^ ((r >> 1) & 3)) << 4), ok ? src + (size_t)(r0 + r) * ld + k0 + 8 * q : src, ok);
+        }
+    }
+}
+
+// address of the 16-byte chunk holding rows r .. r + 7 (T) or row r (else) at k (T) or k .. k + 7
+template <int R, bool T>
+__device__ __forceinline__ unsigned tile_at(unsigned s, int r, int k)
+{
+    return T ? s + k * R * 2 + (((r >> 3) ^ (k & 7)) << 4) : s + r * 64 + (((k >> 3) ^ ((r >> 1) & 3)) << 4);
+}
+
+template <int TA, int TB, bool AT, bool BT, class FE>
+__global__ void __launch_bounds__(256, 2)
+    k_gemm_terms(int M, int N, int K, int kper, const bf16 *__restrict__ A, size_t ta, int lda, const bf16 *__restrict__ B,
+                 size_t tb, int ldb, FE fe)
+{
+    extern __shared__ __align__(128) unsigned char gsm[];
+    constexpr int kA = kGmM * kGmK * 2, kB = kGmN * kGmK * 2, kStage = TA * kA + TB * kB;
+    const unsigned s0 = smem_u32(gsm);
+    const int lane = lane_id(), w = threadIdx.x >> 5, wm = (w >> 1) * 32, wn = (w & 1) * 32;
+    const int m0 = blockIdx.y * kGmM, n0 = blockIdx.x * kGmN;
     const int kbeg = blockIdx.z * kper, kend = min(K, kbeg + kper);
-    float acc[2][2][4] = {};
-    for (int k0 = kbeg; k0 < kend; k0 += kTrK) {
-        for (int e = tid; e < TM * KP; e += 256) {
-            const int r = AKF ? e / KP : e % TM, kp = AKF ? e % KP : e / TM;
-            const int m = m0 + r, k = k0 + 2 * kp;
-            float v0 = 0.0f, v1 = 0.0f;
-            if (m < M) {
-                if (k < kend) v0 = fa(m, k);
-                if (k + 1 < kend) v1 = fa(m, k + 1);
-            }
-            split_store(ta, AS, r * kTrPitch + 2 * kp, v0, v1);
-        }
-        for (int e = tid; e < TN * KP; e += 256) {
-            const int r = BKF ? e / KP : e % TN, kp = BKF ? e % KP : e / TN;
-            const int n = n0 + r, k = k0 + 2 * kp;
-            float v0 = 0.0f, v1 = 0.0f;
-            if (n < N) {
-                if (k < kend) v0 = fb(k, n);
-                if (k + 1 < kend) v1 = fb(k + 1, n);
-            }
-            split_store(tb, BSPLIT ? 2 : 1, r * kTrPitch + 2 * kp, v0, v1);
-        }
-        __syncthreads();
+    const int steps = kend > kbeg ? (kend - kbeg + kGmK - 1) / kGmK : 0;
+    auto fill = [&](int step) {
+        if (step < steps) {
+            const unsigned s = s0 + (step % kGmStages) * kStage;
+            const int k0 = kbeg + step * kGmK;
 #pragma unroll
-        for (int ks = 0; ks < kTrK; ks += 16) {
-            unsigned a[AS][2][4], b[2][2][2];
+            for (int i = 0; i < TA; ++i) stage_tile<kGmM, AT>(s + i * kA, A + i * ta, lda, m0, M, k0, kend);
 #pragma unroll
-            for (int i = 0; i < AS; ++i)
+            for (int i = 0; i < TB; ++i) stage_tile<kGmN, BT>(s + TA * kA + i * kB, B + i * tb, ldb, n0, N, k0, kend);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float acc[2][4][4] = {};
+#pragma unroll
+    for (int i = 0; i < kGmStages - 1; ++i) fill(i);
+    for (int step = 0; step < steps; ++step) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kGmStages - 2) : "memory");
+        __syncthreads();  // the stage has landed for all, and the one filled next is no longer read
+        fill(step + kGmStages - 1);
+        const unsigned s = s0 + (step % kGmStages) * kStage, sb = s + TA * kA;
+#pragma unroll
+        for (int ks = 0; ks < kGmK; ks += 16) {
+            unsigned a[TA][2][4], b[TB][4][2];
+#pragma unroll
+            for (int i = 0; i < TA; ++i)
 #pragma unroll
                 for (int mt = 0; mt < 2; ++mt) {
-                    const bf16 *p = sA[i] + (32 * wm + 16 * mt + g) * kTrPitch + ks + 2 * tq;
-                    a[i][mt][0] = lds32(p);
-                    a[i][mt][1] = lds32(p + 8 * kTrPitch);
-                    a[i][mt][2] = lds32(p + 8);
-                    a[i][mt][3] = lds32(p + 8 * kTrPitch + 8);
+                    const int m = wm + 16 * mt;
+                    if (AT)
+                        ldsm_x4t(tile_at<kGmM, true>(s + i * kA, m + 8 * ((lane >> 3) & 1), ks + (lane & 7) + 8 * (lane >> 4)),
+                                 a[i][mt][0], a[i][mt][1], a[i][mt][2], a[i][mt][3]);
+                    else
+                        ldsm_x4(tile_at<kGmM, false>(s + i * kA, m + (lane & 15), ks + 8 * (lane >> 4)), a[i][mt][0],
+                                a[i][mt][1], a[i][mt][2], a[i][mt][3]);
                 }
 #pragma unroll
-            for (int i = 0; i < (BSPLIT ? 2 : 1); ++i)
+            for (int i = 0; i < TB; ++i)
 #pragma unroll
-                for (int nt = 0; nt < 2; ++nt) {
-                    const bf16 *p = sB[i] + (16 * wn + 8 * nt + g) * kTrPitch + ks + 2 * tq;
-                    b[i][nt][0] = lds32(p);
-                    b[i][nt][1] = lds32(p + 8);
+                for (int np = 0; np < 2; ++np) {
+                    const int n = wn + 16 * np;
+                    if (BT)
+                        ldsm_x4t(tile_at<kGmN, true>(sb + i * kB, n + 8 * (lane >> 4), ks + (lane & 7) + 8 * ((lane >> 3) & 1)),
+                                 b[i][2 * np][0], b[i][2 * np][1], b[i][2 * np + 1][0], b[i][2 * np + 1][1]);
+                    else
+                        ldsm_x4(tile_at<kGmN, false>(sb + i * kB, n + (lane & 7) + 8 * (lane >> 4), ks + 8 * ((lane >> 3) & 1)),
+                                b[i][2 * np][0], b[i][2 * np][1], b[i][2 * np + 1][0], b[i][2 * np + 1][1]);
                 }
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
+            for (int i = 0; i < TA + TB - 1; ++i)  // the products (i, 0), then (0, 1)
 #pragma unroll
-                for (int nt = 0; nt < 2; ++nt) {
+                for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-                    for (int i = 0; i < AS; ++i)
-                        mma_bf16(acc[mt][nt], a[i][mt][0], a[i][mt][1], a[i][mt][2], a[i][mt][3], b[0][nt][0],
-                                 b[0][nt][1]);
-                    if (BSPLIT)
-                        mma_bf16(acc[mt][nt], a[0][mt][0], a[0][mt][1], a[0][mt][2], a[0][mt][3], b[1][nt][0],
-                                 b[1][nt][1]);
-                }
+                    for (int nt = 0; nt < 4; ++nt) {
+                        const unsigned(&x)[4] = a[i < TA ? i : 0][mt];
+                        const unsigned(&y)[2] = b[i < TA ? 0 : TB - 1][nt];
+                        mma_bf16(acc[mt][nt], x[0], x[1], x[2], x[3], y[0], y[1]);
+                    }
         }
-        __syncthreads();
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
+        for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int m = m0 + 32 * wm + 16 * mt + g + 8 * (q >> 1), n = n0 + 16 * wn + 8 * nt + 2 * tq + (q & 1);
-                if (m >= M || n >= N) continue;
-                if (gridDim.z > 1)
-                    part[((size_t)blockIdx.z * M + m) * N + n] = acc[mt][nt][q];
-                else
-                    fe(m, n, acc[mt][nt][q]);
+            for (int e = 0; e < 2; ++e) {
+                const int m = m0 + wm + 16 * mt + (lane >> 2) + 8 * e, n = n0 + wn + 8 * nt + 2 * (lane & 3);
+                if (m < M) fe(m, n, make_float2(acc[mt][nt][2 * e], acc[mt][nt][2 * e + 1]));
             }
 }
 
-template <int TN, int AS, bool BSPLIT, bool AKF, bool BKF, class FA, class FB, class FE>
-cudaError_t gemm_tc(int M, int N, int K, FA fa, FB fb, FE fe, float *part, size_t part_floats, cudaStream_t s)
+struct StorePart {  // part[z][m][n] = acc
+    float *part;
+    int rows, ld;
+    __device__ void operator()(int m, int n, float2 v) const
+    {
+        *reinterpret_cast<float2 *>(part + ((size_t)blockIdx.z * rows + m) * ld + n) = v;
+    }
+};
+struct StoreMask {  // out[m][n] = acc [mask[m][n] > 0]
+    float *out;
+    const float *mask;
+    int ld;
+    __device__ void operator()(int m, int n, float2 v) const
+    {
+        const size_t i = (size_t)m * ld + n;
+        const float2 k = ld2(mask + i);
+        *reinterpret_cast<float2 *>(out + i) = make_float2(k.x > 0.0f ? v.x : 0.0f, k.y > 0.0f ? v.y : 0.0f);
+    }
+};
+
+// K of fc1's forward product in quarters: 4 times the blocks (128 for a batch of 4096), and a quarter of the
+// additions in each of the tensor cores' accumulators, which round toward zero
+constexpr int kFc1Splits = 4;
+
+// splits of the batch in fc1's weight gradient (32 output blocks): a function of N alone, so that a step's
+// sums are in the same order on every run
+int fc1_splits(int N) { return std::max(1, std::min(8, (N + 255) / 256)); }
+
+template <int TA, int TB, bool AT, bool BT, class FE>
+cudaError_t gemm_terms(int M, int N, int K, int splits, const bf16 *A, size_t ta, int lda, const bf16 *B, size_t tb, int ldb,
+                       FE fe, cudaStream_t s)
 {
-    constexpr int TM = 4096 / TN;
-    const int gx = (N + TN - 1) / TN, gy = (M + TM - 1) / TM;
-    int splits = 1;  // split K when the output grid alone cannot fill the GPU and K is long
-    const long long blocks = (long long)gx * gy;
-    while (splits < 64 && blocks * splits < 2LL * sm_count() && K / (splits * 2) >= 256 &&
-           (size_t)(splits * 2) * M * N <= part_floats)
-        splits *= 2;
-    int kper = (K + splits - 1) / splits;
-    kper = (kper + kTrK - 1) / kTrK * kTrK;
-    k_gemm_tc<TN, AS, BSPLIT, AKF, BKF><<<dim3(gx, gy, splits), 256, 0, s>>>(M, N, K, kper, fa, fb, fe, part);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || splits == 1) return e;
-    k_split_reduce<<<grid_cap(((long long)M * N + 255) / 256), 256, 0, s>>>(M, N, splits, part, fe);
+    auto kern = k_gemm_terms<TA, TB, AT, BT, FE>;
+    const int smem = kGmSmem<TA, TB>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const int kper = ((K + splits - 1) / splits + kGmK - 1) / kGmK * kGmK;
+    kern<<<dim3(N / kGmN, (M + kGmM - 1) / kGmM, splits), 256, smem, s>>>(M, N, K, kper, A, ta, lda, B, tb, ldb, fe);
     return cudaGetLastError();
 }
 
-// Data gradient of a stride-2 conv layer (32 -> 32 channels) into the layer below, masked by its
-// ReLU: da[n][s][ci] = [z_prev[n][s][ci] > 0] sum over the taps k and positions t with
-// 2t + k - 1 = s of sum_c dz[n][t][c] W[c][k][ci]. An even s = 2u takes tap 1 at t = u, an odd
-// s = 2u + 1 taps 0 at t = u + 1 and 2 at t = u (the other taps fall between positions), so a
-// warp that takes the 16 positions t = u0 .. u0 + 15 of one beam (32 output positions) stages the
-// dz rows u0 .. u0 + 16 (two BF16 terms each, as k_gemm_tc's backward products; row u0 + 16 is
-// zero past the beam) and runs the even rows as a K = 32 product with tap 1 and the odd rows as a
-// K = 64 product with taps 0 and 2: half the products of the K = 96 im2col form, whose other half
-// are zeros. Weights are staged as [k][ci][c] BF16 (exact), row pitch kTrPitch.
-__global__ void __launch_bounds__(256) k_dgrad_conv(int N, int Lin, const float *__restrict__ dz,
-                                                    const bf16 *__restrict__ w, const float *__restrict__ zprev,
-                                                    float *__restrict__ out)
+// out[e] = sum over z of part[z][e], in order
+__global__ void k_split_reduce(int E, int splits, const float *__restrict__ part, float *__restrict__ out)
 {
-    __shared__ __align__(16) bf16 sW[kK * kCh * kTrPitch];
-    __shared__ __align__(16) bf16 sT[8][2][17 * kTrPitch];
-    const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, g = lane >> 2, tq = lane & 3;
-    for (int e = tid; e < kK * kCh * kCh; e += 256) {
-        const int k = e / (kCh * kCh), ci = (e / kCh) % kCh, c = e % kCh;
-        sW[(k * kCh + ci) * kTrPitch + c] = w[(c * kK + k) * kCh + ci];
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < E; e += gridDim.x * blockDim.x) {
+        float v = 0.0f;
+        for (int z = 0; z < splits; ++z) v += part[(size_t)z * E + e];
+        out[e] = v;
+    }
+}
+
+// ---- head -------------------------------------------------------------------------------------------
+//
+// z4[n][j] = b4[j] + the sums of fc1's product over the quarters of K (part1 [kFc1Splits][N][256]),
+// pred[n] = b5 + sum_j W5[j] relu(z4[n][j]) and, with targets, d = pred - y, dpred = 2 d / N,
+// dz4[n][j] = dpred W5[j] [z4 > 0] as two BF16 terms (dz, N * 256 elements apart) and the block's sums over its
+// rows of dpred relu(z4) (gW5), dz4 (gb4), dpred (gb5) and d^2 (loss) into part[block][514]. A
+// warp takes 4 consecutive rows, a lane the columns 4 lane + k and 128 + 4 lane + k.
+constexpr int kHeadRows = 32, kHeadOut = 2 * kHid + 2;
+__global__ void __launch_bounds__(256)
+    k_head(const float *__restrict__ part1, const bf16 *__restrict__ w, const float *__restrict__ params,
+           const float *__restrict__ y, int N, float *__restrict__ z4, float *__restrict__ pred, bf16 *__restrict__ dz,
+           float *__restrict__ part)
+{
+    __shared__ float sum[8][kHeadOut];
+    const int lane = lane_id(), wp = threadIdx.x >> 5;
+    float w5[8], b4[8], g5[8] = {}, g4[8] = {}, gb = 0.0f, loss = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        w5[k] = bf(w, oW5 + 128 * (k >> 2) + 4 * lane + (k & 3));
+        b4[k] = params[oB4 + 128 * (k >> 2) + 4 * lane + (k & 3)];
+    }
+    const float b5 = params[oB5];
+    for (int r = 0; r < kHeadRows / 8; ++r) {
+        const int n = blockIdx.x * kHeadRows + wp * (kHeadRows / 8) + r;
+        if (n >= N) break;
+        float z[8];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const size_t o = (size_t)n * kHid + 128 * q + 4 * lane;
+            float4 v[kFc1Splits];
+#pragma unroll
+            for (int k = 0; k < kFc1Splits; ++k) v[k] = *reinterpret_cast<const float4 *>(part1 + (size_t)k * N * kHid + o);
+#pragma unroll
+            for (int k = 1; k < kFc1Splits; ++k) v[0] = make_float4(v[0].x + v[k].x, v[0].y + v[k].y, v[0].z + v[k].z, v[0].w + v[k].w);
+            z[4 * q] = v[0].x + b4[4 * q];
+            z[4 * q + 1] = v[0].y + b4[4 * q + 1];
+            z[4 * q + 2] = v[0].z + b4[4 * q + 2];
+            z[4 * q + 3] = v[0].w + b4[4 * q + 3];
+            *reinterpret_cast<float4 *>(z4 + o) = make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
+        }
+        float a = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) a = fmaf(w5[k], relu(z[k]), a);
+        a = warp_sum(a) + b5;
+        if (lane == 0) pred[n] = a;
+        if (y) {
+            const float d = a - y[n], dp = 2.0f * d / (float)N;
+            loss = fmaf(d, d, loss);
+            gb += dp;
+            float v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                v[k] = z[k] > 0.0f ? dp * w5[k] : 0.0f;
+                g4[k] += v[k];
+                g5[k] = fmaf(dp, relu(z[k]), g5[k]);
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                unsigned t0[2], t1[2];
+                split<2>(make_float2(v[4 * q], v[4 * q + 1]), t0);
+                split<2>(make_float2(v[4 * q + 2], v[4 * q + 3]), t1);
+                const size_t o = (size_t)n * kHid + 128 * q + 4 * lane;
+                *reinterpret_cast<uint2 *>(dz + o) = make_uint2(t0[0], t1[0]);
+                *reinterpret_cast<uint2 *>(dz + (size_t)N * kHid + o) = make_uint2(t0[1], t1[1]);
+            }
+        }
+    }
+    if (!y) return;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int j = 128 * (k >> 2) + 4 * lane + (k & 3);
+        sum[wp][j] = g5[k];
+        sum[wp][kHid + j] = g4[k];
+    }
+    if (lane == 0) {
+        sum[wp][2 * kHid] = gb;
+        sum[wp][2 * kHid + 1] = loss;
     }
     __syncthreads();
-    const int Lout = Lin >> 1, tpb = Lout / 16;
-    const long long ntiles = (long long)N * tpb;
-    bf16 *const T[2] = {sT[wp][0], sT[wp][1]};
-    for (long long tile = blockIdx.x * 8LL + wp; tile < ntiles; tile += gridDim.x * 8LL) {
-        const int n = (int)(tile / tpb), u0 = (int)(tile % tpb) * 16;
-        for (int e = lane; e < 17 * (kCh / 2); e += 32) {
-            const int r = e / (kCh / 2), cp = e % (kCh / 2);
-            float2 v = make_float2(0.0f, 0.0f);
-            if (u0 + r < Lout) v = *reinterpret_cast<const float2 *>(dz + ((long long)n * Lout + u0 + r) * kCh + 2 * cp);
-            split_store(T, 2, r * kTrPitch + 2 * cp, v.x, v.y);
-        }
-        __syncwarp();
-        float ev[4][4] = {}, od[4][4] = {};
+    for (int j = threadIdx.x; j < kHeadOut; j += 256) {
+        float t = 0.0f;
 #pragma unroll
-        for (int ks = 0; ks < kCh; ks += 16) {
-            unsigned a[2][4], a1[2][4];  // rows u0 + g, + 8 (a) and u0 + g + 1, + 9 (a1)
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const bf16 *p = T[i] + g * kTrPitch + ks + 2 * tq;
-                a[i][0] = lds32(p);
-                a[i][1] = lds32(p + 8 * kTrPitch);
-                a[i][2] = lds32(p + 8);
-                a[i][3] = lds32(p + 8 * kTrPitch + 8);
-                a1[i][0] = lds32(p + kTrPitch);
-                a1[i][1] = lds32(p + 9 * kTrPitch);
-                a1[i][2] = lds32(p + kTrPitch + 8);
-                a1[i][3] = lds32(p + 9 * kTrPitch + 8);
-            }
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                unsigned b[3][2];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const bf16 *q = sW + (k * kCh + nt * 8 + g) * kTrPitch + ks + 2 * tq;
-                    b[k][0] = lds32(q);
-                    b[k][1] = lds32(q + 8);
-                }
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    mma_bf16(ev[nt], a[i][0], a[i][1], a[i][2], a[i][3], b[1][0], b[1][1]);
-                    mma_bf16(od[nt], a1[i][0], a1[i][1], a1[i][2], a1[i][3], b[0][0], b[0][1]);
-                    mma_bf16(od[nt], a[i][0], a[i][1], a[i][2], a[i][3], b[2][0], b[2][1]);
-                }
-            }
-        }
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int ci = nt * 8 + 2 * tq;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {  // fragment rows g, g + 8
-                const int u = u0 + g + 8 * h;
-#pragma unroll
-                for (int odd = 0; odd < 2; ++odd) {
-                    const long long i = ((long long)n * Lin + 2 * u + odd) * kCh + ci;
-                    const float2 m = *reinterpret_cast<const float2 *>(zprev + i);
-                    const float v0 = odd ? od[nt][2 * h] : ev[nt][2 * h], v1 = odd ? od[nt][2 * h + 1] : ev[nt][2 * h + 1];
-                    *reinterpret_cast<float2 *>(out + i) = make_float2(m.x > 0.0f ? v0 : 0.0f, m.y > 0.0f ? v1 : 0.0f);
-                }
-            }
-        }
-        __syncwarp();
+        for (int k = 0; k < 8; ++k) t += sum[k][j];
+        part[(size_t)blockIdx.x * kHeadOut + j] = t;
     }
 }
 
-cudaError_t dgrad_conv(int N, int Lin, const float *dz, const bf16 *w, const float *zprev, float *out, cudaStream_t s)
+// ---- the convolutions' backward pass ----------------------------------------------------------------
+//
+// One pass per 32 -> 32 conv layer over its dz [N][Lout][32] (Lout = Lin / 2), two warps per strip of 16
+// positions t, each for 16 of the channels of the layer below:
+//   data gradient: an even input position 2t takes tap 1 at t, an odd one 2t + 1 taps 0 at t + 1 and 2
+//     at t, so the strip and the strip one row on, as A operands, give the strips of positions 2t and
+//     2t + 1 (K = 32 and 64, no zero taps), masked by the layer below's ReLU;
+//   weight gradient: gW[c][k][ci] = sum over t of dz[t][c] relu(z)[2t + k - 1][ci], an MMA with the
+//     strip's 16 positions as K. Both operands are the fragments at hand transposed (movmatrix), and
+//     the 32 x 96 sums stay in registers over all of a warp's strips;
+//   bias gradient: the column sums of dz.
+// LAST (conv2): conv1's gradients follow at once from the strips of dz1, which is never stored.
+// The grid, the strips of each warp and the order of the sums depend only on N: the blocks' sums go to
+// part[block][...] and are added in block order (k_grads), so a step gives the same floats on every run.
+// The sums take 52 registers per lane, and two blocks of 8 warps per SM do not hide the strips' loads; the
+// next strip's rows are prefetched toward L1. A batch of 4096: 34 us (conv3) and 68 us (conv2 and conv1); one
+// warp per strip with all 32 channels (255 registers) 38 and 77 us; the separate data, weight and bias
+// gradient kernels 320 us.
+constexpr int kBwdWarps = 8, kBwdBlocks = 304;
+constexpr int kTrPitch = kCh + 8;  // row pitch of the staged weights: 80 B, eight rows in eight bank groups
+template <bool LAST>
+constexpr int kBwdOut = kCh * kK * kCh + kCh + (LAST ? kCh * kK * kCin + kCh : 0);
+
+__device__ __forceinline__ unsigned transpose8(unsigned v)
 {
-    const long long tiles = (long long)N * (Lin / 32);  // 16 output positions t per warp, 8 warps per block
-    k_dgrad_conv<<<grid_cap((tiles + 7) / 8), 256, 0, s>>>(N, Lin, dz, w, zprev, out);
-    return cudaGetLastError();
+    unsigned r;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+    return r;
+}
+
+// acc += (T_0 + T_1)^T (U_0 + U_1) without the last product: T (32 columns) and U (16) strips of 16
+// positions as two BF16 terms, transposed (T: A fragments of the 32 rows c, U: B fragments of two n8 tiles)
+__device__ __forceinline__ void strip_outer(float (&acc)[2][2][4], const unsigned (&T)[4][2][2], const unsigned (&U)[2][2][2])
+{
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const int i = p == 1, j = p == 2;
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+                mma_bf16(acc[mt][nt], T[2 * mt][0][i], T[2 * mt + 1][0][i], T[2 * mt][1][i], T[2 * mt + 1][1][i], U[nt][0][j],
+                         U[nt][1][j]);
+    }
+}
+
+template <bool LAST>
+__global__ void __launch_bounds__(kBwdWarps * 32, 2)
+    k_conv_bwd(int N, int Lin, const float *__restrict__ dz, const bf16 *__restrict__ w, const float *__restrict__ zprev,
+               const bf16 *__restrict__ x, float *__restrict__ out, float *__restrict__ part)
+{
+    constexpr int kO = kBwdOut<LAST>, kW = kCh * kK * kCh;
+    __shared__ __align__(16) bf16 sW[kK * kCh * kTrPitch];  // [k][ci][c]
+    __shared__ float sum[kO];
+    for (int e = threadIdx.x; e < kK * kCh * kCh; e += kBwdWarps * 32) {
+        const int k = e / (kCh * kCh), ci = (e / kCh) % kCh, c = e % kCh;
+        sW[(k * kCh + ci) * kTrPitch + c] = w[(chan(c) * kK + k) * kCh + chan(ci)];
+    }
+    for (int e = threadIdx.x; e < kO; e += kBwdWarps * 32) sum[e] = 0.0f;
+    __syncthreads();
+    const int lane = lane_id(), g = lane >> 2, wq = lane & 3, wp = threadIdx.x >> 5;
+    const int half = wp & 1, ch = 16 * half;  // this warp's columns of the layer below (channels 16 half + 4w .. + 3)
+    const int Lout = Lin >> 1, tpb = Lout / 16;
+    const long long units = (long long)N * tpb, np = (long long)gridDim.x * (kBwdWarps / 2),
+                    me = (long long)blockIdx.x * (kBwdWarps / 2) + (wp >> 1);
+    const long long u0 = units * me / np, u1 = units * (me + 1) / np;
+    float acc[3][2][2][4] = {}, acc1[4] = {};
+    float2 gb[2] = {}, gb1[2] = {};
+    for (long long u = u0; u < u1; ++u) {
+        const int n = (int)(u / tpb), t0 = (int)(u % tpb) * 16;
+        if (u + 1 < u1) {  // the next strip's rows, which follow this one's, toward L1
+            const float *nd = dz + (size_t)(u + 1) * 16 * kCh, *nz = zprev + (size_t)(u + 1) * 32 * kCh;
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(lane < 16 ? nd + lane * kCh : nz + (lane - 16 + 16 * half) * kCh));
+        }
+        unsigned a[4][2][2], b[4][2][2];  // terms of dz at t and at t + 1
+        const float *dr = dz + ((size_t)n * Lout + t0 + g) * kCh + 4 * wq;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            float2 v[4];
+            load8(dr + 8 * e * kCh, v);
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) split<2>(v[nt], a[nt][e]);
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt) {
+                gb[nt].x += half ? v[nt + 2].x : v[nt].x;
+                gb[nt].y += half ? v[nt + 2].y : v[nt].y;
+            }
+        }
+        {  // one row on: lane + 4's row, the last from memory (zero past the beam)
+            float2 v[4] = {};
+            if (g == 7 && t0 + 16 < Lout) load8(dr + 9 * kCh, v);
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) {
+                unsigned t[2];
+                split<2>(v[nt], t);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const unsigned lo = __shfl_sync(kFull, a[nt][0][i], lane + 4), hi = __shfl_sync(kFull, a[nt][1][i], lane + 4);
+                    b[nt][0][i] = g == 7 ? hi : lo;
+                    b[nt][1][i] = g == 7 ? t[i] : hi;
+                }
+            }
+        }
+        float ev[2][4] = {}, od[2][4] = {};
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+            unsigned bw[3][2][2];
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                ldsm_x4(smem_u32(sW + (k * kCh + ch + (lane & 7) + 8 * (lane >> 4)) * kTrPitch + ks * 16 + 8 * ((lane >> 3) & 1)),
+                        bw[k][0][0], bw[k][0][1], bw[k][1][0], bw[k][1][1]);
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    mma_bf16(ev[q], a[2 * ks][0][i], a[2 * ks][1][i], a[2 * ks + 1][0][i], a[2 * ks + 1][1][i], bw[1][q][0],
+                             bw[1][q][1]);
+                    mma_bf16(od[q], b[2 * ks][0][i], b[2 * ks][1][i], b[2 * ks + 1][0][i], b[2 * ks + 1][1][i], bw[0][q][0],
+                             bw[0][q][1]);
+                    mma_bf16(od[q], a[2 * ks][0][i], a[2 * ks][1][i], a[2 * ks + 1][0][i], a[2 * ks + 1][1][i], bw[2][q][0],
+                             bw[2][q][1]);
+                }
+        }
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) a[nt][e][i] = transpose8(a[nt][e][i]);
+        // the layer below at 2t + tap - 1, rows g and g + 8 of the strip: the other factor of the weight
+        // gradient and (taps 1, 2) the mask of the data gradient at 2t and 2t + 1. Tap 0 is tap 2's strip one
+        // row down, its first row from memory.
+        unsigned p[2][2][2], first[2][2];
+        {
+            const int r = 2 * t0 - 1;
+            float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (g == 0 && r >= 0) z = *reinterpret_cast<const float4 *>(zprev + ((size_t)n * Lin + r) * kCh + 16 * half + 4 * wq);
+            split<2>(relu2(make_float2(z.x, z.y)), first[0]);
+            split<2>(relu2(make_float2(z.z, z.w)), first[1]);
+        }
+#pragma unroll
+        for (int tap = 1; tap < 3; ++tap) {
+            const size_t o = ((size_t)n * Lin + 2 * (t0 + g) + tap - 1) * kCh + 16 * half + 4 * wq;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float4 z = *reinterpret_cast<const float4 *>(zprev + o + 16 * e * kCh);
+                split<2>(relu2(make_float2(z.x, z.y)), p[0][e]);
+                split<2>(relu2(make_float2(z.z, z.w)), p[1][e]);
+                float(&d)[2][4] = tap == 1 ? ev : od;
+                d[0][2 * e] = z.x > 0.0f ? d[0][2 * e] : 0.0f;
+                d[0][2 * e + 1] = z.y > 0.0f ? d[0][2 * e + 1] : 0.0f;
+                d[1][2 * e] = z.z > 0.0f ? d[1][2 * e] : 0.0f;
+                d[1][2 * e + 1] = z.w > 0.0f ? d[1][2 * e + 1] : 0.0f;
+                if (!LAST)
+                    *reinterpret_cast<float4 *>(out + o + 16 * e * kCh) =
+                        make_float4(d[0][2 * e], d[0][2 * e + 1], d[1][2 * e], d[1][2 * e + 1]);
+            }
+            unsigned q[2][2][2];
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) q[nt][e][i] = transpose8(p[nt][e][i]);
+            strip_outer(acc[tap], a, q);
+        }
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const unsigned lo = __shfl_sync(kFull, p[nt][0][i], lane + 28), hi = __shfl_sync(kFull, p[nt][1][i], lane + 28);
+                p[nt][0][i] = transpose8(g == 0 ? first[nt][i] : lo);
+                p[nt][1][i] = transpose8(g == 0 ? lo : hi);
+            }
+        strip_outer(acc[0], a, p);
+        if (LAST) {
+            // conv1: gW1[c][k][ci] = sum over positions p of dz1[p][c] x[2p + k - 1][ci], column 2k + ci of the
+            // n8 tile (6 of 8 used; x is exact in BF16)
+            const unsigned short *xr = reinterpret_cast<const unsigned short *>(x) + (size_t)n * kL * kCin;
+#pragma unroll
+            for (int odd = 0; odd < 2; ++odd) {  // p = 2t + odd
+                float(&d)[2][4] = odd ? od : ev;
+                unsigned t[2][2][2], bx[2];
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    gb1[nt].x += d[nt][0] + d[nt][2];
+                    gb1[nt].y += d[nt][1] + d[nt][3];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) split<2>(make_float2(d[nt][2 * e], d[nt][2 * e + 1]), t[nt][e]);
+                }
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int i0 = 4 * (t0 + 2 * wq + 8 * e) + 2 * odd - 1 + (g >> 1);  // sample of row 2w; row 2w + 1: + 4
+                    const unsigned lo = g < 6 && i0 >= 0 ? __ldg(xr + 2 * i0 + (g & 1)) : 0u;
+                    const unsigned hi = g < 6 ? __ldg(xr + 2 * (i0 + 4) + (g & 1)) : 0u;
+                    bx[e] = lo | hi << 16;
+                }
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    mma_bf16(acc1, transpose8(t[0][0][i]), transpose8(t[1][0][i]), transpose8(t[0][1][i]),
+                             transpose8(t[1][1][i]), bx[0], bx[1]);
+            }
+        }
+    }
+    // the columns' sums over the eight row groups, then the block's sums, pair by pair of warps (the two of a
+    // pair hold different outputs)
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            gb[nt].x += __shfl_xor_sync(kFull, gb[nt].x, o);
+            gb[nt].y += __shfl_xor_sync(kFull, gb[nt].y, o);
+            if (LAST) {
+                gb1[nt].x += __shfl_xor_sync(kFull, gb1[nt].x, o);
+                gb1[nt].y += __shfl_xor_sync(kFull, gb1[nt].y, o);
+            }
+        }
+    for (int k = 0; k < kBwdWarps / 2; ++k) {
+        if ((wp >> 1) == k) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int row = g + 8 * (q >> 1), col = 2 * wq + (q & 1);
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                    for (int tap = 0; tap < 3; ++tap)
+#pragma unroll
+                        for (int nt = 0; nt < 2; ++nt)
+                            sum[chan(16 * mt + row) * kK * kCh + tap * kCh + chan(ch + 8 * nt + col)] += acc[tap][mt][nt][q];
+                if (LAST && col < kK * kCin) sum[kW + kCh + chan(ch + row) * kK * kCin + col] += acc1[q];
+            }
+            if (g == 0) {
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    const int c = ch + 4 * wq + 2 * nt;
+                    sum[kW + c] += gb[nt].x;
+                    sum[kW + c + 1] += gb[nt].y;
+                    if (LAST) {
+                        sum[kO - kCh + c] += gb1[nt].x;
+                        sum[kO - kCh + c + 1] += gb1[nt].y;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+    for (int e = threadIdx.x; e < kO; e += kBwdWarps * 32) part[(size_t)blockIdx.x * kO + e] = sum[e];
+}
+
+// The gradients from the blocks' sums: output o of the list [head | conv3 | conv2 and conv1] adds its column
+// over the blocks, in a fixed order: a block takes 32 outputs (one per lane), its 8 warps the 8 contiguous
+// eighths of the blocks, and the eighths' sums are added in order.
+__global__ void __launch_bounds__(256)
+    k_grads(int N, int head_blocks, const float *__restrict__ head, const float *__restrict__ c3, const float *__restrict__ c2,
+            int conv_blocks, float *__restrict__ grad, float *__restrict__ loss)
+{
+    constexpr int O3 = kBwdOut<false>, O2 = kBwdOut<true>, kW = kCh * kK * kCh;
+    __shared__ float sh[8][32];
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const int o = blockIdx.x * 32 + lane;
+    const float *src = nullptr;
+    int stride = 0, nb = 0;
+    float *dst = nullptr;
+    if (o < kHeadOut) {
+        src = head + o;
+        stride = kHeadOut;
+        nb = head_blocks;
+        dst = o < kHid ? grad + oW5 + o : o < 2 * kHid ? grad + oB4 + o - kHid : o == 2 * kHid ? grad + oB5 : loss;
+    } else if (o < kHeadOut + O3) {
+        const int e = o - kHeadOut;
+        src = c3 + e;
+        stride = O3;
+        nb = conv_blocks;
+        dst = grad + (e < kW ? oW3 + e : oB3 + e - kW);
+    } else if (o < kHeadOut + O3 + O2) {
+        const int e = o - kHeadOut - O3;
+        src = c2 + e;
+        stride = O2;
+        nb = conv_blocks;
+        dst = grad + (e < kW ? oW2 + e : e < kW + kCh ? oB2 + e - kW : e < O2 - kCh ? oW1 + e - kW - kCh : oB1 + e - (O2 - kCh));
+    }
+    const int b0 = (int)((long long)nb * w / 8), b1 = (int)((long long)nb * (w + 1) / 8);
+    float t = 0.0f;
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b) t += src[(size_t)b * stride];
+    sh[w][lane] = t;
+    __syncthreads();
+    if (w == 0 && dst) {
+        float v = 0.0f;
+        for (int k = 0; k < 8; ++k) v += sh[k][lane];
+        *dst = dst == loss ? v / (float)N : v;
+    }
 }
 
 // ---- the conv stack in registers ------------------------------------------------------------------
@@ -749,7 +937,6 @@ cudaError_t dgrad_conv(int N, int Lin, const float *dz, const bf16 *w, const flo
 // conv2's weights read per strip, 3.38 - 3.61 ms with the next beam's samples fetched ahead (registers),
 // 3.78 ms with both strips of a beam unrolled.
 constexpr int kConvWarps = 4;
-constexpr int kS2 = 104;  // W2 / W3 row stride (bf16): 208 B, eight rows in eight bank groups
 constexpr int kXWords = 4 + kL;  // a beam's profile, with zeros before it
 // block: W1 [32][8], W2 / W3 [32][104] bf16, kL zero words, then each warp's profile
 constexpr int kConvSmem = kCh * 8 * 2 + 2 * kCh * kS2 * 2 + kL * 4 + kConvWarps * kXWords * 4;
@@ -779,18 +966,6 @@ __device__ __forceinline__ void shift_rows(const unsigned (&P)[4][2], unsigned (
         S[nt][0] = first ? carry[nt] : lo;
         S[nt][1] = first ? lo : hi;
         carry[nt] = hi;
-    }
-}
-
-// Weight fragments of k-step ks (16 of the K = 96 inputs) of a conv layer for the four n8 tiles
-__device__ __forceinline__ void load_wfrag(const bf16 *Wt, int ks, unsigned (&bw)[4][2])
-{
-    const int lane = lane_id();
-#pragma unroll
-    for (int np = 0; np < 2; ++np) {
-        const int row = np * 16 + (lane & 7) + 8 * (lane >> 4);
-        ldsm_x4(smem_u32(Wt + row * kS2 + ks * 16 + 8 * ((lane >> 3) & 1)), bw[2 * np][0], bw[2 * np][1],
-                bw[2 * np + 1][0], bw[2 * np + 1][1]);
     }
 }
 
@@ -1272,9 +1447,8 @@ size_t surrogate_train_floats(int N)
 {
     const size_t n = (size_t)N;
     const size_t z = n * (128 + 64 + 32) * kCh + n * kHid;  // z1..z4
-    const size_t g = n * 128 * kCh;                          // g1, g2: the largest gradient
-    const size_t part = (size_t)64 * kHid * kFlat;           // split-K partials (up to 64 x the largest output), also
-                                                             // the batch reductions' (<= kRedMaxBlocks x 3072)
+    const size_t g = n * 128 * kCh;                          // relu(z3) and dz4 in terms, dz3, dz2: 4864 n of 2 g = 8192 n
+    const size_t part = (size_t)64 * kHid * kFlat;           // the sums over blocks (fc1's, the head's, the convolutions')
     return z + 3 * ((n + 3) & ~(size_t)3) + 2 * g + part + 64;  // pred, dpred, lossp each padded to 4 floats
 }
 
@@ -1291,72 +1465,55 @@ cudaError_t launch_surrogate_loss_grad(const float *params, const void *wbf16, c
                                        float *grad, float *loss, float *pred_out, float *ws, cudaStream_t s)
 {
     const bf16 *w = (const bf16 *)wbf16;
-    const __nv_bfloat162 *xb = (const __nv_bfloat162 *)x;
-    TrainBufs t;
+    const size_t n = (size_t)N, pad = (n + 3) & ~(size_t)3;
     float *q = ws;
-    auto take = [&](size_t n) {  // every buffer 16-byte aligned (float4 loads)
+    auto take = [&](size_t floats) {  // every buffer 16-byte aligned
         float *r = q;
-        q += (n + 3) & ~(size_t)3;
+        q += (floats + 3) & ~(size_t)3;
         return r;
     };
-    t.z1 = take((size_t)N * 128 * kCh);
-    t.z2 = take((size_t)N * 64 * kCh);
-    t.z3 = take((size_t)N * 32 * kCh);
-    t.z4 = take((size_t)N * kHid);
-    t.pred = take(N);
-    t.dpred = take(N);
-    t.lossp = take(N);
-    t.g1 = take((size_t)N * 128 * kCh);
-    t.g2 = take((size_t)N * 128 * kCh);
-    t.part = q;
-    t.part_floats = (size_t)64 * kHid * kFlat;
+    float *z1 = take(n * 128 * kCh), *z2 = take(n * 64 * kCh), *z3 = take(n * 32 * kCh), *z4 = take(n * kHid);
+    float *pred_ws = take(pad);
+    bf16 *h = (bf16 *)take(n * kFlat * 3 / 2);  // relu(z3), three terms
+    bf16 *dz4 = (bf16 *)take(n * kHid);         // two terms
+    float *dz3 = take(n * kFlat), *dz2 = take(n * 64 * kCh);
+    const int splits = fc1_splits(N), head_blocks = (N + kHeadRows - 1) / kHeadRows;
+    float *part4 = take((size_t)splits * kHid * kFlat), *part_h = take((size_t)head_blocks * kHeadOut);
+    float *part3 = take((size_t)kBwdBlocks * kBwdOut<false>), *part2 = take((size_t)kBwdBlocks * kBwdOut<true>);
+    bf16 *w4 = (bf16 *)w + oW4;
     cudaError_t e;
 #define FSMI_TRY(...)            \
     do {                         \
         e = (__VA_ARGS__);       \
         if (e != cudaSuccess) return e; \
     } while (0)
+    if ((uintptr_t)w4 & 15) {  // weights off a 16-byte boundary: the copies of the products need an aligned W4
+        w4 = (bf16 *)take((size_t)kHid * kFlat / 2);
+        FSMI_TRY(cudaMemcpyAsync(w4, w + oW4, (size_t)kHid * kFlat * sizeof(bf16), cudaMemcpyDeviceToDevice, s));
+    }
     // forward
-    FSMI_TRY(gemm_tc<32, 3, false, true, true>(N * 128, kCh, kK * kCin, ConvA1{xb}, WConv{w + oW1, kCin},
-                                            StoreBias{t.z1, params + oB1, kCh}, t.part, t.part_floats, s));
-    FSMI_TRY(gemm_tc<32, 3, false, true, true>(N * 64, kCh, kK * kCh, ConvA{t.z1, 128}, WConv{w + oW2, kCh},
-                                            StoreBias{t.z2, params + oB2, kCh}, t.part, t.part_floats, s));
-    FSMI_TRY(gemm_tc<32, 3, false, true, true>(N * 32, kCh, kK * kCh, ConvA{t.z2, 64}, WConv{w + oW3, kCh},
-                                            StoreBias{t.z3, params + oB3, kCh}, t.part, t.part_floats, s));
-    FSMI_TRY(gemm_tc<64, 3, false, true, true>(N, kHid, kFlat, ReluRow{t.z3, kFlat}, WT{w + oW4, kFlat},
-                                            StoreBias{t.z4, params + oB4, kHid}, t.part, t.part_floats, s));
-    float *pred = pred_out ? pred_out : t.pred;
-    k_head<<<grid_cap((N + 7) / 8), 256, 0, s>>>(t.z4, w, params, y, N, pred, t.dpred, t.lossp);
+    k_convs_fwd<<<grid_cap(((long long)N + kFwdWarps - 1) / kFwdWarps), kFwdWarps * 32, 0, s>>>(N, (const unsigned *)x, w, params, z1,
+                                                                                              z2, z3, h, n * kFlat);
+    FSMI_TRY(cudaGetLastError());
+    float *part1 = dz3;  // fc1's sums by quarters of K, added by the head
+    FSMI_TRY(gemm_terms<3, 1, false, false>(N, kHid, kFlat, kFc1Splits, h, n * kFlat, kFlat, w4, 0, kFlat,
+                                            StorePart{part1, N, kHid}, s));
+    k_head<<<head_blocks, 256, 0, s>>>(part1, w, params, y, N, z4, pred_out ? pred_out : pred_ws, dz4, part_h);
     FSMI_TRY(cudaGetLastError());
     if (!y) return cudaSuccess;
-    k_loss<<<1, 1024, 0, s>>>(t.lossp, N, loss);
+    // backward: fc1's weights gW4[j][i] = sum_n dz4[n][j] relu(z3)[n][i] and data dz3 = (dz4 W4) [z3 > 0]
+    FSMI_TRY(gemm_terms<2, 2, true, true>(kHid, kFlat, N, splits, dz4, n * kHid, kHid, h, n * kFlat, kFlat,
+                                          StorePart{part4, kHid, kFlat}, s));
+    k_split_reduce<<<grid_cap(kHid * kFlat / 256), 256, 0, s>>>(kHid * kFlat, splits, part4, grad + oW4);
     FSMI_TRY(cudaGetLastError());
-    // backward: head
-    FSMI_TRY(colsum(N, kHid, W5Grad{t.dpred, t.z4}, grad + oW5, t.part, s));
-    FSMI_TRY(colsum(N, 1, B5Grad{t.dpred}, grad + oB5, t.part, s));
-    float *dz4 = t.g1;  // [N][256]
-    k_dz4<<<grid_cap(((long long)N * kHid + 255) / 256), 256, 0, s>>>(t.z4, t.dpred, w, N, dz4);
+    FSMI_TRY(gemm_terms<2, 1, false, true>(N, kFlat, kHid, 1, dz4, n * kHid, kHid, w4, 0, kFlat, StoreMask{dz3, z3, kFlat}, s));
+    // conv3, then conv2 and conv1
+    k_conv_bwd<false><<<kBwdBlocks, kBwdWarps * 32, 0, s>>>(N, 64, dz3, w + oW3, z2, nullptr, dz2, part3);
     FSMI_TRY(cudaGetLastError());
-    FSMI_TRY(colsum(N, kHid, SumDz{dz4, kHid}, grad + oB4, t.part, s));
-    // fc1: gW4[j][i] = sum_n dz4[n][j] relu(z3)[n][i]; dz3 = (dz4 W4) [z3 > 0]
-    FSMI_TRY(gemm_tc<64, 2, true, false, false>(kHid, kFlat, N, RowT{dz4, kHid}, ReluRow{t.z3, kFlat},
-                                             Store{grad + oW4, kFlat}, t.part, t.part_floats, s));
-    float *dz3 = t.g2;  // [N][32][32]
-    FSMI_TRY(gemm_tc<64, 2, false, true, false>(N, kFlat, kHid, RowN{dz4, kHid}, WRow{w + oW4, kFlat},
-                                             StoreMask{dz3, t.z3, kFlat}, t.part, t.part_floats, s));
-    // conv3: weights from relu(z2); data gradient into dz2 = (...) [z2 > 0]
-    FSMI_TRY(wgrad<kCh>(N * 32, 64, dz3, t.z2, nullptr, grad + oW3, t.part, s));
-    FSMI_TRY(colsum(N * 32, kCh, SumDz{dz3, kCh}, grad + oB3, t.part, s));
-    float *dz2 = t.g1;  // [N][64][32]
-    FSMI_TRY(dgrad_conv(N, 64, dz3, w + oW3, t.z2, dz2, s));
-    // conv2
-    FSMI_TRY(wgrad<kCh>(N * 64, 128, dz2, t.z1, nullptr, grad + oW2, t.part, s));
-    FSMI_TRY(colsum(N * 64, kCh, SumDz{dz2, kCh}, grad + oB2, t.part, s));
-    float *dz1 = t.g2;  // [N][128][32]
-    FSMI_TRY(dgrad_conv(N, 128, dz2, w + oW2, t.z1, dz1, s));
-    // conv1
-    FSMI_TRY(wgrad<kCin>(N * 128, kL, dz1, nullptr, xb, grad + oW1, t.part, s));
-    FSMI_TRY(colsum(N * 128, kCh, SumDz{dz1, kCh}, grad + oB1, t.part, s));
+    k_conv_bwd<true><<<kBwdBlocks, kBwdWarps * 32, 0, s>>>(N, 128, dz2, w + oW2, z1, (const bf16 *)x, nullptr, part2);
+    FSMI_TRY(cudaGetLastError());
+    const int outs = kHeadOut + kBwdOut<false> + kBwdOut<true>;
+    k_grads<<<(outs + 31) / 32, 256, 0, s>>>(N, head_blocks, part_h, part3, part2, kBwdBlocks, grad, loss);
 #undef FSMI_TRY
     return cudaGetLastError();
 }
