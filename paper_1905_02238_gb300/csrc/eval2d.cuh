@@ -694,7 +694,7 @@ __device__ __forceinline__ float beam_sum(const DevParams &p, int n, float *sl, 
     const float cs = p.inv_s2 * (float)kSqrtLog2e;  // distance -> tail variable
     float I = 0.0f;
     if (n > 0) {
-        const float pe0 = cell_prefixes4(sp, sc, sx, n, VAR == FSMI_UNIFORM);
+        const float pe0 = cell_prefixes(sp, sc, sx, n, VAR == FSMI_UNIFORM);
         if (VAR == FSMI_EXACT || VAR == kExactFullSweep) {
             const float mu0 = sl[0] * cs - 0.5f * cs;  // e_0 centre, l_1 - 1/2 (scaled)
             build_pairs(sl, sc, n, cs);

@@ -27,16 +27,9 @@
 
 namespace fsmi {
 
-// Per-cell gain f(delta_occ, r) (which = 0) or f(delta_emp, r) (which = 1) of the RLE kernels: the
-// host-fitted Chebyshev series when it is accurate for these deltas, else the closed form.
-__device__ __forceinline__ float rle_gain(const DevParams &p, int which, float o)
-{
-    return p.gain_fit ? gain_series(p.gfit[which], o) : cell_gain(which ? p.demp : p.docc, o);
-}
-
-// Both gains of one o: the two series evaluated together in packed FP32 (each half of an f32x2
-// operation rounds as the scalar one does, so fo and fe equal rle_gain(p, 0, o) and
-// rle_gain(p, 1, o) bit for bit), or the closed forms.
+// Gains f(delta_occ, o) and f(delta_emp, o) of one cell: the host-fitted polynomials of h(o) = f / (o (1 - o))
+// where they are accurate for these deltas (both together in packed FP32, Horner's rule), else the closed
+// forms.
 __device__ __forceinline__ void rle_gains(const DevParams &p, float o, float &fo, float &fe)
 {
     if (!p.gain_fit) {
@@ -44,16 +37,18 @@ __device__ __forceinline__ void rle_gains(const DevParams &p, float o, float &fo
         fe = cell_gain(p.demp, o);
         return;
     }
-    const float x2 = __fmaf_rn(4.0f, o, -2.0f);  // 2x, x = 2o - 1
-    const f32x2 X2 = pack2(x2, x2);
-    f32x2 b1 = pack2(0.0f, 0.0f), b2 = b1;
+    const float x = __fmaf_rn(2.0f, o, -1.0f);
+    const f32x2 X = pack2(x, x);
+    f32x2 h;
+    if (p.gain_fit == 2) {
+        h = pack2(p.gfit2[kGainShortTerms - 1][0], p.gfit2[kGainShortTerms - 1][1]);
 #pragma unroll
-    for (int k = kGainFitTerms - 1; k >= 1; --k) {
-        const f32x2 b0 = fma2(X2, b1, sub2(pack2(p.gfit2[k][0], p.gfit2[k][1]), b2));
-        b2 = b1;
-        b1 = b0;
+        for (int k = kGainShortTerms - 2; k >= 0; --k) h = fma2(h, X, pack2(p.gfit2[k][0], p.gfit2[k][1]));
+    } else {
+        h = pack2(p.gfit2[kGainFitTerms - 1][0], p.gfit2[kGainFitTerms - 1][1]);
+#pragma unroll
+        for (int k = kGainFitTerms - 2; k >= 0; --k) h = fma2(h, X, pack2(p.gfit2[k][0], p.gfit2[k][1]));
     }
-    const f32x2 h = fma2(mul2(pack2(0.5f, 0.5f), X2), b1, sub2(pack2(p.gfit2[0][0], p.gfit2[0][1]), b2));
     const float w = __fmul_rn(o, __fsub_rn(1.0f, o));
     unpack2(mul2(pack2(w, w), h), fo, fe);
 }
@@ -156,8 +151,10 @@ static __device__ void run_prefixes(const RunSmem &r, int nr, const DevParams &p
     for (int u = lo; u < hi; ++u) {
         const float o = r.O[u];
         const int L = r.L[u];
+        float fo, fe;
+        rle_gains(p, o, fo, fe);
         prod *= ipowf(1.0f - o, L);
-        sum = fmaf((float)L, rle_gain(p, 1, o), sum);
+        sum = fmaf((float)L, fe, sum);
     }
     const float ip = warp_incl_mul(prod);
     const float is = warp_incl_add(sum);
@@ -171,10 +168,11 @@ static __device__ void run_prefixes(const RunSmem &r, int nr, const DevParams &p
         const float o = r.O[u];
         const int L = r.L[u];
         const float x = 1.0f - o;
-        const float fe = rle_gain(p, 1, o);
+        float fo, fe;
+        rle_gains(p, o, fo, fe);
         r.X[u] = x;
         r.F[u] = fe;
-        r.A[u] = D + rle_gain(p, 0, o);
+        r.A[u] = D + fo;
         r.O[u] = E * o;
         E *= ipowf(x, L);
         D = fmaf((float)L, fe, D);
@@ -246,54 +244,144 @@ static __device__ float pairs_thm5(const RunSmem &r, int nr, const float2 *tab, 
 
 constexpr int kArraysRLE = 7;                  // per-warp shared arrays (each `stride` floats)
 
-// run containing virtual cell i: the last u with S[u] <= i
-__device__ __forceinline__ int run_of(const int *S, int nr, int i)
+// C keeps its first cell at a 16-byte boundary, conv_pad(K) >= K floats after its array's start
+__host__ __device__ constexpr int conv_pad(int K) { return (K + 3) & ~3; }
+
+// ---- the cell form ---------------------------------------------------------------------------------
+//
+// A ray's cells go through in blocks of 128, four consecutive cells per lane: the gains, Algorithm 2's and 3's
+// prefixes within the lane, one warp scan per block for the lanes' totals, and P(e_j) and C_k stored once, 16
+// bytes per lane. The fused kernel runs it on the samples as they arrive (no o, f_occ or f_emp array is
+// written and read back), the run-input kernel on the decompressed runs; the same operations in the
+// same order, so the two give the same floats.
+
+// prefixes carried from block to block
+struct CellScan {
+    float E, q;  // prod (1 - o) and sum f_emp of the cells before the block
+};
+
+// One block: o of this lane's cells i0 .. i0 + 3 (zero from the ray's end on); stores P in CP and C in CB where
+// i0 < n.
+__device__ __forceinline__ void scan_block(const DevParams &p, const float (&o)[4], int i0, int n, CellScan &s, float *CP,
+                                           float *CB)
 {
-    int lo = 0, len = nr;
-    while (len > 0) {
-        const int half = len >> 1;
-        if (S[lo + half] <= i) {
-            lo += half + 1;
-            len -= half + 1;
-        } else {
-            len = half;
-        }
+    float fo[4], fe[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) rle_gains(p, o[t], fo[t], fe[t]);
+    const float prod = warp_incl_mul(((1.0f - o[0]) * (1.0f - o[1])) * ((1.0f - o[2]) * (1.0f - o[3])));
+    const float sum = warp_incl_add((fe[0] + fe[1]) + (fe[2] + fe[3]));
+    float E = __shfl_up_sync(kFull, prod, 1), q = __shfl_up_sync(kFull, sum, 1);
+    const int lane = lane_id();
+    E = lane == 0 ? s.E : s.E * E;
+    q = lane == 0 ? s.q : s.q + q;
+    s.E *= __shfl_sync(kFull, prod, 31);
+    s.q += __shfl_sync(kFull, sum, 31);
+    float4 P, C;
+    P.x = E * o[0];  // Algorithm 2
+    E *= 1.0f - o[0];
+    P.y = E * o[1];
+    E *= 1.0f - o[1];
+    P.z = E * o[2];
+    E *= 1.0f - o[2];
+    P.w = E * o[3];
+    C.x = q + fo[0];  // Algorithm 3
+    q += fe[0];
+    C.y = q + fo[1];
+    q += fe[1];
+    C.z = q + fo[2];
+    q += fe[2];
+    C.w = q + fo[3];
+    if (i0 < n) {
+        *reinterpret_cast<float4 *>(CP + i0) = P;
+        *reinterpret_cast<float4 *>(CB + i0) = C;
     }
-    return lo - 1;
 }
 
-// sum_j P(e_j) sum_{|d| <= K} g(d) C_{j+d} over j in this lane's cells (P in CP, C at CC[K + k],
-// zero-padded by K on both sides), the taps added in increasing d. A compile-time radius KK keeps
-// the 2 KK + 1 kernel values in registers for the whole ray (one shared load per tap instead of
-// two); both forms add the same products in the same order. Only the kernels of the other
-// variants take this register form (FIXED); the Theorem 5 kernel, whose rays mostly take its
-// windowed cell form, keeps the taps in registers in window_conv_k instead.
-template <int KK>
-__device__ __forceinline__ float band_conv_k(const float *CP, const float *CC, const float *gtab, int n)
+// K zeros before C_0 and K + 8 from C_n on (scan_block leaves up to three entries past C_{n-1} undefined)
+__device__ __forceinline__ void pad_conv(float *CB, int K, int n)
 {
-    float g[2 * KK + 1];
-#pragma unroll
-    for (int d = 0; d <= 2 * KK; ++d) g[d] = gtab[d];
+    for (int i = lane_id(); i < K + 8; i += 32) {
+        if (i < K) CB[-1 - i] = 0.0f;
+        CB[n + i] = 0.0f;
+    }
+    __syncwarp();
+}
+
+// sum_j P(e_j) sum_{|d| <= K} g(d) C_{j+d} (P in CP, C at CB, zero-padded on both sides). With a compile-time
+// radius KK a lane takes V consecutive j: C comes in 16-byte loads, (V + 2 KK) / 4 of them for V outputs
+// instead of one load per tap and output, and every loaded pair (C_k, C_{k+1}) meets all the output pairs it
+// belongs to in packed FP32 operations: outputs (j, j + 1) for one parity of the tap, (j - 1, j) for the
+// other, each in accumulators of its own. The kernel values are operands from the launch parameters. On the
+// 512x512x128 batch one output per lane and one load per tap took 329 of 1,741 warp instructions per ray
+// and a third of the shared-memory wavefronts.
+template <int KK, int V>
+__device__ __forceinline__ float band_conv_v(const float *CP, const float *CB, const RleTable &t, int n)
+{
+    constexpr int kPad = conv_pad(KK), kSh = kPad - KK;  // inputs from j0 - kPad: input k meets output j with tap k - j - kSh
+    constexpr int kQuads = (kPad + KK + V + 3) / 4;
+    static_assert(V % 4 == 0 && KK <= kConvMaxRadius, "outputs per lane");
     float v = 0.0f;
-    for (int j = lane_id(); j < n; j += 32) {
-        float acc = 0.0f;
+    for (int j0 = V * lane_id(); j0 < n; j0 += 32 * V) {
+        f32x2 ev[V / 2], od[V / 2 + 1];
 #pragma unroll
-        for (int d = 0; d <= 2 * KK; ++d) acc = fmaf(g[d], CC[j + d], acc);
-        v = fmaf(CP[j], acc, v);
+        for (int q = 0; q < V / 2; ++q) ev[q] = pack2(0.0f, 0.0f);
+#pragma unroll
+        for (int q = 0; q <= V / 2; ++q) od[q] = pack2(0.0f, 0.0f);
+        const float4 *c4 = reinterpret_cast<const float4 *>(CB + j0 - kPad);
+#pragma unroll
+        for (int m = 0; m < kQuads; ++m) {
+            const float4 c = c4[m];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const f32x2 x = h ? pack2(c.z, c.w) : pack2(c.x, c.y);
+                const int k = 4 * m + 2 * h - kSh;
+#pragma unroll
+                for (int q = 0; q < V / 2; ++q) {
+                    const int d = k - 2 * q;  // taps of outputs 2q, 2q + 1
+                    if (d >= 0 && d <= 2 * KK) ev[q] = fma2(x, pack2(t.gdup[d].x, t.gdup[d].y), ev[q]);
+                }
+#pragma unroll
+                for (int q = 0; q <= V / 2; ++q) {
+                    const int d = k - 2 * q + 1;  // of outputs 2q - 1, 2q
+                    if (d >= 0 && d <= 2 * KK) od[q] = fma2(x, pack2(t.gdup[d].x, t.gdup[d].y), od[q]);
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < V / 2; q += 2) {
+            const float4 P = *reinterpret_cast<const float4 *>(CP + j0 + 2 * q);
+            float a0, a1, a2, a3, b0, b1, b2, b3, x;
+            unpack2(ev[q], a0, a1);
+            unpack2(ev[q + 1], a2, a3);
+            unpack2(od[q], x, b0);
+            unpack2(od[q + 1], b1, b2);
+            unpack2(od[q + 2], b3, x);
+            const int j = j0 + 2 * q;
+            if (j < n) v = fmaf(P.x, a0 + b0, v);
+            if (j + 1 < n) v = fmaf(P.y, a1 + b1, v);
+            if (j + 2 < n) v = fmaf(P.z, a2 + b2, v);
+            if (j + 3 < n) v = fmaf(P.w, a3 + b3, v);
+        }
     }
     return v;
 }
 
-template <bool FIXED>
-__device__ __forceinline__ float band_conv(const float *CP, const float *CC, const float *gtab, int K, int n)
+template <int KK>
+__device__ __forceinline__ float band_conv_k(const float *CP, const float *CB, const RleTable &t, int n)
 {
-    if (FIXED && K == 15) return band_conv_k<15>(CP, CC, gtab, n);  // Gaussian kernels at sigma = 2 cells
-    if (FIXED && K == 6) return band_conv_k<6>(CP, CC, gtab, n);    // strict band, Delta = 6
-    if (FIXED && K == 4) return band_conv_k<4>(CP, CC, gtab, n);    // box kernel, H = 4
+    // 8 outputs per lane need half the passes of 4 on a longer ray and waste half a pass on a shorter one
+    return n > 128 ? band_conv_v<KK, 8>(CP, CB, t, n) : band_conv_v<KK, 4>(CP, CB, t, n);
+}
+
+__device__ __forceinline__ float band_conv(const float *CP, const float *CB, const float *gtab, const RleTable &t, int K, int n)
+{
+    if (K == 15) return band_conv_k<15>(CP, CB, t, n);  // Gaussian kernels at sigma = 2 cells
+    if (K == 6) return band_conv_k<6>(CP, CB, t, n);    // strict band, Delta = 6
+    if (K == 4) return band_conv_k<4>(CP, CB, t, n);    // box kernel, H = 4
     float v = 0.0f;
     for (int j = lane_id(); j < n; j += 32) {
         float acc = 0.0f;
-        for (int d = -K; d <= K; ++d) acc = fmaf(gtab[K + d], CC[K + j + d], acc);
+        for (int d = -K; d <= K; ++d) acc = fmaf(gtab[K + d], CB[j + d], acc);
         v = fmaf(CP[j], acc, v);
     }
     return v;
@@ -307,17 +395,23 @@ __device__ __forceinline__ float band_conv(const float *CP, const float *CC, con
 // first cell and one past its last). So Theorem 5 is sum_j P(e_j) sum_{k in [lo_j, hi_j)} g(k - j)
 // C_k, taken here with the taps |k - j| <= K of the banded convolution, in increasing k. RI holds
 // each cell's run index, S the run starts (S[nr] = n).
-__device__ __forceinline__ float window_conv(const float *CP, const float *CC, const float *gtab, int K, int n,
+__device__ __forceinline__ void kept_window(const int *S, const int *RI, int n, int D, int j, int &lo, int &hi)
+{
+    const int u = RI[j], a = max(j - D, 0), b = min(j + D, n - 1);
+    lo = max(S[RI[a]], S[u] - D);
+    hi = min(S[u + 1] + D, S[RI[b] + 1]);
+}
+
+__device__ __forceinline__ float window_conv(const float *CP, const float *CB, const float *gtab, int K, int n,
                                              const int *S, const int *RI, int D)
 {
     float v = 0.0f;
     for (int j = lane_id(); j < n; j += 32) {
-        const int u = RI[j];
-        const int a = max(j - D, 0), b = min(j + D, n - 1);
-        const int lo = max(S[RI[a]], S[u] - D), hi = min(S[u + 1] + D, S[RI[b] + 1]);
+        int lo, hi;
+        kept_window(S, RI, n, D, j, lo, hi);
         const int d0 = max(lo - j, -K), d1 = min(hi - j, K + 1);
         float acc = 0.0f;
-        for (int d = d0; d < d1; ++d) acc = fmaf(gtab[K + d], CC[K + j + d], acc);
+        for (int d = d0; d < d1; ++d) acc = fmaf(gtab[K + d], CB[j + d], acc);
         v = fmaf(CP[j], acc, v);
     }
     return v;
@@ -325,9 +419,10 @@ __device__ __forceinline__ float window_conv(const float *CP, const float *CC, c
 
 // window_conv with a compile-time radius KK: the 2 KK + 1 kernel values in registers and every tap
 // predicated on the window, so that no lane waits for another's longer window; the same products
-// added in the same order (bit-identical).
+// added in the same order (bit-identical). (Four cells per lane with 16-byte loads of C and a mask of taps per
+// cell: 161 against 158 us on the 301x253x77 batch.)
 template <int KK>
-__device__ __forceinline__ float window_conv_k(const float *CP, const float *CC, const float *gtab, int n, const int *S,
+__device__ __forceinline__ float window_conv_k(const float *CP, const float *CB, const float *gtab, int n, const int *S,
                                                const int *RI, int D)
 {
     float g[2 * KK + 1];
@@ -335,62 +430,72 @@ __device__ __forceinline__ float window_conv_k(const float *CP, const float *CC,
     for (int d = 0; d <= 2 * KK; ++d) g[d] = gtab[d];
     float v = 0.0f;
     for (int j = lane_id(); j < n; j += 32) {
-        const int u = RI[j];
-        const int a = max(j - D, 0), b = min(j + D, n - 1);
-        const int lo = max(S[RI[a]], S[u] - D), hi = min(S[u + 1] + D, S[RI[b] + 1]);
+        int lo, hi;
+        kept_window(S, RI, n, D, j, lo, hi);
         const int d0 = lo - j + KK, w = hi - lo;  // taps d0 .. d0 + w - 1 of 0 .. 2 KK
         float acc = 0.0f;
 #pragma unroll
         for (int d = 0; d <= 2 * KK; ++d)
-            if ((unsigned)(d - d0) < (unsigned)w) acc = fmaf(g[d], CC[j + d], acc);
+            if ((unsigned)(d - d0) < (unsigned)w) acc = fmaf(g[d], CB[j + d - KK], acc);
         v = fmaf(CP[j], acc, v);
     }
     return v;
 }
 
-// Cell-level evaluation (eq. eqn_from_fsmi) of one ray: decompress the runs into the n virtual
-// cells, form P(e_j) and C_k by warp scans (Algorithms 2 and 3), then
-// I = sum_j P(e_j) sum_{|d| <= K} g(d) C_{j+d} (FSMI-RLE, Uniform-FSMI-RLE, strict-band
-// Approx-FSMI-RLE), or for Theorem 5 the same sum over each first-hit cell's window of kept pairs
-// (window_conv). Arrays: 0 run o, 1 run f_occ (then, for Theorem 5, each cell's run index), 2 run
-// f_emp, 3 P, 4 run starts S, 5 f_emp per cell, 6 C padded by K zeros on both sides.
-static __device__ float ray_mi_cells(float *base, int stride, int nr, int n, const DevParams &p, const float *gtab, int K,
-                                     bool thm5)
+// Cell-level evaluation (eq. eqn_from_fsmi) of one ray given as runs: decompress the runs into the n virtual
+// cells, form P(e_j) and C_k (Algorithms 2 and 3), then I = sum_j P(e_j) sum_{|d| <= K} g(d) C_{j+d}
+// (FSMI-RLE, Uniform-FSMI-RLE, strict-band Approx-FSMI-RLE), or for Theorem 5 the same sum over each
+// first-hit cell's window of kept pairs (window_conv). Each run's index is put at its first cell and
+// spread by a running maximum. Arrays: 0 run o, 3 P, 4 run starts S, 5 the cells' run indices, 6 C.
+static __device__ float ray_mi_cells(float *base, int stride, int nr, int n, const DevParams &p, const float *gtab,
+                                     const RleTable &t, int K, bool thm5)
 {
     const int lane = lane_id();
-    float *O = base, *RFO = base + stride, *RFE = base + 2 * stride, *CP = base + 3 * stride;
+    const float *O = base;
+    float *CP = base + 3 * stride, *CB = base + 6 * stride + conv_pad(K);
     const int *S = (const int *)(base + 4 * stride);
-    float *CF = base + 5 * stride, *CC = base + 6 * stride;
-    for (int u = lane; u < nr; u += 32) {
-        float fo, fe;
-        rle_gains(p, O[u], fo, fe);
-        RFO[u] = fo;
-        RFE[u] = fe;
-    }
-    for (int i = lane; i < K; i += 32) {
-        CC[i] = 0.0f;
-        CC[K + n + i] = 0.0f;
+    int *RI = (int *)(base + 5 * stride);
+    for (int i = 4 * lane; i < n; i += 128) *reinterpret_cast<int4 *>(RI + i) = make_int4(0, 0, 0, 0);
+    __syncwarp();
+    for (int u = lane; u < nr; u += 32) RI[S[u]] = u;  // every run has a cell, so no two share one
+    __syncwarp();
+    CellScan s{1.0f, 0.0f};
+    int last = 0;  // run of the last cell before the block
+    for (int base_i = 0; base_i < n; base_i += 128) {
+        const int i0 = base_i + 4 * lane;
+        int4 u = make_int4(0, 0, 0, 0);
+        if (i0 < n) u = *reinterpret_cast<const int4 *>(RI + i0);
+        u.y = max(u.x, i0 + 1 < n ? u.y : 0);
+        u.z = max(u.y, i0 + 2 < n ? u.z : 0);
+        u.w = max(u.z, i0 + 3 < n ? u.w : 0);
+        int m = u.w;  // running maximum over the lanes
+#pragma unroll
+        for (int k = 1; k < 32; k <<= 1) {
+            const int v = __shfl_up_sync(kFull, m, k);
+            if (lane >= k) m = max(m, v);
+        }
+        int before = __shfl_up_sync(kFull, m, 1);
+        before = lane == 0 ? last : max(before, last);
+        last = max(last, __shfl_sync(kFull, m, 31));
+        u = make_int4(max(u.x, before), max(u.y, before), max(u.z, before), max(u.w, before));
+        float o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (i0 < n) {
+            o[0] = O[u.x];
+            if (i0 + 1 < n) o[1] = O[u.y];
+            if (i0 + 2 < n) o[2] = O[u.z];
+            if (i0 + 3 < n) o[3] = O[u.w];
+            if (thm5) *reinterpret_cast<int4 *>(RI + i0) = u;
+        }
+        scan_block(p, o, i0, n, s, CP, CB);
     }
     __syncwarp();
-    for (int i = lane; i < n; i += 32) {
-        const int u = run_of(S, nr, i);
-        CP[i] = O[u];
-        CC[K + i] = RFO[u];
-        CF[i] = RFE[u];
-    }
-    __syncwarp();
-    cell_prefixes(CP, CC + K, CF, n, false);  // CP = P(e_j), CC[K + k] = C_k, CC[K + n] = 0
-    if (thm5) {
-        int *RI = (int *)RFO;  // the run gains are spread to the cells by now
-        for (int i = lane; i < n; i += 32) RI[i] = run_of(S, nr, i);
-        __syncwarp();
-        return window_conv(CP, CC, gtab, K, n, S, RI, p.trunc);
-    }
-    return band_conv<false>(CP, CC, gtab, K, n);
+    if (thm5) return window_conv(CP, CB, gtab, K, n, S, RI, p.trunc);
+    pad_conv(CB, K, n);
+    return band_conv(CP, CB, gtab, t, K, n);
 }
 
 __device__ __forceinline__ float ray_mi(float *base, int stride, int nr, const DevParams &p, const float2 *tab,
-                                        const float *gtab, int K, bool have_s)
+                                        const float *gtab, const RleTable &t, int K, bool have_s)
 {
     if (nr <= 0) return 0.0f;
     const RunSmem r = run_smem(base, stride);
@@ -399,7 +504,7 @@ __device__ __forceinline__ float ray_mi(float *base, int stride, int nr, const D
     const bool thm5 = p.variant == FSMI_APPROX && p.approx_reading == 0;
     float v;
     if (n < p.cell_runlen * nr) {
-        v = ray_mi_cells(base, stride, nr, n, p, gtab, K, thm5);
+        v = ray_mi_cells(base, stride, nr, n, p, gtab, t, K, thm5);
     } else {
         run_prefixes(r, nr, p);
         if (p.variant == FSMI_APPROX && p.approx_reading == 0)
@@ -412,22 +517,13 @@ __device__ __forceinline__ float ray_mi(float *base, int stride, int nr, const D
 
 // ---- sampling and encoding -------------------------------------------------------------------
 
-// Virtual cells of ray `ray` (= pose * R + r): sample i is the voxel holding
-// o + (i + 1/2) d, i.e. floor of the Q31 position (o << 15) + (2i + 1) d, for i < nsamp until the
-// first sample outside the grid. Runs are maximal spans of bit-identical values split every `cap`
-// cells from the span's start. Writes O[u] = value, S[u] = first cell, S[nr] = n; returns nr.
-//
-// Fused form (CP != nullptr): also writes every virtual cell's o (CP) and, in SP[k], the value of
-// the k-th span of equal values (k counted over the ray; *nspan_out receives their number), from
-// which span_gains fills in the cells' gains; with RI, every cell's run index. Runs past nrcap are
-// counted but not stored; *n_out receives n.
-static __device__ int sample_encode_ray(const float *__restrict__ vox, int X, int Y, int Z, const int32_t *pose,
-                                        const int32_t *u, int nsamp, int cap, float *O, int *S, int nrcap, int *n_out,
-                                        float *CP, float *SP, int *nspan_out, int *RI = nullptr)
+// Virtual cells of a ray: sample i is the voxel holding o + (i + 1/2) d, i.e. floor of the Q31 position
+// (o << 15) + (2i + 1) d, for i < nsamp until the first sample outside the grid. Runs are maximal spans of
+// bit-identical values split every `cap` cells from the span's start.
+
+// Q31 position of sample 0, less d, and the direction (Q30) of a ray
+__device__ __forceinline__ void ray_dir(const int32_t *pose, const int32_t *u, long long (&o)[3], long long (&d)[3])
 {
-    const int lane = lane_id();
-    int nspan = 0;
-    long long d[3], o[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const long long acc = (long long)pose[3 + 3 * a] * u[0] + (long long)pose[4 + 3 * a] * u[1] +
@@ -435,6 +531,15 @@ static __device__ int sample_encode_ray(const float *__restrict__ vox, int X, in
         d[a] = (acc + (1LL << 29)) >> 30;
         o[a] = (long long)pose[a] << 15;
     }
+}
+
+// The encoder's form: writes O[u] = value, S[u] = first cell, S[nr] = n; returns nr.
+static __device__ int sample_encode_ray(const float *__restrict__ vox, int X, int Y, int Z, const int32_t *pose,
+                                        const int32_t *u, int nsamp, int cap, float *O, int *S)
+{
+    const int lane = lane_id();
+    long long d[3], o[3];
+    ray_dir(pose, u, o, d);
     int nrun = 0, carried = 0, n = 0;
     unsigned prev_bits = 0u;
     // Q31 position o + (2i + 1) d of this lane's sample, advanced by 64 d per chunk of 32
@@ -486,16 +591,8 @@ static __device__ int sample_encode_ray(const float *__restrict__ vox, int X, in
         const unsigned mb = __ballot_sync(kFull, brk);
         if (brk) {
             const int k = nrun + __popc(mb & ((1u << lane) - 1u));
-            if (k < nrcap) {
-                O[k] = val;
-                S[k] = i;
-            }
-        }
-        if (RI && valid) RI[i] = nrun + __popc(mb & lane_le) - 1;  // the run this cell belongs to
-        if (CP) {
-            if (valid) CP[i] = val;
-            if (newval) SP[nspan + __popc(nle) - 1] = val;  // span index <= cell index
-            nspan += __popc(mnew);
+            O[k] = val;
+            S[k] = i;
         }
         nrun += __popc(mb);
         n += nvalid;
@@ -503,36 +600,180 @@ static __device__ int sample_encode_ray(const float *__restrict__ vox, int X, in
         carried = __shfl_sync(kFull, st, 31);
         prev_bits = __shfl_sync(kFull, bits, 31);
     }
-    if (lane == 0 && nrun <= nrcap) S[nrun] = n;
-    if (n_out) *n_out = n;
-    if (nspan_out) *nspan_out = nspan;
+    if (lane == 0) S[nrun] = n;
     __syncwarp();
     return nrun;
 }
 
-static __device__ int sample_encode_ray(const float *__restrict__ vox, int X, int Y, int Z, const int32_t *pose,
-                                        const int32_t *u, int nsamp, int cap, float *O, int *S)
+// Runs of a block of 128 cells, four consecutive ones per lane (nw: a new value begins at the cell): O[k], S[k] of
+// the runs below nrcap, and with RI every cell's run index.
+struct RunScan {
+    int nrun, carried;  // runs so far, start of the span that reaches into the block
+};
+__device__ __forceinline__ void encode_block(const float (&o)[4], const bool (&nw)[4], int i0, int n, int cap, float inv_cap,
+                                             RunScan &s, float *O, int *S, int nrcap, int *RI)
 {
-    return sample_encode_ray(vox, X, Y, Z, pose, u, nsamp, cap, O, S, nsamp + 1, nullptr, nullptr, nullptr, nullptr);
+    const int lane = lane_id();
+    // start of each cell's span: the last cell at or before it where a new value begins
+    int st[4], own = -1;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        if (nw[t]) own = i0 + t;
+        st[t] = own;
+    }
+    int m = own;
+#pragma unroll
+    for (int k = 1; k < 32; k <<= 1) {
+        const int w = __shfl_up_sync(kFull, m, k);
+        if (lane >= k) m = max(m, w);
+    }
+    int from = __shfl_up_sync(kFull, m, 1);
+    from = lane == 0 ? s.carried : max(from, s.carried);
+    s.carried = max(s.carried, __shfl_sync(kFull, m, 31));
+    bool brk[4];
+    int cnt = 0;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const int rel = i0 + t - max(st[t], from);  // a multiple of cap starts a run (exact, see sample_encode_ray)
+        brk[t] = i0 + t < n && rel - __float2int_rn((float)rel * inv_cap) * cap == 0;
+        cnt += brk[t];
+    }
+    const int incl = warp_incl_add_int(cnt);
+    int k = s.nrun + incl - cnt, r[4];
+    s.nrun += __shfl_sync(kFull, incl, 31);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        if (brk[t]) {
+            if (k < nrcap) {
+                O[k] = o[t];
+                S[k] = i0 + t;
+            }
+            ++k;
+        }
+        r[t] = k - 1;
+    }
+    if (RI && i0 < n) *reinterpret_cast<int4 *>(RI + i0) = make_int4(r[0], r[1], r[2], r[3]);
+}
+
+// The fused kernel's form: blocks of 128 samples, four consecutive ones per lane, straight through scan_block into
+// P (CP) and C (CB). Returns n. With ENC the runs are formed on the way (O, S, RI; count = their number), else the
+// values go to CO (for encode_cells) and count = the number of spans of equal values.
+//
+// What bounds it is instructions per sample. One sample per lane and chunk of 32 took, per chunk, a ballot and
+// a scan step for each of the range end, the spans, the run splits and the two prefixes, the gains spread
+// from the spans through shared memory, and six array accesses; a block of 128 pays the warp-wide steps
+// once and stores three 16-byte words. 512x512x128 voxels, 64 poses x 128x128 rays: 1,741 to 1,068 warp
+// instructions per ray and 1,690 to 1,136 us, with the convolution below; Theorem 5 on 301x253x77 voxels,
+// 23 x 80x61 rays: 162 to 149 us. The registers (73) leave 28 warps per SM; held to 64: 1,152 - 1,172 us.
+template <bool ENC>
+__device__ __forceinline__ int sample_cells(const float *__restrict__ vox, int X, int Y, int Z, const int32_t *pose,
+                                            const int32_t *u, int nsamp, const DevParams &p, float *CP, float *CB, float *CO,
+                                            float *O, int *S, int nrcap, int *RI, int &count)
+{
+    const int lane = lane_id();
+    long long d[3], q[3];
+    ray_dir(pose, u, q, d);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) q[a] += (8LL * lane + 1) * d[a];  // sample 4 lane
+    CellScan s{1.0f, 0.0f};
+    RunScan rs{0, 0};
+    const float inv_cap = 1.0f / (float)p.run_cap;
+    unsigned prev = 0u;
+    int n = 0, spans = 0;
+    for (int base = 0; base < nsamp; base += 128) {
+        const int i0 = base + 4 * lane;
+        float o[4];
+        bool in[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            // as in sample_encode_ray
+            const unsigned px = (unsigned)(q[0] >> 31), py = (unsigned)(q[1] >> 31), pz = (unsigned)(q[2] >> 31);
+            in[t] = px < (unsigned)X && py < (unsigned)Y && pz < (unsigned)Z && i0 + t < nsamp;
+            o[t] = in[t] ? __ldg(vox + ((size_t)(pz * (unsigned)Y + py) * (unsigned)X + px)) : 0.0f;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) q[a] += (t < 3 ? 2 : 250) * d[a];
+        }
+        // the ray ends at its first sample outside
+        const int c = !in[0] ? 0 : !in[1] ? 1 : !in[2] ? 2 : !in[3] ? 3 : 4;
+        const unsigned m = __ballot_sync(kFull, c == 4);
+        const int L = m == kFull ? 31 : __ffs(~m) - 1;
+        n = base + 4 * L + __shfl_sync(kFull, c, L);
+        const unsigned left = __shfl_up_sync(kFull, __float_as_uint(o[3]), 1);
+        unsigned before = lane == 0 ? prev : left;
+        prev = __shfl_sync(kFull, __float_as_uint(o[3]), 31);
+        bool nw[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const unsigned bits = __float_as_uint(o[t]);
+            const bool valid = i0 + t < n;
+            nw[t] = valid && (bits != before || i0 + t == 0);
+            spans += nw[t];
+            before = bits;
+            if (!valid) o[t] = 0.0f;
+        }
+        if (ENC)
+            encode_block(o, nw, i0, n, p.run_cap, inv_cap, rs, O, S, nrcap, RI);
+        else if (i0 < n)
+            *reinterpret_cast<float4 *>(CO + i0) = make_float4(o[0], o[1], o[2], o[3]);
+        scan_block(p, o, i0, n, s, CP, CB);
+        if (m != kFull) break;
+    }
+    if (ENC) {
+        if (lane == 0 && rs.nrun <= nrcap) S[rs.nrun] = n;
+        count = rs.nrun;
+    } else {
+        count = __reduce_add_sync(kFull, spans);
+    }
+    __syncwarp();
+    return n;
+}
+
+// Run-length encoding of the n cells in CO; returns the number of runs (S[nr] = n if nr <= nrcap).
+static __device__ int encode_cells(const float *CO, int n, int cap, float *O, int *S, int nrcap)
+{
+    const int lane = lane_id();
+    const float inv_cap = 1.0f / (float)cap;
+    RunScan rs{0, 0};
+    unsigned prev = 0u;
+    for (int base = 0; base < n; base += 128) {
+        const int i0 = base + 4 * lane;
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (i0 < n) v = *reinterpret_cast<const float4 *>(CO + i0);
+        const float o[4] = {v.x, v.y, v.z, v.w};
+        const unsigned left = __shfl_up_sync(kFull, __float_as_uint(o[3]), 1);
+        unsigned before = lane == 0 ? prev : left;
+        prev = __shfl_sync(kFull, __float_as_uint(o[3]), 31);
+        bool nw[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const unsigned bits = __float_as_uint(o[t]);
+            nw[t] = i0 + t < n && (bits != before || i0 + t == 0);
+            before = bits;
+        }
+        encode_block(o, nw, i0, n, cap, inv_cap, rs, O, S, nrcap, nullptr);
+    }
+    if (lane == 0 && rs.nrun <= nrcap) S[rs.nrun] = n;
+    __syncwarp();
+    return rs.nrun;
 }
 
 // ---- the fused 3D ray (sampling and evaluation in one warp) --------------------------------------
 //
-// Per-warp layout: per-cell o / P (CP), f_emp (CF) and C padded by K zeros on both sides (CC), each
+// Per-warp layout: per-cell P (CP), o (CO) and C padded by zeros on both sides (CB), each
 // cell_stride floats (absent for Theorem 5's sub-blocks, which always use the runs), then the six
 // run arrays sized for the runs the run-pair path can see: a ray takes that path only when
 // n >= cell_runlen * n_r, so n_r <= nmax / cell_runlen.
 
 __host__ __device__ inline bool thm5_of(const DevParams &p) { return p.variant == FSMI_APPROX && p.approx_reading == 0; }
-__host__ __device__ inline int ray3d_cell_stride(const DevParams &p) { return ((p.nmax + 2 * p.K + 2) + 3) & ~3; }
+__host__ __device__ inline int ray3d_cell_stride(const DevParams &p) { return (p.nmax + conv_pad(p.K) + p.K + 12 + 3) & ~3; }
 __host__ __device__ inline int ray3d_nrcap(const DevParams &p)
 {
     const int T = p.cell_runlen > 0 ? p.cell_runlen : 1;
     return thm5_of(p) ? p.nmax : min(p.nmax, p.nmax / T + 2);
 }
 __host__ __device__ inline int ray3d_run_stride(const DevParams &p) { return ((ray3d_nrcap(p) + 2) + 3) & ~3; }
-// Per-warp floats of the fused 3D path. The others: [CP | CF | CC | six run arrays]. Theorem 5 (all
-// runs stored): [S | O | four cell-stride arrays], the four holding CP, CF, CC and the cells' run
+// Per-warp floats of the fused 3D path. The others: [CP | CO | CB | six run arrays]. Theorem 5 (all
+// runs stored): [S | O | four cell-stride arrays], the four holding CP, CO, CB and the cells' run
 // indices for the cell form, or the run arrays X, A, F, L for the run pairs.
 __host__ __device__ inline int ray3d_warp_floats(const DevParams &p)
 {
@@ -544,98 +785,64 @@ __host__ __device__ inline int ray3d_warp_floats(const DevParams &p)
 // Theorem 5's sub-blocks only, or the others (cell-level convolution and all run pairs) only.
 enum { kRay3dAny = 0, kRay3dThm5 = 1, kRay3dOther = 2 };
 
-// The cells' gains f(delta_occ, o) (Gk) and f(delta_emp, o) (Gf) of a sampled ray: the nspan spans
-// of equal values (their values in Gf[0 .. nspan), from sampling) get both gains once, stored in
-// place at Gk[k] and Gf[k]; then every cell takes its span's pair, the chunks of 32 cells from the
-// last down, each reading before any lane writes: cell i's span index is at most i, so a chunk
-// only overwrites entries that no cell below it reads. A cell starts a span where its value's bits
-// differ from the previous cell's, as in the sampling.
-__device__ __forceinline__ void span_gains(const DevParams &p, const float *CP, float *Gk, float *Gf, int n, int nspan)
-{
-    const int lane = lane_id();
-    for (int k = lane; k < nspan; k += 32) {
-        float fo, fe;
-        rle_gains(p, Gf[k], fo, fe);
-        Gk[k] = fo;
-        Gf[k] = fe;
-    }
-    __syncwarp();
-    const unsigned lane_le = 0xffffffffu >> (31 - lane);
-    int above = nspan;  // spans that start in the chunks above the current one, counted from the end
-    for (int base = ((n - 1) >> 5) << 5; base >= 0; base -= 32) {
-        const int i = base + lane;
-        const bool in = i < n;
-        const bool start = in && (i == 0 || __float_as_uint(CP[i]) != __float_as_uint(CP[i - 1]));
-        const unsigned m = __ballot_sync(kFull, start);
-        above -= __popc(m);  // now: spans that start before this chunk
-        const int k = above + __popc(m & lane_le) - 1;
-        float go = 0.0f, ge = 0.0f;
-        if (in) {
-            go = Gk[k];
-            ge = Gf[k];
-        }
-        __syncwarp();
-        if (in) {
-            Gk[i] = go;
-            Gf[i] = ge;
-        }
-        __syncwarp();
-    }
-}
-
-// Samples, encodes and evaluates one ray into the warp's region `w` (ray3d_warp_floats floats);
-// returns the MI (warp-reduced) and the run count in *nr_out. MODE must agree with thm5_of(p).
+// Samples and evaluates one ray in the warp's region `w` (ray3d_warp_floats floats); returns the MI
+// (warp-reduced) and, with nr_out, the run count. MODE must agree with thm5_of(p). Outside Theorem 5 the runs are
+// formed (from the sampled values in shared memory) only where they are needed: for a caller who asks for
+// their number, or on a ray whose spans of equal values do not already show that its mean run is short.
 template <int MODE>
 __device__ __forceinline__ float ray_mi_fused(const float *vox, int X, int Y, int Z, const int32_t *pose,
                                               const int32_t *u, int nsamp, const DevParams &p, const float2 *tab,
-                                              const float *gtab, int K, float *w, int *nr_out)
+                                              const float *gtab, const RleTable &t, int K, float *w, int *nr_out)
 {
-    const int lane = lane_id();
     const bool thm5 = MODE == kRay3dAny ? thm5_of(p) : MODE == kRay3dThm5;
     const int cst = ray3d_cell_stride(p), rst = ray3d_run_stride(p);
-    float *CP, *CF, *CC;
+    float *CP, *CO, *CB;
     int *RI = nullptr;
     RunSmem r;
     if (thm5) {
         float *c4 = w + 2 * rst;
         CP = c4;
-        CF = c4 + cst;
-        CC = c4 + 2 * cst;
+        CO = c4 + cst;
+        CB = c4 + 2 * cst + conv_pad(K);
         RI = (int *)(c4 + 3 * cst);
         r.S = (int *)w;
         r.O = w + rst;
         r.X = CP;
-        r.A = CF;
-        r.F = CC;
+        r.A = CO;
+        r.F = c4 + 2 * cst;
         r.L = RI;
     } else {
         CP = w;
-        CF = w + cst;
-        CC = w + 2 * cst;
+        CO = w + cst;
+        CB = w + 2 * cst + conv_pad(K);
         r = run_smem(w + 3 * cst, rst);
     }
-    int n = 0, nspan = 0;
-    const int nr = sample_encode_ray(vox, X, Y, Z, pose, u, nsamp, p.run_cap, r.O, r.S, ray3d_nrcap(p), &n, CP, CF,
-                                     &nspan, RI);
-    *nr_out = nr;
-    if (nr <= 0) return 0.0f;
-    float v;
-    if (n < p.cell_runlen * nr) {
-        // eq. eqn_from_fsmi on the virtual cells: Algorithms 2 and 3, then the banded convolution
-        // (Theorem 5: over each first-hit cell's window of kept pairs)
-        if (!thm5) {
-            for (int i = lane; i < K; i += 32) {
-                CC[i] = 0.0f;
-                CC[K + n + i] = 0.0f;
-            }
+    int n, nr = 0;
+    bool cells;
+    if (thm5) {
+        n = sample_cells<true>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, r.O, r.S, ray3d_nrcap(p), RI, nr);
+        cells = n < p.cell_runlen * nr;
+    } else {
+        int nspan;
+        n = sample_cells<false>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, nullptr, nullptr, 0, nullptr, nspan);
+        cells = n < p.cell_runlen * nspan;  // at least one run per span
+        if (n > 0 && (nr_out || !cells)) {
+            nr = encode_cells(CO, n, p.run_cap, r.O, r.S, ray3d_nrcap(p));
+            cells = n < p.cell_runlen * nr;
         }
-        span_gains(p, CP, CC + K, CF, n, nspan);
-        cell_prefixes(CP, CC + K, CF, n, false);  // CP = P(e_j), CC[K + k] = C_k, CC[K + n] = 0
-        if (thm5) {  // RI was filled while sampling
-            v = MODE == kRay3dThm5 && K == 15 ? window_conv_k<15>(CP, CC, gtab, n, r.S, RI, p.trunc)
-                                               : window_conv(CP, CC, gtab, K, n, r.S, RI, p.trunc);
+    }
+    if (nr_out) *nr_out = nr;
+    if (n == 0) return 0.0f;
+    float v;
+    if (cells) {
+        // eq. eqn_from_fsmi on the virtual cells: the banded convolution (Theorem 5: over each first-hit
+        // cell's window of kept pairs)
+        if (thm5) {
+            v = MODE == kRay3dThm5 && K == 15 ? window_conv_k<15>(CP, CB, gtab, n, r.S, RI, p.trunc)
+                                               : window_conv(CP, CB, gtab, K, n, r.S, RI, p.trunc);
         } else {
-            v = band_conv<MODE == kRay3dOther>(CP, CC, gtab, K, n);
+            pad_conv(CB, K, n);
+            v = band_conv(CP, CB, gtab, t, K, n);
         }
     } else {  // here n_r <= nrcap, so every run was stored
         run_starts(r, nr, true);
@@ -719,7 +926,7 @@ __device__ __forceinline__ RleBlock rle_block(unsigned char *smem_raw, const Dev
 // sampling, encoding and evaluation of one 3D ray (= pose * R + r), fused layout; WIDE: the batch
 // has more than 2^31 - 1 rays (64-bit index division), else a 32-bit one
 template <int MODE, bool WIDE>
-__device__ __forceinline__ void eval_ray_3d(const Vox3D &vx, const DevParams &p, const RleBlock &rb,
+__device__ __forceinline__ void eval_ray_3d(const Vox3D &vx, const DevParams &p, const RleBlock &rb, const RleTable &t,
                                             long long ray, float *__restrict__ out, int32_t *__restrict__ nruns)
 {
     int pi, ri;
@@ -732,7 +939,7 @@ __device__ __forceinline__ void eval_ray_3d(const Vox3D &vx, const DevParams &p,
     }
     int nr = 0;
     const float I = ray_mi_fused<MODE>(vx.vox, vx.X, vx.Y, vx.Z, vx.poses + 12 * (size_t)pi, vx.dirs + 3 * (size_t)ri, p.nmax,
-                                 p, rb.tab, rb.gtab, rb.ts.K, rb.base, &nr);
+                                 p, rb.tab, rb.gtab, t, rb.ts.K, rb.base, nruns ? &nr : nullptr);
     if (lane_id() == 0) {
         out[ray] = I;
         if (nruns) nruns[ray] = nr;
@@ -743,7 +950,7 @@ __device__ __forceinline__ void eval_ray_3d(const Vox3D &vx, const DevParams &p,
 // evaluation of one run-length-encoded ray given in CSR form
 __device__ __forceinline__ void eval_ray_rle(const int32_t *__restrict__ off, const float *__restrict__ ro,
                                              const uint8_t *__restrict__ rl, const DevParams &p, const RleBlock &rb,
-                                             int stride, long long ray, float *__restrict__ out, int *status)
+                                             const RleTable &t, int stride, long long ray, float *__restrict__ out, int *status)
 {
     const int lane = lane_id();
     const RunSmem r = run_smem(rb.base, stride);
@@ -771,7 +978,7 @@ __device__ __forceinline__ void eval_ray_rle(const int32_t *__restrict__ off, co
         __syncwarp();
         return;
     }
-    const float I = ray_mi(rb.base, stride, nr, p, rb.tab, rb.gtab, rb.ts.K, false);
+    const float I = ray_mi(rb.base, stride, nr, p, rb.tab, rb.gtab, t, rb.ts.K, false);
     if (lane == 0) out[ray] = I;
     __syncwarp();
 }

@@ -65,7 +65,7 @@ int gauss_radius(float sigma) { return (int)ceilf(7.45f * sigma); }
 
 enum Use { kUse2D, kUseBeams, kUseRLE };
 
-// ---- the per-cell gain as a Chebyshev series (RLE kernels) --------------------------------------
+// ---- the per-cell gain as a polynomial (RLE kernels) ---------------------------------------------
 
 static double gain_exact(double d, double o)
 {
@@ -73,75 +73,84 @@ static double gain_exact(double d, double o)
     return post * log1p((d - 1.0) * omo * ria) - omo * ria * log1p(a);
 }
 
-// gain_series of fsmi_device.cuh, operation for operation in FP32 (explicit fmaf, nothing left to
+// rle_gains of evalrle.cuh for one delta, operation for operation in FP32 (explicit fmaf, nothing left to
 // contraction), so that the host sees exactly what the kernels compute
-static float gain_series_host(const float *c, float o)
+static float gain_poly_host(const float (*c)[2], int w, int terms, float o)
 {
-    const float x2 = fmaf(4.0f, o, -2.0f);
-    float b1 = 0.0f, b2 = 0.0f;
-    for (int k = kGainFitTerms - 1; k >= 1; --k) {
-        const float t = c[k] - b2;
-        const float b0 = fmaf(x2, b1, t);
-        b2 = b1;
-        b1 = b0;
-    }
-    const float hx = 0.5f * x2;
-    const float t0 = c[0] - b2;
-    const float h = fmaf(hx, b1, t0);
+    const float x = fmaf(2.0f, o, -1.0f);
+    float h = c[terms - 1][w];
+    for (int k = terms - 2; k >= 0; --k) h = fmaf(h, x, c[k][w]);
     const float om = 1.0f - o;
-    const float w = o * om;
-    return w * h;
+    const float ww = o * om;
+    return ww * h;
 }
 
-// Fits h(o) = f(delta, o) / (o (1 - o)) for both deltas at Chebyshev nodes and keeps the series
-// only if, evaluated as the kernels do, it is within 1e-6 of f (relative) everywhere on a dense
-// grid of [0, 1] that includes points down to 1e-7 from either end; otherwise the kernels use the
-// closed form. The last fit is remembered per host thread.
-static void fit_gains(DevParams &d)
+// Interpolates h(o) = f(delta, o) / (o (1 - o)) (smooth on [0, 1]: f vanishes linearly at both ends) for both
+// deltas at `terms` Chebyshev nodes and writes the interpolant in powers of x = 2 o - 1. The nearest
+// singularity of h lies at o = -1 / (delta - 1), so for deltas near 1 the powers' coefficients fall
+// geometrically and Horner's rule rounds no worse than Clenshaw's, in half the operations. Returns
+// whether the polynomial, evaluated as the kernels do, is within `tol` of f (relative) everywhere on a
+// dense grid of [0, 1] that includes points down to 1e-7 from either end.
+static bool fit_gain(DevParams &d, int terms, double tol)
 {
-    thread_local float last_docc = -1.0f, last_demp = -1.0f, last_c[2][kGainFitTerms];
-    thread_local int last_ok = 0;
-    if (d.docc == last_docc && d.demp == last_demp) {
-        d.gain_fit = last_ok;
-        memcpy(d.gfit, last_c, sizeof(last_c));
-        for (int k = 0; k < kGainFitTerms; ++k) {
-            d.gfit2[k][0] = d.gfit[0][k];
-            d.gfit2[k][1] = d.gfit[1][k];
-        }
-        return;
-    }
-    const int N = kGainFitTerms;
     const double pi = 3.14159265358979323846;
-    bool ok = true;
+    memset(d.gfit2, 0, sizeof(d.gfit2));
     for (int w = 0; w < 2; ++w) {
         const double delta = w ? d.demp : d.docc;
-        double h[kGainFitTerms];
-        for (int j = 0; j < N; ++j) {
-            const double oj = 0.5 * (cos(pi * (j + 0.5) / N) + 1.0);
+        double h[kGainFitTerms], pw[kGainFitTerms] = {}, t0[kGainFitTerms] = {}, t1[kGainFitTerms] = {};
+        for (int j = 0; j < terms; ++j) {
+            const double oj = 0.5 * (cos(pi * (j + 0.5) / terms) + 1.0);
             h[j] = gain_exact(delta, oj) / (oj * (1.0 - oj));
         }
-        for (int k = 0; k < N; ++k) {
+        t0[0] = 1.0;  // T_0 and T_1 in powers of x, then T_{k+1} = 2 x T_k - T_{k-1}
+        t1[1] = 1.0;
+        for (int k = 0; k < terms; ++k) {
             double c = 0.0;
-            for (int j = 0; j < N; ++j) c += h[j] * cos(pi * k * (j + 0.5) / N);
-            d.gfit[w][k] = (float)(c * (k == 0 ? 1.0 : 2.0) / N);
+            for (int j = 0; j < terms; ++j) c += h[j] * cos(pi * k * (j + 0.5) / terms);
+            c *= (k == 0 ? 1.0 : 2.0) / terms;
+            const double *t = k == 0 ? t0 : t1;
+            for (int m = 0; m <= k; ++m) pw[m] += c * t[m];
+            if (k >= 1) {
+                double t2[kGainFitTerms] = {};
+                for (int m = 0; m + 1 < kGainFitTerms; ++m) t2[m + 1] = 2.0 * t1[m];
+                for (int m = 0; m < kGainFitTerms; ++m) {
+                    t2[m] -= t0[m];
+                    t0[m] = t1[m];
+                    t1[m] = t2[m];
+                }
+            }
         }
+        for (int k = 0; k < terms; ++k) d.gfit2[k][w] = (float)pw[k];
         auto check = [&](float o) {
             const double e = gain_exact(delta, (double)o);
-            const double g = (double)gain_series_host(d.gfit[w], o);
-            return e == 0.0 ? g == 0.0 : fabs(g - e) <= 1e-6 * fabs(e);
+            const double g = (double)gain_poly_host(d.gfit2, w, terms, o);
+            return e == 0.0 ? g == 0.0 : fabs(g - e) <= tol * fabs(e);
         };
-        for (int i = 0; i <= 8192 && ok; ++i) ok = check((float)i / 8192.0f);
-        for (double t = 1e-7; t < 1e-2 && ok; t *= 1.25) ok = check((float)t) && check((float)(1.0 - t));
+        for (int i = 0; i <= 8192; ++i)
+            if (!check((float)i / 8192.0f)) return false;
+        for (double t = 1e-7; t < 1e-2; t *= 1.25)
+            if (!check((float)t) || !check((float)(1.0 - t))) return false;
     }
-    d.gain_fit = ok ? 1 : 0;
-    for (int k = 0; k < N; ++k) {
-        d.gfit2[k][0] = d.gfit[0][k];
-        d.gfit2[k][1] = d.gfit[1][k];
+    return true;
+}
+
+// The short polynomial where FP32 rounding dominates its error (2e-7: delta 1.5 and 0.67 reach 1.6e-7 with
+// 8 and with 14 terms), else the long one within 1e-6, else the closed form. The last fit is remembered per
+// host thread.
+static void fit_gains(DevParams &d)
+{
+    thread_local float last_docc = -1.0f, last_demp = -1.0f, last_c[kGainFitTerms][2];
+    thread_local int last_fit = 0;
+    if (d.docc == last_docc && d.demp == last_demp) {
+        d.gain_fit = last_fit;
+        memcpy(d.gfit2, last_c, sizeof(last_c));
+        return;
     }
+    d.gain_fit = fit_gain(d, kGainShortTerms, 2e-7) ? 2 : fit_gain(d, kGainFitTerms, 1e-6) ? 1 : 0;
     last_docc = d.docc;
     last_demp = d.demp;
-    last_ok = d.gain_fit;
-    memcpy(last_c, d.gfit, sizeof(last_c));
+    last_fit = d.gain_fit;
+    memcpy(last_c, d.gfit2, sizeof(last_c));
 }
 
 fsmi_status make_params(const fsmi_params *prm, Use use, DevParams &d)
@@ -176,7 +185,6 @@ fsmi_status make_params(const fsmi_params *prm, Use use, DevParams &d)
     d.rend = 0.0f;
     d.K = 0;
     d.gain_fit = 0;
-    memset(d.gfit, 0, sizeof(d.gfit));
     memset(d.gfit2, 0, sizeof(d.gfit2));
     if (use == kUse2D) {
         if (prm->max_range > FSMI_MAX_RANGE_2D) return FSMI_ERR_CAPACITY;

@@ -72,25 +72,6 @@ __device__ __forceinline__ float cell_gain(float delta, float o)
     return __fsub_rn(__fmul_rn(post, l1), __fmul_rn(__fmul_rn(omo, ria), log1pf(a)));
 }
 
-// The same gain from a Chebyshev series: f(delta, o) = o (1 - o) h(o), where h is smooth on
-// [0, 1] (f vanishes linearly at o = 0 and o = 1), evaluated by Clenshaw's recurrence in
-// x = 2 o - 1. The host fits the series per call and keeps it only if, evaluated exactly as here,
-// it stays within 1e-6 of f relative over [0, 1] (delta not too far from 1); about a third of the
-// instructions of the two logarithms and the division of cell_gain.
-__device__ __forceinline__ float gain_series(const float *c, float o)
-{
-    const float x2 = __fmaf_rn(4.0f, o, -2.0f);  // 2x
-    float b1 = 0.0f, b2 = 0.0f;
-#pragma unroll
-    for (int k = kGainFitTerms - 1; k >= 1; --k) {
-        const float b0 = __fmaf_rn(x2, b1, __fsub_rn(c[k], b2));
-        b2 = b1;
-        b1 = b0;
-    }
-    const float h = __fmaf_rn(__fmul_rn(0.5f, x2), b1, __fsub_rn(c[0], b2));
-    return __fmul_rn(__fmul_rn(o, __fsub_rn(1.0f, o)), h);
-}
-
 // Upper Gaussian tail in the erfc variable: 0.5 * erfc(z) = 1 - Phi(z sqrt(2)), z >= 0.
 __device__ __forceinline__ float half_erfc(float z) { return 0.5f * erfcf(z); }
 
@@ -106,60 +87,15 @@ __device__ __forceinline__ float ipowf(float x, int k)
     return r;
 }
 
-// Chunked warp scan over the n cells held in shared memory. On entry sp = o, sc = f_occ,
-// sx = f_emp. On exit sp = P(e_j), sc = C_j (sc[n] = 0), and for the uniform variant sx = D_j.
-// Returns P(e_0).
-__device__ __forceinline__ float cell_prefixes(float *sp, float *sc, float *sx, int n, bool want_d)
-{
-    const int lane = lane_id();
-    const int K = ((n + 31) >> 5) | 1;  // odd block length: the lanes' blocks start in distinct banks
-    const int lo = min(n, lane * K), hi = min(n, lo + K);
-    float prod = 1.0f, sum = 0.0f;
-    for (int i = lo; i < hi; ++i) {
-        prod *= 1.0f - sp[i];
-        sum += sx[i];
-    }
-    const float iprod = warp_incl_mul(prod);
-    const float isum = warp_incl_add(sum);
-    float E = __shfl_up_sync(kFull, iprod, 1);
-    float q = __shfl_up_sync(kFull, isum, 1);
-    if (lane == 0) {
-        E = 1.0f;
-        q = 0.0f;
-    }
-    const float pe0 = __shfl_sync(kFull, iprod, 31);
-    float csum = 0.0f;
-    for (int i = lo; i < hi; ++i) {
-        const float o = sp[i];
-        sp[i] = E * o;  // Algorithm 2
-        E *= 1.0f - o;
-        const float c = q + sc[i];  // Algorithm 3
-        sc[i] = c;
-        q += sx[i];
-        csum += c;
-    }
-    if (want_d) {  // Algorithm 4: D_k = sum_{i<=k} C_i
-        const float ic = warp_incl_add(csum);
-        float Dacc = __shfl_up_sync(kFull, ic, 1);
-        if (lane == 0) Dacc = 0.0f;
-        for (int i = lo; i < hi; ++i) {
-            Dacc += sc[i];
-            sx[i] = Dacc;
-        }
-    }
-    if (lane == 0) sc[n] = 0.0f;
-    __syncwarp();
-    return pe0;
-}
-
-// The same scan on 16-byte aligned arrays with room for n + 4 entries (the 2D kernels): the entries
-// after the last cell are left undefined (sc[n] apart).
+// Warp scan over the n cells held in shared memory (16-byte aligned arrays with room for n + 4). On entry
+// sp = o, sc = f_occ, sx = f_emp. On exit sp = P(e_j), sc = C_j (sc[n] = 0), and for the uniform variant
+// sx = D_j; the entries after the last cell are left undefined (sc[n] apart). Returns P(e_0).
 //
 // A lane takes 4 V consecutive cells as V 16-byte loads per array (V = ceil(n / 128)): a quarter of the
 // shared-memory instructions of one-float accesses for the same wavefronts (with V = 2 the lanes' loads
 // meet two to a bank; 8-byte accesses in odd blocks avoid that and were slower: Uniform-FSMI on the
-// 2048x2048 office batch 688 against 665 us). The virtual cells of the 3D rays are too few to gain.
-__device__ __forceinline__ float cell_prefixes4(float *sp, float *sc, float *sx, int n, bool want_d)
+// 2048x2048 office batch 688 against 665 us).
+__device__ __forceinline__ float cell_prefixes(float *sp, float *sc, float *sx, int n, bool want_d)
 {
     const int lane = lane_id();
     if (lane < 4) {  // the tail of the last group: o = 0, f_emp = 0 change no prefix

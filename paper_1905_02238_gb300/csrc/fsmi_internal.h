@@ -9,7 +9,8 @@
 namespace fsmi {
 
 // Host-validated parameters plus the derived constants every kernel needs.
-constexpr int kGainFitTerms = 14;  // terms of the Chebyshev series of the per-cell gain (degree 13)
+constexpr int kGainFitTerms = 14;   // coefficients of the per-cell gain's polynomial (degree 13)
+constexpr int kGainShortTerms = 8;  // the same where delta_occ and delta_emp are near enough to 1
 
 struct DevParams {
     int variant;        // FSMI_EXACT / FSMI_APPROX / FSMI_UNIFORM
@@ -30,19 +31,21 @@ struct DevParams {
     int K;              // RLE kernel support radius (cells)
     int flags;          // FSMI_FLAG_* bits
     int cell_runlen;    // RLE: rays whose mean run length is below this take the cell-level form
-    // Chebyshev series of h(o) = f(delta, o) / (o (1 - o)) on [0, 1] for delta_occ ([0]) and
-    // delta_emp ([1]), used by the RLE kernels when gain_fit is set (see gain_series)
+    // h(o) = f(delta, o) / (o (1 - o)) on [0, 1] as a polynomial in x = 2 o - 1, coefficient of x^k for
+    // (delta_occ, delta_emp), used by the RLE kernels (rle_gains): gain_fit 0 = closed form, 1 =
+    // kGainFitTerms coefficients, 2 = kGainShortTerms
     int gain_fit;
-    float gfit[2][kGainFitTerms];
-    float gfit2[kGainFitTerms][2];  // the same coefficients interleaved (delta_occ, delta_emp) per term
+    float gfit2[kGainFitTerms][2];
 };
 
 // Noise-kernel tables of the RLE kernels for radius K = table_spec(p).K (fill_rle_table, on the
 // host in double, once per launch): tab[d + K + 1] = (sum_{e <= d} g(e), sum_{e <= d} e g(e))
 // for d = -K-1..K (tab[0] = 0, the second sum 0 at d = K), gtab[K + d] = g(d), d = -K..K.
+constexpr int kConvMaxRadius = 15;  // largest compiled-in radius of the banded convolution
 struct RleTable {
     float2 tab[2 * FSMI_MAX_KERNEL_RADIUS + 2];
     float gtab[2 * FSMI_MAX_KERNEL_RADIUS + 1];
+    float2 gdup[2 * kConvMaxRadius + 1];  // (g(d), g(d)) at [K + d] for the radii the convolution compiles in
 };
 void fill_rle_table(const DevParams &p, RleTable &t);
 

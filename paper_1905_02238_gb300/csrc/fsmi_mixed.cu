@@ -314,10 +314,9 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4)
                     bad = FSMI_STATUS_BEAM_OVERFLOW;
                 }
             } else {
-                int nr = 0;
                 constexpr int kMode = KIND == kMix3DThm5 ? kRay3dThm5 : kRay3dOther;
                 I = ray_mi_fused<kMode>(cc->vox, cc->X, cc->Y, cc->Z, cc->pose + 12 * kp, cc->dir + 3 * kd, cc->nsamp, p3,
-                                        rb.tab, rb.gtab, rb.ts.K, base, &nr);
+                                        rb.tab, rb.gtab, tbl, rb.ts.K, base, nullptr);
             }
             __syncwarp();
             if (lane == 0) {
@@ -360,9 +359,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4)
         } else if (ok && st.kind == FSMI_SET_3D && src.has3d && pi < src.P3 && di < src.R3 && st.volume >= 0 &&
                    st.volume < src.nvol && st.max_range >= 1.0f && st.max_range <= (float)p3.nmax) {
             const fsmi_volume v = src.vols[st.volume];
-            int nr = 0;
             I = ray_mi_fused<kRay3dAny>(v.vox, v.X, v.Y, v.Z, src.poses3 + 12 * pi, src.dirs3 + 3 * di, (int)st.max_range,
-                                        p3, rb.tab, rb.gtab, rb.ts.K, base, &nr);
+                                        p3, rb.tab, rb.gtab, tbl, rb.ts.K, base, nullptr);
         } else {
             bad = FSMI_STATUS_BAD_BEAM;  // a malformed descriptor is never used to index
         }

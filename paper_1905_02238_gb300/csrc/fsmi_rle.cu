@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const RleBlock rb = rle_block(smem_raw, p, tbl, warp_floats);
-    for_each_item(nrays, queue, chunk, [&](long long ray) { eval_ray_3d<MODE, WIDE>(vx, p, rb, ray, out, nruns); });
+    for_each_item(nrays, queue, chunk, [&](long long ray) { eval_ray_3d<MODE, WIDE>(vx, p, rb, tbl, ray, out, nruns); });
 }
 
 __global__ void __launch_bounds__(kMaxWarps * 32)
@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const RleBlock rb = rle_block(smem_raw, p, tbl, kArraysRLE * stride);
     for_each_item(nrays, queue, chunk,
-                  [&](long long ray) { eval_ray_rle(off, ro, rl, p, rb, stride, ray, out, status); });
+                  [&](long long ray) { eval_ray_rle(off, ro, rl, p, rb, tbl, stride, ray, out, status); });
 }
 
 __global__ void __launch_bounds__(kWarpsRLE * 32)
@@ -174,7 +174,7 @@ __global__ void k_scan_add(int32_t *a, long long n, const int32_t *tot)
 
 // ---- launchers ---------------------------------------------------------------------------------
 
-static int rle_stride(int nmax, int K) { return ((nmax + 2 * K + 4) + 3) & ~3; }  // cells + 2K padding
+static int rle_stride(int nmax, int K) { return (nmax + conv_pad(K) + K + 12 + 3) & ~3; }  // cells and C's padding
 
 // The noise-kernel tables of one launch (RleTable), from g(d) = (1/(sqrt(2 pi) sigma))
 // exp(-d^2 / (2 sigma^2)) (Theorem 3's density), the cell mass Phi((d + 1/2)/sigma) -
@@ -197,6 +197,7 @@ void fill_rle_table(const DevParams &p, RleTable &t)
         g[a] = v;
         t.gtab[K + a] = (float)v;
         t.gtab[K - a] = (float)v;
+        if (K <= kConvMaxRadius) t.gdup[K + a] = t.gdup[K - a] = make_float2((float)v, (float)v);
     }
     double c0 = 0.0, c1 = 0.0;
     t.tab[0] = make_float2(0.0f, 0.0f);
