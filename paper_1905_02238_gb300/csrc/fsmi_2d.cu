@@ -67,23 +67,16 @@ static cudaError_t launch_variant(const Src2D &src, const DevParams &p, long lon
     const int wpb = fit_warps(sc.warps_per_block, per_warp, 0);
     const size_t smem = (size_t)wpb * per_warp;
     auto kern = k_eval_2d<VAR, SRC>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    WarpGrid g;
+    cudaError_t e = warp_grid((const void *)kern, nbeams, wpb, smem, sc.blocks_per_sm, g);
     if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, wpb * 32, smem);
-    if (e != cudaSuccess) return e;
-    if (occ < 1) return cudaErrorInvalidConfiguration;
-    if (sc.blocks_per_sm > 0 && sc.blocks_per_sm < occ) occ = sc.blocks_per_sm;
-    long long want = (nbeams + wpb - 1) / wpb;
-    long long grid = (long long)sm_count() * occ;
-    if (grid > want) grid = want;
-    if (grid < 1) grid = 1;
+    if (g.one_each) queue = nullptr;  // nothing to balance: no counter to clear (one launch less)
     if (queue) {
         e = cudaMemsetAsync(queue, 0, sizeof(unsigned long long), s);
         if (e != cudaSuccess) return e;
     }
-    kern<<<(unsigned)grid, wpb * 32, smem, s>>>(src, p, nbeams, stride, out, status, queue,
-                                                 sc.queue_chunk > 0 ? sc.queue_chunk : 1);
+    kern<<<g.grid, wpb * 32, smem, s>>>(src, p, nbeams, stride, out, status, queue,
+                                         sc.queue_chunk > 0 ? sc.queue_chunk : 1);
     return cudaGetLastError();
 }
 

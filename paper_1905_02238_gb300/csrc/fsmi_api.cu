@@ -279,6 +279,47 @@ int sm_count()
     return g_sms[dev];
 }
 
+cudaError_t resident_blocks(const void *kern, int threads, size_t smem, int &blocks)
+{
+    struct Entry {
+        const void *kern;
+        int dev, threads, blocks;
+        size_t smem;
+    };
+    constexpr int kEntries = 128;
+    thread_local Entry table[kEntries];  // direct-mapped; a pure function of its key
+    const int dev = current_device();
+    Entry &t = table[((uintptr_t)kern / 16 + smem / 16 + (size_t)threads) % kEntries];
+    if (t.kern == kern && t.dev == dev && t.threads == threads && t.smem == smem) {
+        blocks = t.blocks;
+        return cudaSuccess;
+    }
+    int optin = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kern);
+    // every caller sets the same limit, so that no thread lowers it under another's launch
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, threads, smem);
+    if (e != cudaSuccess) return e;
+    if (blocks < 1) return cudaErrorInvalidConfiguration;
+    t = Entry{kern, dev, threads, blocks, smem};
+    return cudaSuccess;
+}
+
+cudaError_t warp_grid(const void *kern, long long n, int wpb, size_t smem, int max_blocks_per_sm, WarpGrid &g)
+{
+    int occ = 0;
+    cudaError_t e = resident_blocks(kern, wpb * 32, smem, occ);
+    if (e != cudaSuccess) return e;
+    if (max_blocks_per_sm > 0 && max_blocks_per_sm < occ) occ = max_blocks_per_sm;
+    const long long want = (n + wpb - 1) / wpb, fit = (long long)sm_count() * occ;
+    g.one_each = want <= fit;
+    g.grid = (unsigned)(want < 1 ? 1 : want < fit ? want : fit);
+    return cudaSuccess;
+}
+
 int fit_warps(int warps, size_t per_warp, size_t fixed)
 {
     const int dev = current_device();

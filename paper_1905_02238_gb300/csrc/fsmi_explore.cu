@@ -263,7 +263,8 @@ cudaError_t launch_traj_stamps(int W, int H, const int32_t *poses, int P, const 
     if (nbeams == 0) return cudaSuccess;
     const int stride = ((cap + 2) + 3) & ~3;
     const size_t smem = (size_t)kWarpsExplore * 2 * stride * sizeof(float);
-    e = cudaFuncSetAttribute(k_traj_stamps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int occ = 0;
+    e = resident_blocks((const void *)k_traj_stamps, kWarpsExplore * 32, smem, occ);
     if (e != cudaSuccess) return e;
     k_traj_stamps<<<explore_grid(nbeams, kWarpsExplore), kWarpsExplore * 32, smem, s>>>(
         W, H, poses, P, traj_off, T, dirs, B, rfix, rend, cap, stride, stamp, status);
@@ -302,7 +303,8 @@ cudaError_t launch_update_map_2d(float *map, int W, int H, const int32_t *poses,
     if (nbeams == 0) return cudaSuccess;
     const int stride = ((cap + 2) + 3) & ~3;
     const size_t smem = (size_t)kWarpsExplore * 2 * stride * sizeof(float);
-    e = cudaFuncSetAttribute(k_update_counts, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int occ = 0;
+    e = resident_blocks((const void *)k_update_counts, kWarpsExplore * 32, smem, occ);
     if (e != cudaSuccess) return e;
     k_update_counts<<<explore_grid(nbeams, kWarpsExplore), kWarpsExplore * 32, smem, s>>>(
         W, H, poses, P, dirs, B, ranges, rfix, cap, stride, counts, status);

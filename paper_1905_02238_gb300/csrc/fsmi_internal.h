@@ -65,6 +65,14 @@ const Schedule &current_schedule(int kind);  // FSMI_KIND_2D / FSMI_KIND_RLE
 // memory fit in one block of the current device (at least 1).
 int fit_warps(int warps, size_t per_warp, size_t fixed);
 
+// One launch of a persistent kernel over n items, one item per warp at a time: as many blocks as fit on the
+// GPU (at most max_blocks_per_sm per SM, 0 = no cap) or as n needs.
+struct WarpGrid {
+    unsigned grid;
+    bool one_each;  // a warp for every item: static assignment gives each warp at most one, a queue nothing
+};
+cudaError_t warp_grid(const void *kern, long long n, int wpb, size_t smem, int max_blocks_per_sm, WarpGrid &g);
+
 // Bytes at the front of an evaluation workspace reserved for the work-queue counter.
 constexpr size_t kQueueBytes = 256;
 
@@ -113,6 +121,12 @@ cudaError_t launch_rle_encode_3d_static(const Vox3D &v, const DevParams &p, int3
                                         cudaStream_t s);
 
 int sm_count();
+
+// Resident blocks per SM of `kern` with `threads` threads and `smem` bytes of dynamic shared memory on the
+// current device, its dynamic shared memory limit raised to the device's maximum. Looked up once per
+// kernel, block size and device and remembered per host thread (the attribute and occupancy calls were 4 of the
+// 10 us of a launch).
+cudaError_t resident_blocks(const void *kern, int threads, size_t smem, int &blocks);
 // records e as the calling thread's last CUDA error and returns FSMI_ERR_CUDA
 fsmi_status record_cuda_error(cudaError_t e);
 // poll limit of the surrogate fc kernel's epilogue wait for this host thread (< 0: the default)

@@ -387,15 +387,9 @@ cudaError_t launch_mixed_variant(const MixedSrc &src, const DevParams &p2, const
     const int wpb = fit_warps(sc.warps_per_block, per_warp, table);
     const size_t smem = table + (size_t)wpb * per_warp;
     auto kern = k_eval_mixed<VAR, KIND>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    WarpGrid g;
+    cudaError_t e = warp_grid((const void *)kern, nitems, wpb, smem, sc.blocks_per_sm, g);
     if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, wpb * 32, smem);
-    if (e != cudaSuccess) return e;
-    if (occ < 1) return cudaErrorInvalidConfiguration;
-    if (sc.blocks_per_sm > 0 && sc.blocks_per_sm < occ) occ = sc.blocks_per_sm;
-    long long grid = (long long)sm_count() * occ;
-    if (grid > (nitems + wpb - 1) / wpb) grid = (nitems + wpb - 1) / wpb;
     if (queue) {
         e = cudaMemsetAsync(queue, 0, sizeof(unsigned long long), s);
         if (e != cudaSuccess) return e;
@@ -406,7 +400,7 @@ cudaError_t launch_mixed_variant(const MixedSrc &src, const DevParams &p2, const
     }
     RleTable tbl{};
     if (src.has3d) fill_rle_table(p3, tbl);
-    kern<<<(unsigned)grid, wpb * 32, smem, s>>>(src, p2, p3, tbl, nitems, stride2, stride3, out, times, status, queue,
+    kern<<<g.grid, wpb * 32, smem, s>>>(src, p2, p3, tbl, nitems, stride2, stride3, out, times, status, queue,
                                                 sc.queue_chunk > 0 ? sc.queue_chunk : 1, plan, bucket);
     return cudaGetLastError();
 }

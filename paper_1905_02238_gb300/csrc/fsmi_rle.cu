@@ -209,23 +209,6 @@ void fill_rle_table(const DevParams &p, RleTable &t)
     }
 }
 
-template <typename Kern>
-static cudaError_t grid_for(Kern k, size_t smem, long long nitems, int wpb, int bps, long long &grid)
-{
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, wpb * 32, smem);
-    if (e != cudaSuccess) return e;
-    if (occ < 1) return cudaErrorInvalidConfiguration;
-    if (bps > 0 && bps < occ) occ = bps;
-    const long long want = (nitems + wpb - 1) / wpb;
-    grid = (long long)sm_count() * occ;
-    if (grid > want) grid = want;
-    if (grid < 1) grid = 1;
-    return cudaSuccess;
-}
-
 static cudaError_t reset_queue(unsigned long long *queue, cudaStream_t s)
 {
     return queue ? cudaMemsetAsync(queue, 0, sizeof(unsigned long long), s) : cudaSuccess;
@@ -242,16 +225,17 @@ cudaError_t launch_eval_3d(const Vox3D &v, const DevParams &p, float *out, int32
     const size_t per_warp = (size_t)wf * sizeof(float);
     const int wpb = fit_warps(sc.warps_per_block, per_warp, rle_table_bytes(p.K));
     const size_t smem = rle_table_bytes(p.K) + (size_t)wpb * per_warp;
-    long long grid;
+    WarpGrid g;
     const bool wide = nrays > 0x7fffffffLL;
     auto kern = thm5_of(p) ? (wide ? k_eval_3d<kRay3dThm5, true> : k_eval_3d<kRay3dThm5, false>)
                            : (wide ? k_eval_3d<kRay3dOther, true> : k_eval_3d<kRay3dOther, false>);
-    cudaError_t e = grid_for(kern, smem, nrays, wpb, sc.blocks_per_sm, grid);
+    cudaError_t e = warp_grid((const void *)kern, nrays, wpb, smem, sc.blocks_per_sm, g);
+    if (e == cudaSuccess && g.one_each) queue = nullptr;  // nothing to balance
     if (e == cudaSuccess) e = reset_queue(queue, s);
     if (e != cudaSuccess) return e;
     RleTable tbl;
     fill_rle_table(p, tbl);
-    kern<<<(unsigned)grid, wpb * 32, smem, s>>>(v, p, tbl, nrays, wf, out, nruns, queue,
+    kern<<<g.grid, wpb * 32, smem, s>>>(v, p, tbl, nrays, wf, out, nruns, queue,
                                                 sc.queue_chunk > 0 ? sc.queue_chunk : 1);
     return cudaGetLastError();
 }
@@ -265,13 +249,14 @@ cudaError_t launch_eval_rle(const int32_t *run_off, const float *run_o, const ui
     const size_t per_warp = (size_t)kArraysRLE * stride * sizeof(float);
     const int wpb = fit_warps(sc.warps_per_block, per_warp, rle_table_bytes(p.K));
     const size_t smem = rle_table_bytes(p.K) + (size_t)wpb * per_warp;
-    long long grid;
-    cudaError_t e = grid_for(k_eval_rle, smem, nrays, wpb, sc.blocks_per_sm, grid);
+    WarpGrid g;
+    cudaError_t e = warp_grid((const void *)k_eval_rle, nrays, wpb, smem, sc.blocks_per_sm, g);
+    if (e == cudaSuccess && g.one_each) queue = nullptr;
     if (e == cudaSuccess) e = reset_queue(queue, s);
     if (e != cudaSuccess) return e;
     RleTable tbl;
     fill_rle_table(p, tbl);
-    k_eval_rle<<<(unsigned)grid, wpb * 32, smem, s>>>(run_off, run_o, run_len, p, tbl, nrays, stride, out, status,
+    k_eval_rle<<<g.grid, wpb * 32, smem, s>>>(run_off, run_o, run_len, p, tbl, nrays, stride, out, status,
                                                       queue, sc.queue_chunk > 0 ? sc.queue_chunk : 1);
     return cudaGetLastError();
 }
@@ -286,10 +271,10 @@ cudaError_t launch_rle_encode_3d(const Vox3D &v, const DevParams &p, int32_t *ru
     }
     const int stride = rle_stride(p.nmax, 0);
     const size_t smem = (size_t)kWarpsRLE * 2 * stride * sizeof(float);
-    long long grid;
-    cudaError_t e = grid_for(k_rle_count, smem, nrays, kWarpsRLE, 0, grid);
+    WarpGrid g;
+    cudaError_t e = warp_grid((const void *)k_rle_count, nrays, kWarpsRLE, smem, 0, g);
     if (e != cudaSuccess) return e;
-    k_rle_count<<<(unsigned)grid, kWarpsRLE * 32, smem, s>>>(v, p, nrays, stride, run_off);
+    k_rle_count<<<g.grid, kWarpsRLE * 32, smem, s>>>(v, p, nrays, stride, run_off);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_scan_tiles<<<ntiles, 1024, 0, s>>>(run_off + 1, nrays, ws_tiles);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -299,9 +284,9 @@ cudaError_t launch_rle_encode_3d(const Vox3D &v, const DevParams &p, int32_t *ru
     if (ag > (long long)sm_count() * 8) ag = (long long)sm_count() * 8;
     k_scan_add<<<(unsigned)ag, 256, 0, s>>>(run_off + 1, nrays, ws_tiles);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    e = grid_for(k_rle_write, smem, nrays, kWarpsRLE, 0, grid);
+    e = warp_grid((const void *)k_rle_write, nrays, kWarpsRLE, smem, 0, g);
     if (e != cudaSuccess) return e;
-    k_rle_write<<<(unsigned)grid, kWarpsRLE * 32, smem, s>>>(v, p, nrays, stride, run_off, run_o, run_len,
+    k_rle_write<<<g.grid, kWarpsRLE * 32, smem, s>>>(v, p, nrays, stride, run_off, run_o, run_len,
                                                               run_capacity, status);
     return cudaGetLastError();
 }

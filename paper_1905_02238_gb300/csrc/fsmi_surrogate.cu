@@ -520,7 +520,8 @@ cudaError_t gemm_terms(int M, int N, int K, int splits, const bf16 *A, size_t ta
 {
     auto kern = k_gemm_terms<TA, TB, AT, BT, FE>;
     const int smem = kGmSmem<TA, TB>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    int occ = 0;
+    cudaError_t e = resident_blocks((const void *)kern, 256, smem, occ);
     if (e != cudaSuccess) return e;
     const int kper = ((K + splits - 1) / splits + kGmK - 1) / kGmK * kGmK;
     kern<<<dim3(N / kGmN, (M + kGmM - 1) / kGmM, splits), 256, smem, s>>>(M, N, K, kper, A, ta, lda, B, tb, ldb, fe);
@@ -1585,12 +1586,9 @@ cudaError_t launch_surrogate_infer(const float *map, int W, int H, const int32_t
     unsigned long long *queue = (unsigned long long *)ws;
     bf16 *h0 = (bf16 *)((char *)ws + kQueueBytes);
     const size_t smem_conv = kConvSmem;
-    cudaError_t e = cudaFuncSetAttribute(k_conv_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_conv);
-    if (e != cudaSuccess) return e;
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_conv_infer, kConvWarps * 32, smem_conv);
+    cudaError_t e = resident_blocks((const void *)k_conv_infer, kConvWarps * 32, smem_conv, occ);
     if (e != cudaSuccess) return e;
-    if (occ < 1) return cudaErrorInvalidConfiguration;
     e = cudaMemsetAsync(queue, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
     long long grid = (long long)sm_count() * occ;
@@ -1606,7 +1604,7 @@ cudaError_t launch_surrogate_infer(const float *map, int W, int H, const int32_t
     e = encode_bf16_2d(&tmA, h0, kFlat, (unsigned long long)N, kTcK, kTcRows);
     if (e == cudaSuccess) e = encode_bf16_2d(&tmB, w + oW4, kFlat, kHid, kTcK, kHid);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_fc_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
+    e = resident_blocks((const void *)k_fc_tc, kTcThreads, kTcSmem, occ);
     if (e != cudaSuccess) return e;
     k_fc_tc<<<(unsigned)(tiles < (long long)sm_count() ? tiles : sm_count()), kTcThreads, kTcSmem, s>>>(
         tmA, tmB, N, w, params, pred, status, g_epi_polls);

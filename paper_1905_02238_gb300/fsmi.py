@@ -202,7 +202,8 @@ def _raise(code: int, what: str):
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The current stream's handle (the raw form: building a torch.cuda.Stream takes ten times as long)."""
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _ptr(t):
@@ -227,6 +228,12 @@ def _default_ws(nbytes: int, dev):
     if _capturing():
         return None
     return torch.empty(nbytes, dtype=torch.uint8, device=dev)
+
+
+def _small_2d(nbeams: int, cells: int, max_range: float) -> bool:
+    """Whether fsmi_eval_2d has no use for a workspace: fewer cell visits than map cells (no per-cell gains,
+    the library's own rule) and a warp for every beam (no queue; 1,216 warps fit at the longest range)."""
+    return nbeams <= 1024 and 0 < max_range <= MAX_RANGE_2D and nbeams * ((int(max_range * 1.41421357) + 3) // 2) < cells
 
 
 def _out(out, shape, m):
@@ -276,10 +283,10 @@ def eval_2d(grid: torch.Tensor, poses: torch.Tensor, dirs: torch.Tensor, prm: Pa
     ds = m.arg(dirs, torch.int32, "dirs", 2, 2)
     P, B = ps.shape[0], ds.shape[0]
     out = _out(out, (P, B), m)
-    if ws is None:
+    cp = prm.c()
+    if ws is None and not _small_2d(P * B, g.numel(), cp.max_range):
         ws = _default_ws(workspace_size(FN_EVAL_2D, g.numel()), m.dev)
     wp, wb = _ws_args(ws)
-    cp = prm.c()
     _raise(lib.fsmi_eval_2d(_ptr(g), g.shape[1], g.shape[0], _ptr(ps), P, _ptr(ds), B, ctypes.byref(cp),
                             _ptr(out), wp, wb, _stream()), "fsmi_eval_2d")
     return m.out(out)
@@ -499,8 +506,8 @@ def trace_2d(W: int, H: int, poses, dirs, max_range: float, cap: int):
 def workspace_size(fn: int, nitems: int, prm: Params | None = None) -> int:
     lib = load()
     b = ctypes.c_size_t(0)
-    cp = (prm or Params()).c()
-    _raise(lib.fsmi_workspace_size(fn, nitems, ctypes.byref(cp), ctypes.byref(b)), "fsmi_workspace_size")
+    cp = ctypes.byref(prm.c()) if prm is not None else None
+    _raise(lib.fsmi_workspace_size(fn, nitems, cp, ctypes.byref(b)), "fsmi_workspace_size")
     return int(b.value)
 
 
