@@ -53,6 +53,11 @@ __device__ __forceinline__ void rle_gains(const DevParams &p, float o, float &fo
     unpack2(mul2(pack2(w, w), h), fo, fe);
 }
 
+// C keeps its first cell at a 16-byte boundary, conv_pad(K) >= K floats after its array's start; four outputs
+// read conv_quads(K) groups of four of it
+__host__ __device__ constexpr int conv_pad(int K) { return (K + 3) & ~3; }
+__host__ __device__ constexpr int conv_quads(int K) { return (conv_pad(K) + K + 7) / 4; }
+
 // ---- noise-kernel prefix tables --------------------------------------------------------------
 
 // tab[i] = (Psi(m), Psi1(m)) for m = i - K - 1, i in [0, 2K + 1]; Psi(-K-1) = 0, Psi(K) = total;
@@ -60,10 +65,15 @@ __device__ __forceinline__ void rle_gains(const DevParams &p, float o, float &fo
 // density (Theorem 3), 1 Gaussian cell mass, 2 box 1[|d| <= H] (Theorem 6); band >= 0 zeroes
 // |d| > band, the strict-band reading of Approx-FSMI-RLE; normalisation folded into g; in double,
 // stored as float); each block copies them from the launch's parameters into shared memory.
-static __device__ void load_table(float2 *tab, float *gtab, int K, const RleTable &t)
+// gz (for band_conv_any) is g with zeros around it: gz[4 + (conv_pad(K) - K) + d] = g(d - K), d = 0 .. 2K.
+static __device__ void load_table(float2 *tab, float *gtab, float *gz, int K, const RleTable &t)
 {
     for (int i = threadIdx.x; i < 2 * K + 2; i += blockDim.x) tab[i] = t.tab[i];
     for (int i = threadIdx.x; i < 2 * K + 1; i += blockDim.x) gtab[i] = t.gtab[i];
+    for (int i = threadIdx.x; i < 4 * (conv_quads(K) + 1); i += blockDim.x) {
+        const int d = i - 4 - (conv_pad(K) - K);
+        gz[i] = d >= 0 && d <= 2 * K ? t.gtab[d] : 0.0f;
+    }
     __syncthreads();
 }
 
@@ -244,9 +254,6 @@ static __device__ float pairs_thm5(const RunSmem &r, int nr, const float2 *tab, 
 
 constexpr int kArraysRLE = 7;                  // per-warp shared arrays (each `stride` floats)
 
-// C keeps its first cell at a 16-byte boundary, conv_pad(K) >= K floats after its array's start
-__host__ __device__ constexpr int conv_pad(int K) { return (K + 3) & ~3; }
-
 // ---- the cell form ---------------------------------------------------------------------------------
 //
 // A ray's cells go through in blocks of 128, four consecutive cells per lane: the gains, Algorithm 2's and 3's
@@ -255,53 +262,71 @@ __host__ __device__ constexpr int conv_pad(int K) { return (K + 3) & ~3; }
 // written and read back), the run-input kernel on the decompressed runs; the same operations in the
 // same order, so the two give the same floats.
 
+// 16 or 8 bytes of consecutive cells
+__device__ __forceinline__ void store_cells(float *p, const float (&v)[4])
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void store_cells(float *p, const float (&v)[2])
+{
+    *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
+}
+__device__ __forceinline__ void store_cells(int *p, const int (&v)[4])
+{
+    *reinterpret_cast<int4 *>(p) = make_int4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void store_cells(int *p, const int (&v)[2]) { *reinterpret_cast<int2 *>(p) = make_int2(v[0], v[1]); }
+
 // prefixes carried from block to block
 struct CellScan {
     float E, q;  // prod (1 - o) and sum f_emp of the cells before the block
 };
 
-// One block: o of this lane's cells i0 .. i0 + 3 (zero from the ray's end on); stores P in CP and C in CB where
-// i0 < n.
-__device__ __forceinline__ void scan_block(const DevParams &p, const float (&o)[4], int i0, int n, CellScan &s, float *CP,
+// cells per lane: rays of at most 64 samples go in one block of 64, so that half the lanes' work is not idle
+__host__ __device__ constexpr int kShortRay = 64;
+
+// One block of 32 CPL cells (CPL = 4, or 2 on short rays): o of this lane's cells i0 .. i0 + CPL - 1 (zero from
+// the ray's end on); stores P in CP and C in CB where i0 < n.
+template <int CPL>
+__device__ __forceinline__ void scan_block(const DevParams &p, const float (&o)[CPL], int i0, int n, CellScan &s, float *CP,
                                            float *CB)
 {
-    float fo[4], fe[4];
+    float fo[CPL], fe[CPL];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) rle_gains(p, o[t], fo[t], fe[t]);
-    const float prod = warp_incl_mul(((1.0f - o[0]) * (1.0f - o[1])) * ((1.0f - o[2]) * (1.0f - o[3])));
-    const float sum = warp_incl_add((fe[0] + fe[1]) + (fe[2] + fe[3]));
+    for (int t = 0; t < CPL; ++t) rle_gains(p, o[t], fo[t], fe[t]);
+    float prod = (1.0f - o[0]) * (1.0f - o[1]), sum = fe[0] + fe[1];
+    if (CPL == 4) {
+        prod *= (1.0f - o[CPL - 2]) * (1.0f - o[CPL - 1]);
+        sum += fe[CPL - 2] + fe[CPL - 1];
+    }
+    prod = warp_incl_mul(prod);
+    sum = warp_incl_add(sum);
     float E = __shfl_up_sync(kFull, prod, 1), q = __shfl_up_sync(kFull, sum, 1);
     const int lane = lane_id();
     E = lane == 0 ? s.E : s.E * E;
     q = lane == 0 ? s.q : s.q + q;
     s.E *= __shfl_sync(kFull, prod, 31);
     s.q += __shfl_sync(kFull, sum, 31);
-    float4 P, C;
-    P.x = E * o[0];  // Algorithm 2
-    E *= 1.0f - o[0];
-    P.y = E * o[1];
-    E *= 1.0f - o[1];
-    P.z = E * o[2];
-    E *= 1.0f - o[2];
-    P.w = E * o[3];
-    C.x = q + fo[0];  // Algorithm 3
-    q += fe[0];
-    C.y = q + fo[1];
-    q += fe[1];
-    C.z = q + fo[2];
-    q += fe[2];
-    C.w = q + fo[3];
+    float P[CPL], C[CPL];
+#pragma unroll
+    for (int t = 0; t < CPL; ++t) {
+        P[t] = E * o[t];  // Algorithm 2
+        E *= 1.0f - o[t];
+        C[t] = q + fo[t];  // Algorithm 3
+        q += fe[t];
+    }
     if (i0 < n) {
-        *reinterpret_cast<float4 *>(CP + i0) = P;
-        *reinterpret_cast<float4 *>(CB + i0) = C;
+        store_cells(CP + i0, P);
+        store_cells(CB + i0, C);
     }
 }
 
-// K zeros before C_0 and K + 8 from C_n on (scan_block leaves up to three entries past C_{n-1} undefined)
+// conv_pad(K) zeros before C_0 and K + 8 from C_n on (scan_block leaves up to three entries past C_{n-1}
+// undefined)
 __device__ __forceinline__ void pad_conv(float *CB, int K, int n)
 {
     for (int i = lane_id(); i < K + 8; i += 32) {
-        if (i < K) CB[-1 - i] = 0.0f;
+        if (i < conv_pad(K)) CB[-1 - i] = 0.0f;
         CB[n + i] = 0.0f;
     }
     __syncwarp();
@@ -373,18 +398,49 @@ __device__ __forceinline__ float band_conv_k(const float *CP, const float *CB, c
     return n > 128 ? band_conv_v<KK, 8>(CP, CB, t, n) : band_conv_v<KK, 4>(CP, CB, t, n);
 }
 
-__device__ __forceinline__ float band_conv(const float *CP, const float *CB, const float *gtab, const RleTable &t, int K, int n)
+// The same for any radius: four outputs per lane, and per group of four inputs one 16-byte load of C and one
+// (the same for all lanes) of the zero-padded kernel, for 16 products. (A load of C and one of g per product:
+// BANDANY_NOTE.)
+__device__ __forceinline__ float band_conv_any(const float *CP, const float *CB, const float *gz, int K, int n)
 {
-    if (K == 15) return band_conv_k<15>(CP, CB, t, n);  // Gaussian kernels at sigma = 2 cells
-    if (K == 6) return band_conv_k<6>(CP, CB, t, n);    // strict band, Delta = 6
-    if (K == 4) return band_conv_k<4>(CP, CB, t, n);    // box kernel, H = 4
+    const int quads = conv_quads(K);
     float v = 0.0f;
-    for (int j = lane_id(); j < n; j += 32) {
-        float acc = 0.0f;
-        for (int d = -K; d <= K; ++d) acc = fmaf(gtab[K + d], CB[j + d], acc);
-        v = fmaf(CP[j], acc, v);
+    for (int j0 = 4 * lane_id(); j0 < n; j0 += 128) {
+        const float4 *c4 = reinterpret_cast<const float4 *>(CB + j0 - conv_pad(K)), *g4 = reinterpret_cast<const float4 *>(gz);
+        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        float4 a = g4[0];
+        for (int m = 0; m < quads; ++m) {
+            const float4 c = c4[m], b = g4[m + 1];
+            const float x[4] = {c.x, c.y, c.z, c.w}, g[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int h = 0; h < 4; ++h)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[q] = fmaf(x[h], g[4 + h - q], acc[q]);
+            a = b;
+        }
+        const float4 P = *reinterpret_cast<const float4 *>(CP + j0);
+        v = fmaf(P.x, acc[0], v);
+        if (j0 + 1 < n) v = fmaf(P.y, acc[1], v);
+        if (j0 + 2 < n) v = fmaf(P.z, acc[2], v);
+        if (j0 + 3 < n) v = fmaf(P.w, acc[3], v);
     }
     return v;
+}
+
+// radii with a compiled-in convolution: Gaussian kernels at sigma = 2 cells, the strict band of Delta = 6, the
+// box of H = 4
+__host__ __device__ constexpr bool conv_fixed(int K) { return K == 15 || K == 6 || K == 4; }
+
+// FIXED / ANY: whether the kernel holds the compiled-in radii and the general form
+template <bool FIXED, bool ANY>
+__device__ __forceinline__ float band_conv(const float *CP, const float *CB, const float *gz, const RleTable &t, int K, int n)
+{
+    if (FIXED) {
+        if (K == 15) return band_conv_k<15>(CP, CB, t, n);
+        if (K == 6) return band_conv_k<6>(CP, CB, t, n);
+        if (K == 4 || !ANY) return band_conv_k<4>(CP, CB, t, n);
+    }
+    return band_conv_any(CP, CB, gz, K, n);
 }
 
 // Theorem 5 at the cell level. The pairs (j, k) its sub-blocks keep (the whole diagonal block of
@@ -442,13 +498,46 @@ __device__ __forceinline__ float window_conv_k(const float *CP, const float *CB,
     return v;
 }
 
+// The cells of a ray given as runs through scan_block: RI holds run u's index at its first cell and 0
+// elsewhere; with keep it receives every cell's run index.
+template <int CPL>
+__device__ __forceinline__ void decompress(const DevParams &p, const float *O, int *RI, int n, float *CP, float *CB, bool keep)
+{
+    const int lane = lane_id();
+    CellScan s{1.0f, 0.0f};
+    int last = 0;  // run of the last cell before the block
+    for (int base = 0; base < n; base += 32 * CPL) {
+        const int i0 = base + CPL * lane;
+        int u[CPL];
+#pragma unroll
+        for (int t = 0; t < CPL; ++t) u[t] = max(t ? u[t > 0 ? t - 1 : 0] : 0, i0 + t < n ? RI[i0 + t] : 0);
+        int m = u[CPL - 1];  // running maximum over the lanes
+#pragma unroll
+        for (int k = 1; k < 32; k <<= 1) {
+            const int v = __shfl_up_sync(kFull, m, k);
+            if (lane >= k) m = max(m, v);
+        }
+        int before = __shfl_up_sync(kFull, m, 1);
+        before = lane == 0 ? last : max(before, last);
+        last = max(last, __shfl_sync(kFull, m, 31));
+        float o[CPL];
+#pragma unroll
+        for (int t = 0; t < CPL; ++t) {
+            u[t] = max(u[t], before);
+            o[t] = i0 + t < n ? O[u[t]] : 0.0f;
+        }
+        if (keep && i0 < n) store_cells(RI + i0, u);
+        scan_block<CPL>(p, o, i0, n, s, CP, CB);
+    }
+}
+
 // Cell-level evaluation (eq. eqn_from_fsmi) of one ray given as runs: decompress the runs into the n virtual
 // cells, form P(e_j) and C_k (Algorithms 2 and 3), then I = sum_j P(e_j) sum_{|d| <= K} g(d) C_{j+d}
 // (FSMI-RLE, Uniform-FSMI-RLE, strict-band Approx-FSMI-RLE), or for Theorem 5 the same sum over each
 // first-hit cell's window of kept pairs (window_conv). Each run's index is put at its first cell and
 // spread by a running maximum. Arrays: 0 run o, 3 P, 4 run starts S, 5 the cells' run indices, 6 C.
 static __device__ float ray_mi_cells(float *base, int stride, int nr, int n, const DevParams &p, const float *gtab,
-                                     const RleTable &t, int K, bool thm5)
+                                     const float *gz, const RleTable &t, int K, bool thm5)
 {
     const int lane = lane_id();
     const float *O = base;
@@ -459,43 +548,18 @@ static __device__ float ray_mi_cells(float *base, int stride, int nr, int n, con
     __syncwarp();
     for (int u = lane; u < nr; u += 32) RI[S[u]] = u;  // every run has a cell, so no two share one
     __syncwarp();
-    CellScan s{1.0f, 0.0f};
-    int last = 0;  // run of the last cell before the block
-    for (int base_i = 0; base_i < n; base_i += 128) {
-        const int i0 = base_i + 4 * lane;
-        int4 u = make_int4(0, 0, 0, 0);
-        if (i0 < n) u = *reinterpret_cast<const int4 *>(RI + i0);
-        u.y = max(u.x, i0 + 1 < n ? u.y : 0);
-        u.z = max(u.y, i0 + 2 < n ? u.z : 0);
-        u.w = max(u.z, i0 + 3 < n ? u.w : 0);
-        int m = u.w;  // running maximum over the lanes
-#pragma unroll
-        for (int k = 1; k < 32; k <<= 1) {
-            const int v = __shfl_up_sync(kFull, m, k);
-            if (lane >= k) m = max(m, v);
-        }
-        int before = __shfl_up_sync(kFull, m, 1);
-        before = lane == 0 ? last : max(before, last);
-        last = max(last, __shfl_sync(kFull, m, 31));
-        u = make_int4(max(u.x, before), max(u.y, before), max(u.z, before), max(u.w, before));
-        float o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        if (i0 < n) {
-            o[0] = O[u.x];
-            if (i0 + 1 < n) o[1] = O[u.y];
-            if (i0 + 2 < n) o[2] = O[u.z];
-            if (i0 + 3 < n) o[3] = O[u.w];
-            if (thm5) *reinterpret_cast<int4 *>(RI + i0) = u;
-        }
-        scan_block(p, o, i0, n, s, CP, CB);
-    }
+    if (p.nmax > kShortRay)
+        decompress<4>(p, O, RI, n, CP, CB, thm5);
+    else
+        decompress<2>(p, O, RI, n, CP, CB, thm5);
     __syncwarp();
     if (thm5) return window_conv(CP, CB, gtab, K, n, S, RI, p.trunc);
     pad_conv(CB, K, n);
-    return band_conv(CP, CB, gtab, t, K, n);
+    return band_conv<true, true>(CP, CB, gz, t, K, n);
 }
 
 __device__ __forceinline__ float ray_mi(float *base, int stride, int nr, const DevParams &p, const float2 *tab,
-                                        const float *gtab, const RleTable &t, int K, bool have_s)
+                                        const float *gtab, const float *gz, const RleTable &t, int K, bool have_s)
 {
     if (nr <= 0) return 0.0f;
     const RunSmem r = run_smem(base, stride);
@@ -504,7 +568,7 @@ __device__ __forceinline__ float ray_mi(float *base, int stride, int nr, const D
     const bool thm5 = p.variant == FSMI_APPROX && p.approx_reading == 0;
     float v;
     if (n < p.cell_runlen * nr) {
-        v = ray_mi_cells(base, stride, nr, n, p, gtab, t, K, thm5);
+        v = ray_mi_cells(base, stride, nr, n, p, gtab, gz, t, K, thm5);
     } else {
         run_prefixes(r, nr, p);
         if (p.variant == FSMI_APPROX && p.approx_reading == 0)
@@ -605,19 +669,20 @@ static __device__ int sample_encode_ray(const float *__restrict__ vox, int X, in
     return nrun;
 }
 
-// Runs of a block of 128 cells, four consecutive ones per lane (nw: a new value begins at the cell): O[k], S[k] of
+// Runs of a block of cells, CPL consecutive ones per lane (nw: a new value begins at the cell): O[k], S[k] of
 // the runs below nrcap, and with RI every cell's run index.
 struct RunScan {
     int nrun, carried;  // runs so far, start of the span that reaches into the block
 };
-__device__ __forceinline__ void encode_block(const float (&o)[4], const bool (&nw)[4], int i0, int n, int cap, float inv_cap,
+template <int CPL>
+__device__ __forceinline__ void encode_block(const float (&o)[CPL], const bool (&nw)[CPL], int i0, int n, int cap, float inv_cap,
                                              RunScan &s, float *O, int *S, int nrcap, int *RI)
 {
     const int lane = lane_id();
     // start of each cell's span: the last cell at or before it where a new value begins
-    int st[4], own = -1;
+    int st[CPL], own = -1;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
+    for (int t = 0; t < CPL; ++t) {
         if (nw[t]) own = i0 + t;
         st[t] = own;
     }
@@ -630,19 +695,19 @@ __device__ __forceinline__ void encode_block(const float (&o)[4], const bool (&n
     int from = __shfl_up_sync(kFull, m, 1);
     from = lane == 0 ? s.carried : max(from, s.carried);
     s.carried = max(s.carried, __shfl_sync(kFull, m, 31));
-    bool brk[4];
+    bool brk[CPL];
     int cnt = 0;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
+    for (int t = 0; t < CPL; ++t) {
         const int rel = i0 + t - max(st[t], from);  // a multiple of cap starts a run (exact, see sample_encode_ray)
         brk[t] = i0 + t < n && rel - __float2int_rn((float)rel * inv_cap) * cap == 0;
         cnt += brk[t];
     }
     const int incl = warp_incl_add_int(cnt);
-    int k = s.nrun + incl - cnt, r[4];
+    int k = s.nrun + incl - cnt, r[CPL];
     s.nrun += __shfl_sync(kFull, incl, 31);
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
+    for (int t = 0; t < CPL; ++t) {
         if (brk[t]) {
             if (k < nrcap) {
                 O[k] = o[t];
@@ -652,7 +717,7 @@ __device__ __forceinline__ void encode_block(const float (&o)[4], const bool (&n
         }
         r[t] = k - 1;
     }
-    if (RI && i0 < n) *reinterpret_cast<int4 *>(RI + i0) = make_int4(r[0], r[1], r[2], r[3]);
+    if (RI && i0 < n) store_cells(RI + i0, r);
 }
 
 // The fused kernel's form: blocks of 128 samples, four consecutive ones per lane, straight through scan_block into
@@ -665,7 +730,7 @@ __device__ __forceinline__ void encode_block(const float (&o)[4], const bool (&n
 // once and stores three 16-byte words. 512x512x128 voxels, 64 poses x 128x128 rays: 1,741 to 1,068 warp
 // instructions per ray and 1,690 to 1,136 us, with the convolution below; Theorem 5 on 301x253x77 voxels,
 // 23 x 80x61 rays: 162 to 149 us. The registers (73) leave 28 warps per SM; held to 64: 1,152 - 1,172 us.
-template <bool ENC>
+template <int CPL, bool ENC>
 __device__ __forceinline__ int sample_cells(const float *__restrict__ vox, int X, int Y, int Z, const int32_t *pose,
                                             const int32_t *u, int nsamp, const DevParams &p, float *CP, float *CB, float *CO,
                                             float *O, int *S, int nrcap, int *RI, int &count)
@@ -674,36 +739,36 @@ __device__ __forceinline__ int sample_cells(const float *__restrict__ vox, int X
     long long d[3], q[3];
     ray_dir(pose, u, q, d);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) q[a] += (8LL * lane + 1) * d[a];  // sample 4 lane
+    for (int a = 0; a < 3; ++a) q[a] += (2LL * CPL * lane + 1) * d[a];  // sample CPL lane
     CellScan s{1.0f, 0.0f};
     RunScan rs{0, 0};
     const float inv_cap = 1.0f / (float)p.run_cap;
     unsigned prev = 0u;
     int n = 0, spans = 0;
-    for (int base = 0; base < nsamp; base += 128) {
-        const int i0 = base + 4 * lane;
-        float o[4];
-        bool in[4];
+    for (int base = 0; base < nsamp; base += 32 * CPL) {
+        const int i0 = base + CPL * lane;
+        float o[CPL];
+        bool in[CPL];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < CPL; ++t) {
             // as in sample_encode_ray
             const unsigned px = (unsigned)(q[0] >> 31), py = (unsigned)(q[1] >> 31), pz = (unsigned)(q[2] >> 31);
             in[t] = px < (unsigned)X && py < (unsigned)Y && pz < (unsigned)Z && i0 + t < nsamp;
             o[t] = in[t] ? __ldg(vox + ((size_t)(pz * (unsigned)Y + py) * (unsigned)X + px)) : 0.0f;
 #pragma unroll
-            for (int a = 0; a < 3; ++a) q[a] += (t < 3 ? 2 : 250) * d[a];
+            for (int a = 0; a < 3; ++a) q[a] += (t < CPL - 1 ? 2 : 64 * CPL - 2 * CPL + 2) * d[a];
         }
         // the ray ends at its first sample outside
-        const int c = !in[0] ? 0 : !in[1] ? 1 : !in[2] ? 2 : !in[3] ? 3 : 4;
-        const unsigned m = __ballot_sync(kFull, c == 4);
+        const int c = !in[0] ? 0 : !in[1] ? 1 : CPL == 2 || !in[CPL - 2] ? 2 : !in[CPL - 1] ? 3 : 4;
+        const unsigned m = __ballot_sync(kFull, c == CPL);
         const int L = m == kFull ? 31 : __ffs(~m) - 1;
-        n = base + 4 * L + __shfl_sync(kFull, c, L);
-        const unsigned left = __shfl_up_sync(kFull, __float_as_uint(o[3]), 1);
+        n = base + CPL * L + __shfl_sync(kFull, c, L);
+        const unsigned left = __shfl_up_sync(kFull, __float_as_uint(o[CPL - 1]), 1);
         unsigned before = lane == 0 ? prev : left;
-        prev = __shfl_sync(kFull, __float_as_uint(o[3]), 31);
-        bool nw[4];
+        prev = __shfl_sync(kFull, __float_as_uint(o[CPL - 1]), 31);
+        bool nw[CPL];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < CPL; ++t) {
             const unsigned bits = __float_as_uint(o[t]);
             const bool valid = i0 + t < n;
             nw[t] = valid && (bits != before || i0 + t == 0);
@@ -712,10 +777,10 @@ __device__ __forceinline__ int sample_cells(const float *__restrict__ vox, int X
             if (!valid) o[t] = 0.0f;
         }
         if (ENC)
-            encode_block(o, nw, i0, n, p.run_cap, inv_cap, rs, O, S, nrcap, RI);
+            encode_block<CPL>(o, nw, i0, n, p.run_cap, inv_cap, rs, O, S, nrcap, RI);
         else if (i0 < n)
-            *reinterpret_cast<float4 *>(CO + i0) = make_float4(o[0], o[1], o[2], o[3]);
-        scan_block(p, o, i0, n, s, CP, CB);
+            store_cells(CO + i0, o);
+        scan_block<CPL>(p, o, i0, n, s, CP, CB);
         if (m != kFull) break;
     }
     if (ENC) {
@@ -750,7 +815,7 @@ static __device__ int encode_cells(const float *CO, int n, int cap, float *O, in
             nw[t] = i0 + t < n && (bits != before || i0 + t == 0);
             before = bits;
         }
-        encode_block(o, nw, i0, n, cap, inv_cap, rs, O, S, nrcap, nullptr);
+        encode_block<4>(o, nw, i0, n, cap, inv_cap, rs, O, S, nrcap, nullptr);
     }
     if (lane == 0 && rs.nrun <= nrcap) S[rs.nrun] = n;
     __syncwarp();
@@ -781,18 +846,26 @@ __host__ __device__ inline int ray3d_warp_floats(const DevParams &p)
                       : 3 * ray3d_cell_stride(p) + 6 * ray3d_run_stride(p);
 }
 
-// Which evaluation paths a fused-ray kernel is compiled with: both (the variant read at run time),
-// Theorem 5's sub-blocks only, or the others (cell-level convolution and all run pairs) only.
-enum { kRay3dAny = 0, kRay3dThm5 = 1, kRay3dOther = 2 };
+// Which evaluation paths a fused-ray kernel is compiled with (each kernel holds as little as it can, for its
+// registers): everything, with the variant and the ray's length read at run time; Theorem 5's sub-blocks;
+// the others (cell-level convolution and all run pairs) with a general or with a compiled-in radius
+// (conv_fixed).
+enum { kRay3dAny = 0, kRay3dThm5 = 1, kRay3dOther = 2, kRay3dFixed = 3 };
+__host__ __device__ inline int ray3d_mode(const DevParams &p)
+{
+    return thm5_of(p) ? kRay3dThm5 : conv_fixed(p.K) ? kRay3dFixed : kRay3dOther;
+}
 
 // Samples and evaluates one ray in the warp's region `w` (ray3d_warp_floats floats); returns the MI
-// (warp-reduced) and, with nr_out, the run count. MODE must agree with thm5_of(p). Outside Theorem 5 the runs are
+// (warp-reduced) and, with nr_out, the run count. MODE must agree with ray3d_mode(p). Outside Theorem 5 the runs are
 // formed (from the sampled values in shared memory) only where they are needed: for a caller who asks for
 // their number, or on a ray whose spans of equal values do not already show that its mean run is short.
-template <int MODE>
+// CPL: cells per lane of a block, 2 for rays of at most kShortRay samples, else 4 (0: read at run time).
+template <int MODE, int CPL>
 __device__ __forceinline__ float ray_mi_fused(const float *vox, int X, int Y, int Z, const int32_t *pose,
                                               const int32_t *u, int nsamp, const DevParams &p, const float2 *tab,
-                                              const float *gtab, const RleTable &t, int K, float *w, int *nr_out)
+                                              const float *gtab, const float *gz, const RleTable &t, int K, float *w,
+                                              int *nr_out)
 {
     const bool thm5 = MODE == kRay3dAny ? thm5_of(p) : MODE == kRay3dThm5;
     const int cst = ray3d_cell_stride(p), rst = ray3d_run_stride(p);
@@ -820,11 +893,15 @@ __device__ __forceinline__ float ray_mi_fused(const float *vox, int X, int Y, in
     int n, nr = 0;
     bool cells;
     if (thm5) {
-        n = sample_cells<true>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, r.O, r.S, ray3d_nrcap(p), RI, nr);
+        n = CPL == 4 || (CPL == 0 && nsamp > kShortRay)
+                ? sample_cells<4, true>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, r.O, r.S, ray3d_nrcap(p), RI, nr)
+                : sample_cells<2, true>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, r.O, r.S, ray3d_nrcap(p), RI, nr);
         cells = n < p.cell_runlen * nr;
     } else {
         int nspan;
-        n = sample_cells<false>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, nullptr, nullptr, 0, nullptr, nspan);
+        n = CPL == 4 || (CPL == 0 && nsamp > kShortRay)
+                ? sample_cells<4, false>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, nullptr, nullptr, 0, nullptr, nspan)
+                : sample_cells<2, false>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, nullptr, nullptr, 0, nullptr, nspan);
         cells = n < p.cell_runlen * nspan;  // at least one run per span
         if (n > 0 && (nr_out || !cells)) {
             nr = encode_cells(CO, n, p.run_cap, r.O, r.S, ray3d_nrcap(p));
@@ -842,7 +919,7 @@ __device__ __forceinline__ float ray_mi_fused(const float *vox, int X, int Y, in
                                                : window_conv(CP, CB, gtab, K, n, r.S, RI, p.trunc);
         } else {
             pad_conv(CB, K, n);
-            v = band_conv(CP, CB, gtab, t, K, n);
+            v = band_conv<MODE == kRay3dAny || MODE == kRay3dFixed, MODE == kRay3dAny || MODE == kRay3dOther>(CP, CB, gz, t, K, n);
         }
     } else {  // here n_r <= nrcap, so every run was stored
         run_starts(r, nr, true);
@@ -896,36 +973,44 @@ __host__ __device__ inline TabSpec table_spec(const DevParams &p)
     return t;
 }
 
-// shared memory: [table float2 (2K+2)] [g scratch double (K+1)] [g float (2K+1)] [per-warp arrays]
-__host__ __device__ inline size_t rle_table_bytes(int K)
+// shared memory: [tab float2 (2K+2)] [gtab float (2K+1)] [gz float 4 (conv_quads + 1)] [per-warp arrays]
+__host__ __device__ inline size_t rle_gz_at(int K)
 {
     return ((size_t)(2 * K + 2) * sizeof(float2) + (size_t)(2 * K + 1) * sizeof(float) + 15) & ~(size_t)15;
 }
+__host__ __device__ inline size_t rle_table_bytes(int K) { return rle_gz_at(K) + 16 * (size_t)(conv_quads(K) + 1); }
 
-// Shared-memory layout of the RLE evaluation kernels: the block's kernel table, then each warp's
-// kArraysRLE arrays of `stride` floats.
+// Shared-memory layout of the RLE evaluation kernels: the block's kernel table, then each warp's arrays.
 struct RleBlock {
     TabSpec ts;
     float2 *tab;
-    float *gtab;
+    float *gtab, *gz;
     float *base;
 };
 
-__device__ __forceinline__ RleBlock rle_block(unsigned char *smem_raw, const DevParams &p, const RleTable &t,
-                                              int warp_floats)
+// the tables at the front of the block's shared memory, loaded
+__device__ __forceinline__ RleBlock rle_tables(unsigned char *smem_raw, const DevParams &p, const RleTable &t, bool load)
 {
     RleBlock rb;
     rb.ts = table_spec(p);
     rb.tab = (float2 *)smem_raw;
     rb.gtab = (float *)(smem_raw + (size_t)(2 * rb.ts.K + 2) * sizeof(float2));
-    load_table(rb.tab, rb.gtab, rb.ts.K, t);
+    rb.gz = (float *)(smem_raw + rle_gz_at(rb.ts.K));
+    if (load) load_table(rb.tab, rb.gtab, rb.gz, rb.ts.K, t);
+    return rb;
+}
+
+__device__ __forceinline__ RleBlock rle_block(unsigned char *smem_raw, const DevParams &p, const RleTable &t,
+                                              int warp_floats)
+{
+    RleBlock rb = rle_tables(smem_raw, p, t, true);
     rb.base = (float *)(smem_raw + rle_table_bytes(rb.ts.K)) + (size_t)(threadIdx.x >> 5) * warp_floats;
     return rb;
 }
 
 // sampling, encoding and evaluation of one 3D ray (= pose * R + r), fused layout; WIDE: the batch
 // has more than 2^31 - 1 rays (64-bit index division), else a 32-bit one
-template <int MODE, bool WIDE>
+template <int MODE, int CPL, bool WIDE>
 __device__ __forceinline__ void eval_ray_3d(const Vox3D &vx, const DevParams &p, const RleBlock &rb, const RleTable &t,
                                             long long ray, float *__restrict__ out, int32_t *__restrict__ nruns)
 {
@@ -938,8 +1023,8 @@ __device__ __forceinline__ void eval_ray_3d(const Vox3D &vx, const DevParams &p,
         ri = (int)((unsigned)ray - (unsigned)pi * (unsigned)vx.R);
     }
     int nr = 0;
-    const float I = ray_mi_fused<MODE>(vx.vox, vx.X, vx.Y, vx.Z, vx.poses + 12 * (size_t)pi, vx.dirs + 3 * (size_t)ri, p.nmax,
-                                 p, rb.tab, rb.gtab, t, rb.ts.K, rb.base, nruns ? &nr : nullptr);
+    const float I = ray_mi_fused<MODE, CPL>(vx.vox, vx.X, vx.Y, vx.Z, vx.poses + 12 * (size_t)pi, vx.dirs + 3 * (size_t)ri, p.nmax,
+                                 p, rb.tab, rb.gtab, rb.gz, t, rb.ts.K, rb.base, nruns ? &nr : nullptr);
     if (lane_id() == 0) {
         out[ray] = I;
         if (nruns) nruns[ray] = nr;
@@ -978,7 +1063,7 @@ __device__ __forceinline__ void eval_ray_rle(const int32_t *__restrict__ off, co
         __syncwarp();
         return;
     }
-    const float I = ray_mi(rb.base, stride, nr, p, rb.tab, rb.gtab, t, rb.ts.K, false);
+    const float I = ray_mi(rb.base, stride, nr, p, rb.tab, rb.gtab, rb.gz, t, rb.ts.K, false);
     if (lane == 0) out[ray] = I;
     __syncwarp();
 }

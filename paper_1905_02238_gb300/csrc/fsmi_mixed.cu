@@ -24,7 +24,8 @@ __host__ __device__ constexpr int mix_bound(int c)
 static_assert(kMixBuckets <= 32, "the plan warp keeps one class per lane");
 // which kinds a launch of k_eval_mixed takes: both (the single launch), or one class's kind, 3D with
 // the evaluation path its variant uses (as fsmi_eval_3d compiles one kernel per path)
-enum { kMixAny = 0, kMix2D = 1, kMix3DOther = 2, kMix3DThm5 = 3 };
+enum { kMixAny = 0, kMix2D = 1, kMix3D = 2 };  // kMix3D + ray3d_mode: 3D on that path; + kMixShort: short rays
+constexpr int kMixShort = 16;
 
 // the set holding item i (sets sorted by out_offset), or -1
 __device__ __forceinline__ int mixed_set_of(const fsmi_set *sets, int nsets, long long i)
@@ -120,8 +121,8 @@ __device__ __forceinline__ int mixed_class(const fsmi_set &st, const MixedSrc &s
         if (!src.has3d || !(st.max_range >= 1.0f && st.max_range <= (float)p3.nmax)) return -1;
         if (st.volume < 0 || st.volume >= src.nvol) return -1;
         if ((long long)st.pose_offset + st.npose > src.P3 || (long long)st.dir_offset + st.ndir > src.R3) return -1;
-        int c = 0;  // by the range itself: a class launch takes ranges up to its bound (and its nmax)
-        while (c < kMixClasses - 1 && st.max_range > (float)mix_bound(c)) ++c;
+        int c = 0;  // by the virtual cells per ray: a class launch takes rays up to its bound (and its nmax)
+        while (c < kMixClasses - 1 && (int)st.max_range > mix_bound(c)) ++c;
         return kMixClasses + c;
     }
     return -1;
@@ -220,11 +221,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4)
     }
     if (nloc <= 0) return;  // a class without sets
     // block: the RLE kernel table of the 3D parameters; then each warp's arrays, used by either kind
-    RleBlock rb;
-    rb.ts = table_spec(p3);
-    rb.tab = (float2 *)smem_raw;
-    rb.gtab = (float *)(smem_raw + (size_t)(2 * rb.ts.K + 2) * sizeof(float2));
-    if (src.has3d) load_table(rb.tab, rb.gtab, rb.ts.K, tbl);
+    RleBlock rb = rle_tables(smem_raw, p3, tbl, src.has3d);
     const int per_warp = max(warp_floats_2d(stride2), ray3d_warp_floats(p3));  // then the set cache
     float *base = (float *)(smem_raw + rle_table_bytes(rb.ts.K)) + (size_t)(threadIdx.x >> 5) * (per_warp + kSetCacheFloats);
     rb.base = base;
@@ -314,9 +311,9 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4)
                     bad = FSMI_STATUS_BEAM_OVERFLOW;
                 }
             } else {
-                constexpr int kMode = KIND == kMix3DThm5 ? kRay3dThm5 : kRay3dOther;
-                I = ray_mi_fused<kMode>(cc->vox, cc->X, cc->Y, cc->Z, cc->pose + 12 * kp, cc->dir + 3 * kd, cc->nsamp, p3,
-                                        rb.tab, rb.gtab, tbl, rb.ts.K, base, nullptr);
+                constexpr bool kShort = KIND >= kMixShort;
+                I = ray_mi_fused<KIND - kMix3D - (kShort ? kMixShort : 0), kShort ? 2 : 4>(cc->vox, cc->X, cc->Y, cc->Z, cc->pose + 12 * kp, cc->dir + 3 * kd, cc->nsamp, p3,
+                                        rb.tab, rb.gtab, rb.gz, tbl, rb.ts.K, base, nullptr);
             }
             __syncwarp();
             if (lane == 0) {
@@ -359,8 +356,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4)
         } else if (ok && st.kind == FSMI_SET_3D && src.has3d && pi < src.P3 && di < src.R3 && st.volume >= 0 &&
                    st.volume < src.nvol && st.max_range >= 1.0f && st.max_range <= (float)p3.nmax) {
             const fsmi_volume v = src.vols[st.volume];
-            I = ray_mi_fused<kRay3dAny>(v.vox, v.X, v.Y, v.Z, src.poses3 + 12 * pi, src.dirs3 + 3 * di, (int)st.max_range,
-                                        p3, rb.tab, rb.gtab, tbl, rb.ts.K, base, nullptr);
+            I = ray_mi_fused<kRay3dAny, 0>(v.vox, v.X, v.Y, v.Z, src.poses3 + 12 * pi, src.dirs3 + 3 * di, (int)st.max_range,
+                                        p3, rb.tab, rb.gtab, rb.gz, tbl, rb.ts.K, base, nullptr);
         } else {
             bad = FSMI_STATUS_BAD_BEAM;  // a malformed descriptor is never used to index
         }
@@ -379,7 +376,7 @@ cudaError_t launch_mixed_variant(const MixedSrc &src, const DevParams &p2, const
                                  cudaStream_t s, const unsigned char *plan = nullptr, int bucket = -1)
 {
     // a 3D class runs under the RLE family's schedule, like fsmi_eval_3d; everything else the 2D one
-    const Schedule &sc = current_schedule(KIND == kMix3DOther || KIND == kMix3DThm5 ? FSMI_KIND_RLE : FSMI_KIND_2D);
+    const Schedule &sc = current_schedule(KIND >= kMix3D ? FSMI_KIND_RLE : FSMI_KIND_2D);
     const int stride2 = stride_2d(p2.nmax);
     const int stride3 = ((p3.nmax + 2 * p3.K + 4) + 3) & ~3;
     const size_t per_warp = ((size_t)max(warp_floats_2d(stride2), ray3d_warp_floats(p3)) + kSetCacheFloats) * sizeof(float);
@@ -442,11 +439,19 @@ cudaError_t launch_mixed_planned(const MixedSrc &src, const DevParams &d2, const
             p.nmax = min(mix_bound(c), d3.nmax);
             MixedSrc sc3 = src;
             sc3.has2d = false;
-            // (a 3D class holds no 2D path: one instantiation whatever the 2D variant)
-            e = thm5_of(p) ? launch_mixed_variant<FSMI_EXACT, kMix3DThm5>(sc3, n2, p, nitems, out, times, status, queue,
-                                                                         s, plan, kMixClasses + c)
-                           : launch_mixed_variant<FSMI_EXACT, kMix3DOther>(sc3, n2, p, nitems, out, times, status, queue,
-                                                                          s, plan, kMixClasses + c);
+            // (a 3D class holds no 2D path: one instantiation whatever the 2D variant; the classes' bounds
+            // include kShortRay, so a class holds short rays only or none)
+            auto go = [&](auto mode) {
+                constexpr int K3 = kMix3D + decltype(mode)::value;
+                return p.nmax > kShortRay ? launch_mixed_variant<FSMI_EXACT, K3>(sc3, n2, p, nitems, out, times, status,
+                                                                               queue, s, plan, kMixClasses + c)
+                                          : launch_mixed_variant<FSMI_EXACT, K3 + kMixShort>(
+                                                sc3, n2, p, nitems, out, times, status, queue, s, plan, kMixClasses + c);
+            };
+            const int mode = ray3d_mode(p);
+            e = mode == kRay3dThm5    ? go(std::integral_constant<int, kRay3dThm5>{})
+                : mode == kRay3dFixed ? go(std::integral_constant<int, kRay3dFixed>{})
+                                      : go(std::integral_constant<int, kRay3dOther>{});
             if (e != cudaSuccess) return e;
         }
     }
@@ -498,6 +503,15 @@ static cudaError_t prepare_mixed_var()
     return e;
 }
 
+template <int MODE>
+static cudaError_t prepare_mixed_3d()
+{
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, k_eval_mixed<FSMI_EXACT, kMix3D + MODE>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_mixed<FSMI_EXACT, kMix3D + MODE + kMixShort>);
+    return e;
+}
+
 size_t mixed_plan_bytes(int nsets)
 {
     return sizeof(MixedPlan) + plan_list_bytes(nsets) + (size_t)kMixBuckets * (nsets + 1) * sizeof(long long);
@@ -507,8 +521,9 @@ cudaError_t prepare_mixed()
 {
     cudaFuncAttributes a;
     cudaError_t e = cudaFuncGetAttributes(&a, k_mixed_plan);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_mixed<FSMI_EXACT, kMix3DOther>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_mixed<FSMI_EXACT, kMix3DThm5>);
+    if (e == cudaSuccess) e = prepare_mixed_3d<kRay3dThm5>();
+    if (e == cudaSuccess) e = prepare_mixed_3d<kRay3dFixed>();
+    if (e == cudaSuccess) e = prepare_mixed_3d<kRay3dOther>();
     if (e == cudaSuccess) e = prepare_mixed_var<kExactMass3>();
     if (e == cudaSuccess) e = prepare_mixed_var<kExactMass4>();
     if (e == cudaSuccess) e = prepare_mixed_var<FSMI_EXACT>();

@@ -6,17 +6,26 @@
 
 namespace fsmi {
 
-// MODE: kRay3dThm5 for Theorem 5's sub-blocks, kRay3dOther for every other variant (the launcher
-// picks by thm5_of(p)), so that each kernel holds only the paths it can take; WIDE for batches of
-// more than 2^31 - 1 rays (a 64-bit ray index division, which costs the others registers).
-template <int MODE, bool WIDE>
+// MODE, CPL: the paths of the call's variant and radius and its rays' length (the launcher picks them by
+// ray3d_mode(p) and kShortRay), so that each kernel holds only what it can take; WIDE for batches of more than
+// 2^31 - 1 rays (a 64-bit ray index division, which costs the others registers).
+template <int MODE, int CPL, bool WIDE>
 __global__ void __launch_bounds__(kMaxWarps * 32)
     k_eval_3d(Vox3D vx, DevParams p, const __grid_constant__ RleTable tbl, long long nrays, int warp_floats,
               float *__restrict__ out, int32_t *__restrict__ nruns, unsigned long long *queue, int chunk)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const RleBlock rb = rle_block(smem_raw, p, tbl, warp_floats);
-    for_each_item(nrays, queue, chunk, [&](long long ray) { eval_ray_3d<MODE, WIDE>(vx, p, rb, tbl, ray, out, nruns); });
+    for_each_item(nrays, queue, chunk, [&](long long ray) { eval_ray_3d<MODE, CPL, WIDE>(vx, p, rb, tbl, ray, out, nruns); });
+}
+
+using Eval3DKernel = void (*)(Vox3D, DevParams, const RleTable, long long, int, float *, int32_t *, unsigned long long *, int);
+
+template <int MODE>
+static Eval3DKernel eval_3d_kernel(const DevParams &p, bool wide)
+{
+    if (wide) return k_eval_3d<MODE, 0, true>;
+    return p.nmax > kShortRay ? k_eval_3d<MODE, 4, false> : k_eval_3d<MODE, 2, false>;
 }
 
 __global__ void __launch_bounds__(kMaxWarps * 32)
@@ -227,8 +236,10 @@ cudaError_t launch_eval_3d(const Vox3D &v, const DevParams &p, float *out, int32
     const size_t smem = rle_table_bytes(p.K) + (size_t)wpb * per_warp;
     WarpGrid g;
     const bool wide = nrays > 0x7fffffffLL;
-    auto kern = thm5_of(p) ? (wide ? k_eval_3d<kRay3dThm5, true> : k_eval_3d<kRay3dThm5, false>)
-                           : (wide ? k_eval_3d<kRay3dOther, true> : k_eval_3d<kRay3dOther, false>);
+    const int mode = ray3d_mode(p);
+    const Eval3DKernel kern = mode == kRay3dThm5    ? eval_3d_kernel<kRay3dThm5>(p, wide)
+                              : mode == kRay3dFixed ? eval_3d_kernel<kRay3dFixed>(p, wide)
+                                                    : eval_3d_kernel<kRay3dOther>(p, wide);
     cudaError_t e = warp_grid((const void *)kern, nrays, wpb, smem, sc.blocks_per_sm, g);
     if (e == cudaSuccess && g.one_each) queue = nullptr;  // nothing to balance
     if (e == cudaSuccess) e = reset_queue(queue, s);
@@ -307,14 +318,23 @@ int32_t *g_scratch_ptr[64];
 
 cudaError_t encode_scratch_ptr(int32_t **ptr);
 
+template <int MODE>
+static cudaError_t prepare_eval_3d()
+{
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, k_eval_3d<MODE, 4, false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_3d<MODE, 2, false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_3d<MODE, 0, true>);
+    return e;
+}
+
 // Loads every RLE kernel on the current device (a kernel's first use loads it lazily).
 cudaError_t prepare_rle()
 {
     cudaFuncAttributes a;
-    cudaError_t e = cudaFuncGetAttributes(&a, k_eval_3d<kRay3dThm5, false>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_3d<kRay3dOther, false>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_3d<kRay3dThm5, true>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_3d<kRay3dOther, true>);
+    cudaError_t e = prepare_eval_3d<kRay3dThm5>();
+    if (e == cudaSuccess) e = prepare_eval_3d<kRay3dFixed>();
+    if (e == cudaSuccess) e = prepare_eval_3d<kRay3dOther>();
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_rle);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_rle_count);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_rle_write);
