@@ -283,7 +283,7 @@ struct CellScan {
 };
 
 // cells per lane: rays of at most 64 samples go in one block of 64, so that half the lanes' work is not idle
-__host__ __device__ constexpr int kShortRay = 64;
+constexpr int kShortRay = 64;
 
 // One block of 32 CPL cells (CPL = 4, or 2 on short rays): o of this lane's cells i0 .. i0 + CPL - 1 (zero from
 // the ray's end on); stores P in CP and C in CB where i0 < n.
@@ -399,8 +399,8 @@ __device__ __forceinline__ float band_conv_k(const float *CP, const float *CB, c
 }
 
 // The same for any radius: four outputs per lane, and per group of four inputs one 16-byte load of C and one
-// (the same for all lanes) of the zero-padded kernel, for 16 products. (A load of C and one of g per product:
-// BANDANY_NOTE.)
+// (the same for all lanes) of the zero-padded kernel, for 16 products, where one of each went with every
+// product before.
 __device__ __forceinline__ float band_conv_any(const float *CP, const float *CB, const float *gz, int K, int n)
 {
     const int quads = conv_quads(K);

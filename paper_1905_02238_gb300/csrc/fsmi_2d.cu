@@ -14,7 +14,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, FSMI_MIN_BLOCKS_2D)
               unsigned long long *queue, int chunk)
 {
     extern __shared__ float smem[];
-    const int lane = lane_id(), warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    const int warp = threadIdx.x >> 5;
     float *sl, *sc, *sp, *sx;
     carve_2d(smem + (size_t)warp * warp_floats_2d(stride), stride, sl, sc, sp, sx);
     for_each_item(nbeams, queue, chunk,
