@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(128)
 __global__ void k_map_gains(const float *__restrict__ map, long long ncell, float docc, float demp,
                             float4 *__restrict__ gains)
 {
+    launch_dependents();
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < ncell; i += (long long)gridDim.x * blockDim.x) {
         const float o = __ldg(map + i);
         gains[i] = make_float4(o, cell_gain(docc, o), cell_gain(demp, o), 0.0f);

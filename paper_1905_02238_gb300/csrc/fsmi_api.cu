@@ -592,12 +592,9 @@ fsmi_status fsmi_eval_mixed(const float *map, int W, int H, const int32_t *poses
     unsigned char *plan = (ws && aligned16(ws) && ws_bytes >= plan_at + mixed_plan_bytes(nsets))
                               ? (unsigned char *)ws + plan_at
                               : nullptr;
-    cudaError_t e = cudaSuccess;
-    if (gains) e = map_gains(map, W, H, d2, gains, s);
-    if (e == cudaSuccess)
-        e = launch_eval_mixed(map, W, H, gains, poses2, P2, dirs2, B2, prm2 ? &d2 : nullptr, vols, nvol, poses3, P3,
-                              dirs3, R3, prm3 ? &d3 : nullptr, sets, nsets, nitems, out, times, sp,
-                              queue_of(FSMI_KIND_2D, ws, ws_bytes), plan, s);
+    cudaError_t e = launch_eval_mixed(map, W, H, gains, poses2, P2, dirs2, B2, prm2 ? &d2 : nullptr, vols, nvol, poses3, P3,
+                                      dirs3, R3, prm3 ? &d3 : nullptr, sets, nsets, nitems, out, times, sp,
+                                      queue_of(FSMI_KIND_2D, ws, ws_bytes), plan, s);
     return e == cudaSuccess ? FSMI_OK : cuda_fail(e);
 }
 

@@ -187,6 +187,21 @@ __device__ __forceinline__ void for_each_item(long long n, unsigned long long *q
     }
 }
 
+// Lets an early launch behind this one start once every block has got here.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Waits for the end of the launch before this one and for its writes (returns at once on a launch that was not
+// early). The last statement of a kernel's block 0 makes the kernel end no earlier than the one before it.
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+struct EndAfterPrevious {
+    bool on;
+    __device__ __forceinline__ ~EndAfterPrevious()
+    {
+        if (on) wait_previous();
+    }
+};
+
 __device__ __forceinline__ void set_status(int *status, int bits)
 {
     if (status) atomicOr(status, bits);

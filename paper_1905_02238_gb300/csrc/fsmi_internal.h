@@ -122,6 +122,25 @@ cudaError_t launch_rle_encode_3d_static(const Vox3D &v, const DevParams &p, int3
 
 int sm_count();
 
+// Launches kern; `early`: its blocks may start as soon as every block of the launch before it in the stream, a
+// kernel of the same call that says launch_dependents(), has said so or ended, instead of after its end.
+template <class... P, class... A>
+cudaError_t launch_kernel(bool early, void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
+                          A &&...args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // Resident blocks per SM of `kern` with `threads` threads and `smem` bytes of dynamic shared memory on the
 // current device, its dynamic shared memory limit raised to the device's maximum. Looked up once per
 // kernel, block size and device and remembered per host thread (the attribute and occupancy calls were 4 of the
@@ -145,8 +164,8 @@ cudaError_t launch_update_map_2d(float *map, int W, int H, const int32_t *poses,
                                  uint32_t *counts, int *status, cudaStream_t s);
 cudaError_t prepare_explore();
 
-// mixed 2D / 3D candidate sets in one launch (fsmi_mixed.cu)
-cudaError_t launch_eval_mixed(const float *map, int W, int H, const float4 *gains, const int32_t *poses2, int P2,
+// mixed 2D / 3D candidate sets in one launch (fsmi_mixed.cu); fills gains (null: none)
+cudaError_t launch_eval_mixed(const float *map, int W, int H, float4 *gains, const int32_t *poses2, int P2,
                               const int32_t *dirs2, int B2, const DevParams *p2, const fsmi_volume *vols, int nvol,
                               const int32_t *poses3, int P3, const int32_t *dirs3, int R3, const DevParams *p3,
                               const fsmi_set *sets, int nsets, long long nitems, float *out, unsigned long long *times,
