@@ -506,9 +506,18 @@ struct StoreMask {  // out[m][n] = acc [mask[m][n] > 0]
     }
 };
 
-// K of fc1's forward product in quarters: 4 times the blocks (128 for a batch of 4096), and a quarter of the
-// additions in each of the tensor cores' accumulators, which round toward zero
-constexpr int kFc1Splits = 4;
+// Splits of K in fc1's forward product, for two 64-row by 64-column tiles per SM at least and 256 of K per split: 2
+// for a batch of 4096, whose 256 blocks of 128 x 64 run in one wave. Each sum's value depends on the split (the
+// tensor cores' accumulators round toward zero), so this rule is part of the results: a sum next to
+// zero decides whether a hidden unit's gradient counts.
+constexpr int kFc1Splits = 4;  // at most
+int fc1_forward_splits(int N)
+{
+    const long long tiles = (long long)(N + 63) / 64 * (kHid / 64);
+    int splits = 1;
+    while (splits < kFc1Splits && tiles * splits < 2LL * sm_count()) splits *= 2;
+    return splits;
+}
 
 // splits of the batch in fc1's weight gradient (32 output blocks): a function of N alone, so that a step's
 // sums are in the same order on every run
@@ -540,7 +549,7 @@ __global__ void k_split_reduce(int E, int splits, const float *__restrict__ part
 
 // ---- head -------------------------------------------------------------------------------------------
 //
-// z4[n][j] = b4[j] + the sums of fc1's product over the quarters of K (part1 [kFc1Splits][N][256]),
+// z4[n][j] = b4[j] + the sums of fc1's product over the splits of K (part1 [splits][N][256]),
 // pred[n] = b5 + sum_j W5[j] relu(z4[n][j]) and, with targets, d = pred - y, dpred = 2 d / N,
 // dz4[n][j] = dpred W5[j] [z4 > 0] as two BF16 terms (dz, N * 256 elements apart) and the block's sums over its
 // rows of dpred relu(z4) (gW5), dz4 (gb4), dpred (gb5) and d^2 (loss) into part[block][514]. A
@@ -549,7 +558,7 @@ constexpr int kHeadRows = 32, kHeadOut = 2 * kHid + 2;
 __global__ void __launch_bounds__(256)
     k_head(const float *__restrict__ part1, const bf16 *__restrict__ w, const float *__restrict__ params,
            const float *__restrict__ y, int N, float *__restrict__ z4, float *__restrict__ pred, bf16 *__restrict__ dz,
-           float *__restrict__ part)
+           float *__restrict__ part, int splits)
 {
     __shared__ float sum[8][kHeadOut];
     const int lane = lane_id(), wp = threadIdx.x >> 5;
@@ -569,9 +578,11 @@ __global__ void __launch_bounds__(256)
             const size_t o = (size_t)n * kHid + 128 * q + 4 * lane;
             float4 v[kFc1Splits];
 #pragma unroll
-            for (int k = 0; k < kFc1Splits; ++k) v[k] = *reinterpret_cast<const float4 *>(part1 + (size_t)k * N * kHid + o);
+            for (int k = 0; k < kFc1Splits; ++k)
+                if (k < splits) v[k] = *reinterpret_cast<const float4 *>(part1 + (size_t)k * N * kHid + o);
 #pragma unroll
-            for (int k = 1; k < kFc1Splits; ++k) v[0] = make_float4(v[0].x + v[k].x, v[0].y + v[k].y, v[0].z + v[k].z, v[0].w + v[k].w);
+            for (int k = 1; k < kFc1Splits; ++k)
+                if (k < splits) v[0] = make_float4(v[0].x + v[k].x, v[0].y + v[k].y, v[0].z + v[k].z, v[0].w + v[k].w);
             z[4 * q] = v[0].x + b4[4 * q];
             z[4 * q + 1] = v[0].y + b4[4 * q + 1];
             z[4 * q + 2] = v[0].z + b4[4 * q + 2];
@@ -1496,10 +1507,11 @@ cudaError_t launch_surrogate_loss_grad(const float *params, const void *wbf16, c
     k_convs_fwd<<<grid_cap(((long long)N + kFwdWarps - 1) / kFwdWarps), kFwdWarps * 32, 0, s>>>(N, (const unsigned *)x, w, params, z1,
                                                                                               z2, z3, h, n * kFlat);
     FSMI_TRY(cudaGetLastError());
-    float *part1 = dz3;  // fc1's sums by quarters of K, added by the head
-    FSMI_TRY(gemm_terms<3, 1, false, false>(N, kHid, kFlat, kFc1Splits, h, n * kFlat, kFlat, w4, 0, kFlat,
+    float *part1 = dz3;  // fc1's sums by splits of K, added by the head
+    const int fsplits = fc1_forward_splits(N);
+    FSMI_TRY(gemm_terms<3, 1, false, false>(N, kHid, kFlat, fsplits, h, n * kFlat, kFlat, w4, 0, kFlat,
                                             StorePart{part1, N, kHid}, s));
-    k_head<<<head_blocks, 256, 0, s>>>(part1, w, params, y, N, z4, pred_out ? pred_out : pred_ws, dz4, part_h);
+    k_head<<<head_blocks, 256, 0, s>>>(part1, w, params, y, N, z4, pred_out ? pred_out : pred_ws, dz4, part_h, fsplits);
     FSMI_TRY(cudaGetLastError());
     if (!y) return cudaSuccess;
     // backward: fc1's weights gW4[j][i] = sum_n dz4[n][j] relu(z3)[n][i] and data dz3 = (dz4 W4) [z3 > 0]
