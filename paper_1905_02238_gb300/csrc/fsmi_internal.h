@@ -125,14 +125,14 @@ int sm_count();
 // Launches kern; `early`: its blocks may start as soon as every block of the launch before it in the stream, a
 // kernel of the same call that says launch_dependents(), has said so or ended, instead of after its end.
 template <class... P, class... A>
-cudaError_t launch_kernel(bool early, void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
+cudaError_t launch_kernel(bool early, void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
                           A &&...args)
 {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
