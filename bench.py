@@ -39,18 +39,19 @@ FMA_LANES_PER_SM_CLK = 128  # FP32 FMA-pipe lane operations per SM per clock (4 
 EX2_PER_SM_CLK = 32  # SFU ex2.approx results per SM per clock (csrc/pipe_probe.cu measured 31.8)
 RCP_PER_SM_CLK = 16  # SFU rcp.approx results per SM per clock (measured 15.95)
 SFU_CLK_PER_TERM = 1.0 / EX2_PER_SM_CLK + 1.0 / RCP_PER_SM_CLK  # one ex2 and one rcp per tail term
-OPS_PER_TERM = 10  # FP32 FMA-pipe operations per boundary tail term (csrc/gauss_tail.cuh): distance,
-#                    square, 1 + p|d|, 4 Horner FMAs, two products, accumulate
+MASS_OPS_PER_TERM = 7  # FP32 FMA-pipe operations per cell-mass term of the exact kernel (csrc/cell_mass.cuh): distance,
+#                        square, weight, 3 Horner FMAs, accumulate (and one ex2)
 TAIL_CUT = 4.81  # scaled half-width of the exact kernel's default window (csrc/eval2d.cuh)
 
 # DRAM bytes (read + write) per launch of the 2D kernel on the benchmark workload (exact; the
 # Approx and Uniform legs by name), from an ncu capture of one full-size launch each
 # (dram__bytes_read.sum + dram__bytes_write.sum), valid only for the kernel sources whose hash is
 # recorded with them; reported as null once those sources change.
-TRAFFIC = {"sources_sha1": "d04b34a3db90ae157f6964bfca6621c5e603dcaa", "bytes_per_launch": 111.34e6,
-           "approx_fsmi_delta6": 82.83e6, "uniform_fsmi_h4": 83.00e6}
+TRAFFIC = {"sources_sha1": "52f8249a4fb04430fb57f54504022df6889b266c", "bytes_per_launch": 82.68e6,
+           "approx_fsmi_delta6": 93.93e6, "uniform_fsmi_h4": 82.52e6}
 KERNEL_SOURCES = ["paper_1905_02238_gb300/csrc/fsmi_2d.cu", "paper_1905_02238_gb300/csrc/eval2d.cuh",
                   "paper_1905_02238_gb300/csrc/dda2d.cuh", "paper_1905_02238_gb300/csrc/gauss_tail.cuh",
+                  "paper_1905_02238_gb300/csrc/cell_mass.cuh",
                   "paper_1905_02238_gb300/csrc/fsmi_device.cuh"]
 
 
@@ -58,8 +59,8 @@ KERNEL_SOURCES = ["paper_1905_02238_gb300/csrc/fsmi_2d.cu", "paper_1905_02238_gb
 # ncu capture each (valid for the sources hashed with them, like TRAFFIC)
 KERNEL_SOURCES_3D = ["paper_1905_02238_gb300/csrc/fsmi_rle.cu", "paper_1905_02238_gb300/csrc/evalrle.cuh",
                      "paper_1905_02238_gb300/csrc/fsmi_device.cuh"]
-TRAFFIC_3D = {"sources_sha1": "8140517dbdd4473d1c65def9bad5f71ddea9e91f", "fsmi_rle_3d": 563.77e6, "approx_fsmi_rle_3d_delta6": 566.51e6,
-              "approx_fsmi_rle_3d_delta6_band": 563.41e6, "uniform_fsmi_rle_3d_h4": 563.24e6}
+TRAFFIC_3D = {"sources_sha1": "3c136d66d7502086606b7a6ba8592c4e3100799f", "fsmi_rle_3d": 567.60e6, "approx_fsmi_rle_3d_delta6": 568.81e6,
+              "approx_fsmi_rle_3d_delta6_band": 568.19e6, "uniform_fsmi_rle_3d_h4": 568.38e6}
 
 
 def kernel_sources_sha1(files=None) -> str:
@@ -981,8 +982,8 @@ def run_fsmi(args):
         sm_max = clocks.get("sm_max_mhz") or peaks.get("sm_max_mhz") or 2070.0
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         peak_ops = sms * FMA_LANES_PER_SM_CLK * sm_max * 1e6  # FMA-pipe ops/s at the maximum SM clock
-        achieved_ops = terms * OPS_PER_TERM / (ms * 1e-3)
-        peak_terms = sms * sm_max * 1e6 / SFU_CLK_PER_TERM  # tail terms/s the SFU allows
+        achieved_ops = terms * MASS_OPS_PER_TERM / (ms * 1e-3)
+        peak_terms = peak_ops / MASS_OPS_PER_TERM  # cell-mass terms/s the FMA pipe allows
         achieved_terms = terms / (ms * 1e-3)
         traffic = TRAFFIC["bytes_per_launch"] if TRAFFIC["sources_sha1"] == kernel_sources_sha1() else None
         line = {
@@ -998,13 +999,14 @@ def run_fsmi(args):
                                        for c, t in zip(cands, tune_ms)},
                        "parallelism": f"dp{ws} (poses sharded, map replicated)"},
             "roofline": {"bound": "alu", "achieved": achieved_terms / 1e12, "peak": peak_terms / 1e12,
-                         "unit": "T tail-terms/s (SFU)", "frac": achieved_terms / peak_terms, "traffic": traffic,
+                         "unit": "T pair-terms/s (FP32 FMA)", "frac": achieved_terms / peak_terms, "traffic": traffic,
                          "kernel": "k_eval_2d<EXACT,map>",
                          "fma_frac": achieved_ops / peak_ops,
-                         "model": f"{terms:.4g} evaluated tail terms per launch, each one ex2 and one rcp on the "
-                                  f"SFU ({EX2_PER_SM_CLK} and {RCP_PER_SM_CLK} per SM per clock: the binding pipe) "
-                                  f"and {OPS_PER_TERM} FMA-pipe ops ({FMA_LANES_PER_SM_CLK} lanes per SM per clock; "
-                                  f"fma_frac); peak = {sms} SMs x {sm_max:.0f} MHz"},
+                         "sfu_frac": achieved_terms / (sms * sm_max * 1e6 * EX2_PER_SM_CLK),
+                         "model": f"{terms:.4g} terms within the window per launch, each {MASS_OPS_PER_TERM} FMA-pipe ops "
+                                  f"({FMA_LANES_PER_SM_CLK} lanes per SM per clock: the binding pipe; fma_frac) and one ex2 "
+                                  f"on the SFU ({EX2_PER_SM_CLK} per SM per clock; sfu_frac); peak = {sms} SMs x "
+                                  f"{sm_max:.0f} MHz"},
             "clocks": clocks,
             "e2e": {"value": whole_job_rate(P * B, ws, e2e_s), "unit": "beams/s", "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h,
@@ -1017,7 +1019,7 @@ def run_fsmi(args):
             exact_out = out.cpu().numpy()  # the timed steps' result, before the context runs reuse `out`
             line["pipe_rates"] = pipe_rates_leg(dev)
             line["variants"] = other_variants(g, p, d, out, cells=cells, terms=terms, band=band,
-                                              peak_terms=peak_terms, pipes=line["pipe_rates"], sm_mhz=sm_max)
+                                              peak_terms=sms * sm_max * 1e6 / SFU_CLK_PER_TERM, pipes=line["pipe_rates"], sm_mhz=sm_max)
             fw = line["variants"]["exact_fsmi_full_window"]
             # beside the headline: the same batch with every non-zero term of Theorem 1's n(n+1) sum,
             # bit-identical to the full sweep (FSMI_FLAG_FULL_WINDOW); 5 back-to-back calls, no graph
