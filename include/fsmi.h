@@ -85,10 +85,13 @@ typedef struct {
     int flags;          /* FSMI_FLAG_* bits, 0 by default */
 } fsmi_params;
 
-/* Exact 2D FSMI evaluates, for each first-hit cell j, the terms of Theorem 1's pair sum within about
- * 5.7 sigma of the cell's centre: what lies beyond on one side weighs less than 2^-24 of the largest
- * C_k, so the MI differs from the full n(n+1) sweep by about one FP32 rounding at most (not bit for
- * bit).
+/* Exact 2D FSMI on a grid evaluates, for each first-hit cell j, the terms C_k G_{k,j} of Theorem 1's pair sum
+ * whose cell k lies at most about 5.7 sigma before or 6.1 sigma after the centre of cell j: the Gaussian mass beyond
+ * is below 2^-27 before it and below 2^-31 after it, so what is left out weighs less than that share of the
+ * largest C_k on its side (C_k grows along a beam), and on occupancy maps the MI differs from the full
+ * n(n+1) sweep by less than one FP32 rounding (sigma up to 20 cells; not bit for bit). For sigma below one cell
+ * and for explicit beams the terms are those of the boundary form within 5.7 sigma on either side, what is left out
+ * below 2^-27 of its weight |C_m - C_{m-1}| each.
  * FSMI_FLAG_FULL_WINDOW widens the window to every term whose Gaussian tail is non-zero in FP32
  * (about 13.3 sigma; the tail underflows to exactly 0 beyond), which gives the full sweep's result
  * bit for bit; FSMI_FLAG_FULL_SWEEP evaluates all n(n+1) terms (both for verification and timing

@@ -399,11 +399,16 @@ __device__ __forceinline__ float approx_pairs_sum(const float2 *LW, const float 
 // A pair of terms costs 7 packed FP32 operations and two ex2 (14 FMA-pipe cycles and 8 SFU cycles per
 // warp at D = 3) where the boundary form costs 10 and two ex2 and two rcp (20 and 24).
 //
-// Windows: a cell whose centre lies beyond the cut adds at most its mass beyond that distance less
-// half its width; kMassCut plus half the widest cell leaves out at most 3e-8 on one side, half an
-// FP32 ulp. (FSMI_FLAG_FULL_WINDOW: kTailCut, beyond which 2^(-d^2) is exactly 0;
-// FSMI_FLAG_FULL_SWEEP: no cut. Both add the same non-zero terms in the same order.)
-constexpr float kMassCut = 4.58f;
+// Windows: a cell whose centre lies beyond a cut plus half its width holds, together with all the cells behind
+// it, less Gaussian mass than the tail at the cut. Its weight is C_k itself, a running sum that grows along the
+// beam, not the difference of two neighbours as in the boundary form, and what is left out has one sign;
+// so the cells after the first hit, whose C_k is the larger, need a wider cut than the boundary form's:
+// T(kMassCut) = 4.6e-10 < 2^-31; for those before it (C_k about C_j at most) T(kTailCutDefault) = 7.4e-9 < 2^-27
+// does. Largest relative change of a beam's MI, sigma 2 / 5 / 20, on the office map and on random cells: 1.2e-7 /
+// 2.1e-7 / 5.2e-7 with both cuts at 4.58, 1.5e-9 / 3.7e-9 / 7.6e-9 here for 6 % more terms and 5 % more time on the
+// 2048x2048 office batch (both cuts at 5.2: the same, 11 % more terms; 5.0: 3.7e-9 / 1.1e-8 / 2.8e-8, 9 %). (FSMI_FLAG_FULL_WINDOW: kTailCut, beyond which
+// 2^(-d^2) is exactly 0; FSMI_FLAG_FULL_SWEEP: no cut. Both add the same non-zero terms in the same order.)
+constexpr float kMassCut = 5.2f, kMassCutStep = kMassCut - kTailCutDefault;
 
 // Builds Tg in place over sl and the scratch array after it, from the top pair down (writing Tg[p]
 // overwrites l_4p .. l_4p+3, which only Tg[2p - 1], Tg[2p] and Tg[2p + 1] read: they lie higher, or
@@ -447,7 +452,8 @@ __device__ __forceinline__ void build_targets(float *sl, float *sp, int n, float
 // Exact sum. Sources in rounds of 64 while more than 32 remain, lane i the adjacent cells A = 2i and
 // B = A + 1 of the round, then one per lane. In every round all lanes run over the same number of
 // pairs below and above their own (the fewest that cover every window of the round, by coverage
-// trials from the previous round's counts), clamped to the beam.
+// trials from the previous round's counts), clamped to the beam. `cut` bounds the targets below a
+// source, cut - kMassCutStep those above it.
 template <int D>
 __device__ __forceinline__ float exact_mass_sum(const float4 *Tg, const float *sc, const float *sw, int n, bool e0, float cut)
 {
@@ -468,7 +474,7 @@ __device__ __forceinline__ float exact_mass_sum(const float4 *Tg, const float *s
         const int b = actB ? a + 1 : a;
         const int pa = a >> 1;
         const float xa = xq(a), xb = xq(b);
-        const float below = xa - cut, above = xb + cut;
+        const float below = xa - cut, above = xb + (cut - kMassCutStep);
         auto neg_ok = [&](int G) {
             const int m = 2 * (pa - G) - 1;
             return !act || m < mlo || xq(m) < below;
@@ -715,7 +721,7 @@ __device__ __forceinline__ float beam_sum(const DevParams &p, int n, float *sl, 
             build_targets(sl, sp, n, cs, e0 ? pe0 : 0.0f, mu0);
             const float4 *Tg = reinterpret_cast<const float4 *>(sl);
             float cut = fmaf(0.70710678f, cs, kMassCut);
-            if (p.flags & FSMI_FLAG_FULL_WINDOW) cut = kTailCut;
+            if (p.flags & FSMI_FLAG_FULL_WINDOW) cut = kTailCut + kMassCutStep;
             if (p.flags & FSMI_FLAG_FULL_SWEEP) cut = __int_as_float(0x7f800000);
             I = exact_mass_sum<VAR == kExactMass3 ? 3 : 4>(Tg, sc, sp, n, e0, cut);
         }
