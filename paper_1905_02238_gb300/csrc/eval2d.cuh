@@ -55,7 +55,9 @@ __device__ __forceinline__ void carve_2d(float *base, int stride, float *&sl, fl
 constexpr int kExactFullSweep = 3, kExactMass3 = 4, kExactMass4 = 5;
 __host__ __device__ constexpr bool mass_variant(int v) { return v == kExactMass3 || v == kExactMass4; }
 
-// The kernel variant of a call whose cells come from the grid (every width at most sqrt 2 cells).
+// The kernel variant of a call whose cells come from the grid (widths of at most sqrt 2 cells along unit vectors;
+// a beam along a shorter vector, whose cells are wider than the form's table covers, takes the boundary form by
+// itself, see beam_sum).
 // The exact sum takes the mass form (cell_mass.cuh) from sigma = 1 cell on; below that, and for
 // explicit beams, whose cells may be any width, the boundary form. Approx-FSMI stays in boundary form:
 // its band is too short to pay for the sources' polynomials (Delta = 3, 517 poses x 181 beams, R = 181.5:
@@ -527,6 +529,33 @@ __device__ __forceinline__ float exact_mass_sum(const float4 *Tg, const float *s
     return r;
 }
 
+// Widest cell (scaled) that the mass form's table of degree D covers: sqrt 2 cells at the smallest sigma of the
+// degree, and 1 / 1000 more for rounded direction vectors.
+template <int D>
+constexpr float kMassWidth = (float)(1.001 * kSqrtLog2e / (D == 3 ? kMassSigma3 : kMassSigma4));
+
+// The boundary form for a beam of a mass kernel whose cells are wider than that, all n (n + 1) terms: no beam
+// along a unit vector gets here, so it is kept small (a call of exact_pairs_sum costs the mass kernels' other
+// beams 44 bytes of spilled registers each).
+__device__ __forceinline__ float wide_beam_sum(const float *sl, const float *sc, const float *sp, int n, bool e0, float pe0,
+                                               float cs)
+{
+    float r = 0.0f;
+#pragma unroll 1
+    for (int j = lane_id() - (e0 ? 1 : 0); j < n; j += 32) {
+        const float mu = j < 0 ? sl[0] * cs - 0.5f * cs : 0.5f * (sl[j] * cs + sl[j + 1] * cs);
+        float acc = j < 0 ? 0.0f : sc[j], c = 0.0f;
+#pragma unroll 1
+        for (int m = 0; m <= n; ++m) {  // sc[n] = 0
+            const float dc = sc[m] - c, t = gauss_tail(sl[m] * cs - mu);
+            c = sc[m];
+            acc = fmaf(m <= j ? -dc : dc, t, acc);
+        }
+        r = fmaf(j < 0 ? pe0 : sp[j], acc, r);
+    }
+    return r;
+}
+
 // Uniform-FSMI (Algorithm 4) from D = inclusive prefix of C (sd), with Algorithm 4's clamps.
 __device__ __forceinline__ float uniform_sum(const float *sd, const float *sp, int n, bool e0, float pe0, int H,
                                              float inv_2h1)
@@ -585,12 +614,13 @@ __device__ __forceinline__ int traj_of(const int32_t *traj_off, int T, int p)
 // Cells of one beam on the map: traversal from `pose` along the sensor-frame direction (ux, uy)
 // up to rfix (Q16) / rend, then per cell o (sp), f(delta_occ, o) (sc), f(delta_emp, o) (sx) and
 // the entry distances (sl). With TRAJ, cells whose visit stamp is below `state` keep o but lose
-// their gains (Section 2.4). Returns n, or -1 if the beam has more than cap cells.
+// their gains (Section 2.4). Returns n, or -1 if the beam has more than cap cells; `wmax` is at least the width
+// of its widest cell (the distance between two crossings along its major axis).
 template <bool TRAJ>
 __device__ __forceinline__ int beam_cells(const float *__restrict__ map, int W, int H, const float4 *__restrict__ gains,
                                           const int32_t *pose, int ux, int uy, long long rfix, float rend, int cap,
                                           const DevParams &p, int state, const int32_t *stamps, float *sl, float *sc,
-                                          float *sp, float *sx, int *status)
+                                          float *sp, float *sx, int *status, float &wmax)
 {
     const int lane = lane_id();
     int dx, dy;
@@ -598,7 +628,9 @@ __device__ __forceinline__ int beam_cells(const float *__restrict__ map, int W, 
     const unsigned ncell = (unsigned)W * (unsigned)H;
     Geo g;
     int K;
+    wmax = 0.0f;
     if (!beam_geo(W, H, pose[0], pose[1], dx, dy, rfix, rend, g, K)) return 0;
+    wmax = 65536.0f * g.rM;
     float lend = 0.0f;
     bool by_range, bad = false;
     int n = -1;
@@ -691,9 +723,10 @@ __device__ __forceinline__ int beam_cells(const float *__restrict__ map, int W, 
 }
 
 // The variant's mutual information of one beam of n cells held in shared memory (sl: n + 1
-// distances, sp: o, sc: f_occ, sx: f_emp): Algorithm 2, Algorithm 3 (4), then the pair sum.
+// distances, sp: o, sc: f_occ, sx: f_emp; no cell wider than wmax, which only the mass form asks for):
+// Algorithm 2, Algorithm 3 (4), then the pair sum.
 template <int VAR>
-__device__ __forceinline__ float beam_sum(const DevParams &p, int n, float *sl, float *sc, float *sp, float *sx)
+__device__ __forceinline__ float beam_sum(const DevParams &p, int n, float wmax, float *sl, float *sc, float *sp, float *sx)
 {
     const int lane = lane_id();
     const bool e0 = p.e0 != 0;
@@ -717,13 +750,17 @@ __device__ __forceinline__ float beam_sum(const DevParams &p, int n, float *sl, 
                            : approx_pairs_sum<true>(LW, sc, sp, n, e0, pe0, mu0, D);
         }
         if (mass_variant(VAR)) {
-            const float mu0 = sl[0] * cs - 0.5f * cs;  // e_0 centre, l_1 - 1/2 (scaled)
-            build_targets(sl, sp, n, cs, e0 ? pe0 : 0.0f, mu0);
-            const float4 *Tg = reinterpret_cast<const float4 *>(sl);
-            float cut = fmaf(0.70710678f, cs, kMassCut);
-            if (p.flags & FSMI_FLAG_FULL_WINDOW) cut = kTailCut + kMassCutStep;
-            if (p.flags & FSMI_FLAG_FULL_SWEEP) cut = __int_as_float(0x7f800000);
-            I = exact_mass_sum<VAR == kExactMass3 ? 3 : 4>(Tg, sc, sp, n, e0, cut);
+            constexpr int D = VAR == kExactMass3 ? 3 : 4;
+            if (wmax * cs > kMassWidth<D>) {
+                I = wide_beam_sum(sl, sc, sp, n, e0, pe0, cs);
+            } else {
+                const float mu0 = sl[0] * cs - 0.5f * cs;  // e_0 centre, l_1 - 1/2 (scaled)
+                build_targets(sl, sp, n, cs, e0 ? pe0 : 0.0f, mu0);
+                float cut = fmaf(0.5f * wmax, cs, kMassCut);
+                if (p.flags & FSMI_FLAG_FULL_WINDOW) cut = kTailCut + kMassCutStep;
+                if (p.flags & FSMI_FLAG_FULL_SWEEP) cut = __int_as_float(0x7f800000);
+                I = exact_mass_sum<D>(reinterpret_cast<const float4 *>(sl), sc, sp, n, e0, cut);
+            }
         }
         if (VAR == FSMI_UNIFORM) I = uniform_sum(sx, sp, n, e0, pe0, p.H, p.inv_2h1);
         I = warp_sum(I);
@@ -747,6 +784,7 @@ __device__ __forceinline__ void eval_beam(const Src2D &src, const DevParams &p, 
 {
     const int lane = lane_id();
     int n;
+    float wmax = 0.0f;
     if (SRC != kSrcBeams) {
         const int32_t *pose;
         int ux, uy;
@@ -797,7 +835,7 @@ __device__ __forceinline__ void eval_beam(const Src2D &src, const DevParams &p, 
             uy = src.dirs[2 * bi + 1];
         }
         n = beam_cells<SRC == kSrcTraj>(src.map, src.W, src.H, src.gains, pose, ux, uy, rfix, rend, p.nmax, p, state,
-                                        stamps, sl, sc, sp, sx, status);
+                                        stamps, sl, sc, sp, sx, status, wmax);
         if (n < 0) return store_nan(out, beam, status, FSMI_STATUS_BEAM_OVERFLOW);
     } else {
         const int base = src.off[beam];
@@ -813,7 +851,7 @@ __device__ __forceinline__ void eval_beam(const Src2D &src, const DevParams &p, 
         if (lane == 0) sl[n] = __ldg(src.lend + beam);
         __syncwarp();
     }
-    const float I = beam_sum<VAR>(p, n, sl, sc, sp, sx);
+    const float I = beam_sum<VAR>(p, n, wmax, sl, sc, sp, sx);
     if (lane == 0) out[beam] = I;
     __syncwarp();
 }

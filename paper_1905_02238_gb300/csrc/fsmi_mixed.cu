@@ -309,10 +309,11 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4)
                 float *sl, *sc, *sp, *sx;
                 carve_2d(base, stride2, sl, sc, sp, sx);
                 const int32_t *d = cc->dir + 2 * kd;
+                float wmax;
                 const int n = beam_cells<false>(src.map, src.W, src.H, src.gains, cc->pose + 4 * kp, d[0], d[1], cc->rfix,
-                                                cc->rend, p2.nmax, p2, 0, nullptr, sl, sc, sp, sx, status);
+                                                cc->rend, p2.nmax, p2, 0, nullptr, sl, sc, sp, sx, status, wmax);
                 if (n >= 0) {
-                    I = beam_sum<VAR>(p2, n, sl, sc, sp, sx);
+                    I = beam_sum<VAR>(p2, n, wmax, sl, sc, sp, sx);
                 } else {
                     I = __int_as_float(0x7fc00000);
                     bad = FSMI_STATUS_BEAM_OVERFLOW;
@@ -351,13 +352,13 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4)
             st.max_range <= p2.rmax) {
             const long long rfix = __double2ll_rn((double)st.max_range * 65536.0);
             const float rend = (float)((double)rfix * (1.0 / 65536.0));
-            float *sl, *sc, *sp, *sx;
+            float *sl, *sc, *sp, *sx, wmax;
             carve_2d(base, stride2, sl, sc, sp, sx);
             const int n = beam_cells<false>(src.map, src.W, src.H, src.gains, src.poses2 + 4 * pi,
                                             src.dirs2[2 * di], src.dirs2[2 * di + 1], rfix, rend, p2.nmax, p2, 0,
-                                            nullptr, sl, sc, sp, sx, status);
+                                            nullptr, sl, sc, sp, sx, status, wmax);
             if (n >= 0)
-                I = beam_sum<VAR>(p2, n, sl, sc, sp, sx);
+                I = beam_sum<VAR>(p2, n, wmax, sl, sc, sp, sx);
             else
                 bad = FSMI_STATUS_BEAM_OVERFLOW;
         } else if (ok && st.kind == FSMI_SET_3D && src.has3d && pi < src.P3 && di < src.R3 && st.volume >= 0 &&
