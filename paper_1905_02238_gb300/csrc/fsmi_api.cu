@@ -90,8 +90,9 @@ static float gain_poly_host(const float (*c)[2], int w, int terms, float o)
 // singularity of h lies at o = -1 / (delta - 1), so for deltas near 1 the powers' coefficients fall
 // geometrically and Horner's rule rounds no worse than Clenshaw's, in half the operations. Returns
 // whether the polynomial, evaluated as the kernels do, is within `tol` of f (relative) everywhere on a
-// dense grid of [0, 1] that includes points down to 1e-7 from either end.
-static bool fit_gain(DevParams &d, int terms, double tol)
+// dense grid of [0, 1] that includes points down to 1e-7 from either end, and the interpolant itself, in
+// double, within `cut`.
+static bool fit_gain(DevParams &d, int terms, double tol, double cut)
 {
     const double pi = 3.14159265358979323846;
     memset(d.gfit2, 0, sizeof(d.gfit2));
@@ -123,8 +124,11 @@ static bool fit_gain(DevParams &d, int terms, double tol)
         for (int k = 0; k < terms; ++k) d.gfit2[k][w] = (float)pw[k];
         auto check = [&](float o) {
             const double e = gain_exact(delta, (double)o);
-            const double g = (double)gain_poly_host(d.gfit2, w, terms, o);
-            return e == 0.0 ? g == 0.0 : fabs(g - e) <= tol * fabs(e);
+            const double g = (double)gain_poly_host(d.gfit2, w, terms, o), x = 2.0 * o - 1.0;
+            double h = pw[terms - 1];
+            for (int k = terms - 2; k >= 0; --k) h = h * x + pw[k];
+            h *= o * (1.0 - o);
+            return e == 0.0 ? g == 0.0 : fabs(g - e) <= tol * fabs(e) && fabs(h - e) <= cut * fabs(e);
         };
         for (int i = 0; i <= 8192; ++i)
             if (!check((float)i / 8192.0f)) return false;
@@ -134,9 +138,10 @@ static bool fit_gain(DevParams &d, int terms, double tol)
     return true;
 }
 
-// The short polynomial where FP32 rounding dominates its error (2e-7: delta 1.5 and 0.67 reach 1.6e-7 with
-// 8 and with 14 terms), else the long one within 1e-6, else the closed form. The last fit is remembered per
-// host thread.
+// The short polynomial where FP32 rounding (1.5e-7 with 8 and with 14 terms) dominates its error: its own at most
+// 3/4 of 2^-24 (4.2e-8 at delta 1.5, 3.8e-8 at 0.67; at 1.56 it is 8.8e-8 and the FP32 error 1.9e-7 against
+// 1.3e-7 of the long one), else the long one within 1e-6, else the closed form. The last fit is remembered
+// per host thread.
 static void fit_gains(DevParams &d)
 {
     thread_local float last_docc = -1.0f, last_demp = -1.0f, last_c[kGainFitTerms][2];
@@ -146,7 +151,7 @@ static void fit_gains(DevParams &d)
         memcpy(d.gfit2, last_c, sizeof(last_c));
         return;
     }
-    d.gain_fit = fit_gain(d, kGainShortTerms, 2e-7) ? 2 : fit_gain(d, kGainFitTerms, 1e-6) ? 1 : 0;
+    d.gain_fit = fit_gain(d, kGainShortTerms, 2e-7, 4.47e-8) ? 2 : fit_gain(d, kGainFitTerms, 1e-6, 1e-6) ? 1 : 0;
     last_docc = d.docc;
     last_demp = d.demp;
     last_fit = d.gain_fit;
