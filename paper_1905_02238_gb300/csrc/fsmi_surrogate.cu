@@ -178,13 +178,14 @@ __device__ __forceinline__ void load_wfrag(const bf16 *Wt, int ks, unsigned (&bw
 // a_3 = bf16(a - a_1 - a_2), whose sum is a (1 + d) with |d| <= 2^-18 for two terms and 2^-27 for three
 // (the split-BF16 products of Henry, Tang and Heinecke, "Leveraging the bfloat16 artificial
 // intelligence datatype for higher-precision computations", 2019). The forward pass, whose outputs feed
-// the loss and its derivative, takes three terms (weights are exact in one); the backward pass two,
-// A_1 B_1 + A_2 B_1 + A_1 B_2 where both operands are FP32 (the A_2 B_2 term is below 2^-18 of the
-// product).
+// the loss and its derivative, takes three terms (weights are exact in one); the data gradients and
+// fc1's weight gradient take two, A_1 B_1 + A_2 B_1 + A_1 B_2 where both operands are FP32 (the A_2 B_2 term is
+// below 2^-18 of the product); the convolutions' weight gradients take three and all products above 2^-26, as
+// accurate as FP32 multiply-adds (strip_outer).
 //
 // The convolutions work on strips of 16 output positions per warp whose MMA fragments are formed in
 // registers: nothing is staged, and the im2col matrix exists nowhere. A step of 4096 beams with its sampling
-// takes 265 us; 754 us with every layer an index-function GEMM (operands gathered element by element through
+// takes 268 us; 754 us with every layer an index-function GEMM (operands gathered element by element through
 // shared memory) and the reductions in 21 launches.
 
 // (v.x, v.y) as T BF16 pairs
@@ -659,8 +660,10 @@ __global__ void __launch_bounds__(256)
 // The grid, the strips of each warp and the order of the sums depend only on N: the blocks' sums go to
 // part[block][...] and are added in block order (k_grads), so a step gives the same floats on every run.
 // The sums take 52 registers per lane, and two blocks of 8 warps per SM do not hide the strips' loads; the
-// next strip's rows are prefetched toward L1. A batch of 4096: 34 us (conv3) and 68 us (conv2 and conv1); one
-// warp per strip with all 32 channels (255 registers) 38 and 77 us; the separate data, weight and bias
+// next strip's rows are prefetched toward L1. A batch of 4096: 38 us (conv3) and 85 us (conv2 and conv1); with the
+// weight gradients from two terms per operand 33 and 66 us, but up to 2.5 times as far from 64 bits. Blocks
+// of 6 warps with 168 registers instead of 128 (56 bytes spilled instead of 224): the same time. In the two-term form one
+// warp per strip with all 32 channels took 38 and 77 us against 34 and 68; the separate data, weight and bias
 // gradient kernels 320 us.
 constexpr int kBwdWarps = 8, kBwdBlocks = 304;
 constexpr int kTrPitch = kCh + 8;  // row pitch of the staged weights: 80 B, eight rows in eight bank groups
@@ -674,19 +677,23 @@ __device__ __forceinline__ unsigned transpose8(unsigned v)
     return r;
 }
 
-// acc += (T_0 + T_1)^T (U_0 + U_1) without the last product: T (32 columns) and U (16) strips of 16
-// positions as two BF16 terms, transposed (T: A fragments of the 32 rows c, U: B fragments of two n8 tiles)
-__device__ __forceinline__ void strip_outer(float (&acc)[2][2][4], const unsigned (&T)[4][2][2], const unsigned (&U)[2][2][2])
+// acc += (T_0 + T_1 + T_2)^T (U_0 + U_1 + U_2) without the products below 2^-26: T (32 columns) and U (tile nt's 8)
+// strips of 16 positions as three BF16 terms, transposed (A fragments of the 32 rows c, B fragments of an n8
+// tile). The strip's sum is formed by itself, from its smallest products on, and added in FP32: the tensor cores'
+// accumulators round toward zero, and a sum kept in them over all strips would shrink.
+__device__ __forceinline__ void strip_outer(float (&acc)[2][2][4], int nt, const unsigned (&T)[4][2][3], const unsigned (&U)[2][3])
 {
+    constexpr int kI[6] = {0, 2, 1, 0, 1, 0}, kJ[6] = {2, 0, 1, 1, 0, 0};
 #pragma unroll
-    for (int p = 0; p < 3; ++p) {
-        const int i = p == 1, j = p == 2;
+    for (int mt = 0; mt < 2; ++mt) {
+        float s[4] = {};
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+        for (int p = 0; p < 6; ++p) {
+            const int i = kI[p], j = kJ[p];
+            mma_bf16(s, T[2 * mt][0][i], T[2 * mt + 1][0][i], T[2 * mt][1][i], T[2 * mt + 1][1][i], U[0][j], U[1][j]);
+        }
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
-                mma_bf16(acc[mt][nt], T[2 * mt][0][i], T[2 * mt + 1][0][i], T[2 * mt][1][i], T[2 * mt + 1][1][i], U[nt][0][j],
-                         U[nt][1][j]);
+        for (int q = 0; q < 4; ++q) acc[mt][nt][q] += s[q];
     }
 }
 
@@ -711,130 +718,144 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2)
     const int Lout = Lin >> 1, tpb = Lout / 16;
     const long long units = (long long)N * tpb, np = (long long)gridDim.x * (kBwdWarps / 2),
                     me = (long long)blockIdx.x * (kBwdWarps / 2) + (wp >> 1);
-    const long long u0 = units * me / np, u1 = units * (me + 1) / np;
+    const int u0 = (int)(units * me / np), u1 = (int)(units * (me + 1) / np);  // (a strip's rows take 6 KB and more)
     float acc[3][2][2][4] = {}, acc1[4] = {};
     float2 gb[2] = {}, gb1[2] = {};
-    for (long long u = u0; u < u1; ++u) {
-        const int n = (int)(u / tpb), t0 = (int)(u % tpb) * 16;
+    for (int u = u0; u < u1; ++u) {
+        const int n = u / tpb, t0 = u % tpb * 16;
         if (u + 1 < u1) {  // the next strip's rows, which follow this one's, toward L1
             const float *nd = dz + (size_t)(u + 1) * 16 * kCh, *nz = zprev + (size_t)(u + 1) * 32 * kCh;
             asm volatile("prefetch.global.L1 [%0];" ::"l"(lane < 16 ? nd + lane * kCh : nz + (lane - 16 + 16 * half) * kCh));
         }
-        unsigned a[4][2][2], b[4][2][2];  // terms of dz at t and at t + 1
+        // weight gradient: three terms of dz's strip, transposed
+        unsigned a[4][2][3];
         const float *dr = dz + ((size_t)n * Lout + t0 + g) * kCh + 4 * wq;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             float2 v[4];
             load8(dr + 8 * e * kCh, v);
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) split<2>(v[nt], a[nt][e]);
+            for (int nt = 0; nt < 4; ++nt) split<3>(v[nt], a[nt][e]);
 #pragma unroll
             for (int nt = 0; nt < 2; ++nt) {
                 gb[nt].x += half ? v[nt + 2].x : v[nt].x;
                 gb[nt].y += half ? v[nt + 2].y : v[nt].y;
             }
         }
-        {  // one row on: lane + 4's row, the last from memory (zero past the beam)
-            float2 v[4] = {};
-            if (g == 7 && t0 + 16 < Lout) load8(dr + 9 * kCh, v);
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                unsigned t[2];
-                split<2>(v[nt], t);
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const unsigned lo = __shfl_sync(kFull, a[nt][0][i], lane + 4), hi = __shfl_sync(kFull, a[nt][1][i], lane + 4);
-                    b[nt][0][i] = g == 7 ? hi : lo;
-                    b[nt][1][i] = g == 7 ? t[i] : hi;
-                }
-            }
-        }
-        float ev[2][4] = {}, od[2][4] = {};
-#pragma unroll
-        for (int ks = 0; ks < 2; ++ks) {
-            unsigned bw[3][2][2];
-#pragma unroll
-            for (int k = 0; k < 3; ++k)
-                ldsm_x4(smem_u32(sW + (k * kCh + ch + (lane & 7) + 8 * (lane >> 4)) * kTrPitch + ks * 16 + 8 * ((lane >> 3) & 1)),
-                        bw[k][0][0], bw[k][0][1], bw[k][1][0], bw[k][1][1]);
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    mma_bf16(ev[q], a[2 * ks][0][i], a[2 * ks][1][i], a[2 * ks + 1][0][i], a[2 * ks + 1][1][i], bw[1][q][0],
-                             bw[1][q][1]);
-                    mma_bf16(od[q], b[2 * ks][0][i], b[2 * ks][1][i], b[2 * ks + 1][0][i], b[2 * ks + 1][1][i], bw[0][q][0],
-                             bw[0][q][1]);
-                    mma_bf16(od[q], a[2 * ks][0][i], a[2 * ks][1][i], a[2 * ks + 1][0][i], a[2 * ks + 1][1][i], bw[2][q][0],
-                             bw[2][q][1]);
-                }
-        }
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
             for (int e = 0; e < 2; ++e)
 #pragma unroll
-                for (int i = 0; i < 2; ++i) a[nt][e][i] = transpose8(a[nt][e][i]);
+                for (int i = 0; i < 3; ++i) a[nt][e][i] = transpose8(a[nt][e][i]);
         // the layer below at 2t + tap - 1, rows g and g + 8 of the strip: the other factor of the weight
         // gradient and (taps 1, 2) the mask of the data gradient at 2t and 2t + 1. Tap 0 is tap 2's strip one
         // row down, its first row from memory.
-        unsigned p[2][2][2], first[2][2];
-        {
-            const int r = 2 * t0 - 1;
-            float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (g == 0 && r >= 0) z = *reinterpret_cast<const float4 *>(zprev + ((size_t)n * Lin + r) * kCh + 16 * half + 4 * wq);
-            split<2>(relu2(make_float2(z.x, z.y)), first[0]);
-            split<2>(relu2(make_float2(z.z, z.w)), first[1]);
-        }
+        unsigned p[2][2][3], mask = 0u;
+        const size_t zo = ((size_t)n * Lin + 2 * (t0 + g)) * kCh + 16 * half + 4 * wq;
 #pragma unroll
         for (int tap = 1; tap < 3; ++tap) {
-            const size_t o = ((size_t)n * Lin + 2 * (t0 + g) + tap - 1) * kCh + 16 * half + 4 * wq;
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const float4 z = *reinterpret_cast<const float4 *>(zprev + o + 16 * e * kCh);
-                split<2>(relu2(make_float2(z.x, z.y)), p[0][e]);
-                split<2>(relu2(make_float2(z.z, z.w)), p[1][e]);
-                float(&d)[2][4] = tap == 1 ? ev : od;
-                d[0][2 * e] = z.x > 0.0f ? d[0][2 * e] : 0.0f;
-                d[0][2 * e + 1] = z.y > 0.0f ? d[0][2 * e + 1] : 0.0f;
-                d[1][2 * e] = z.z > 0.0f ? d[1][2 * e] : 0.0f;
-                d[1][2 * e + 1] = z.w > 0.0f ? d[1][2 * e + 1] : 0.0f;
-                if (!LAST)
-                    *reinterpret_cast<float4 *>(out + o + 16 * e * kCh) =
-                        make_float4(d[0][2 * e], d[0][2 * e + 1], d[1][2 * e], d[1][2 * e + 1]);
+                const float4 z = *reinterpret_cast<const float4 *>(zprev + zo + (tap - 1 + 16 * e) * kCh);
+                split<3>(relu2(make_float2(z.x, z.y)), p[0][e]);
+                split<3>(relu2(make_float2(z.z, z.w)), p[1][e]);
+                mask |= ((z.x > 0.0f) | (z.y > 0.0f) << 1 | (z.z > 0.0f) << 2 | (z.w > 0.0f) << 3) << (8 * (tap - 1) + 4 * e);
             }
-            unsigned q[2][2][2];
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
+            for (int nt = 0; nt < 2; ++nt) {
+                unsigned q[2][3];
 #pragma unroll
                 for (int e = 0; e < 2; ++e)
 #pragma unroll
-                    for (int i = 0; i < 2; ++i) q[nt][e][i] = transpose8(p[nt][e][i]);
-            strip_outer(acc[tap], a, q);
+                    for (int i = 0; i < 3; ++i) q[e][i] = transpose8(p[nt][e][i]);
+                strip_outer(acc[tap], nt, a, q);
+            }
+        }
+        {
+            float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (g == 0 && t0 > 0) z = *reinterpret_cast<const float4 *>(zprev + zo - kCh);
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt) {
+                unsigned first[3], q[2][3];
+                split<3>(relu2(nt ? make_float2(z.z, z.w) : make_float2(z.x, z.y)), first);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const unsigned lo = __shfl_sync(kFull, p[nt][0][i], lane + 28), hi = __shfl_sync(kFull, p[nt][1][i], lane + 28);
+                    q[0][i] = transpose8(g == 0 ? first[i] : lo);
+                    q[1][i] = transpose8(g == 0 ? lo : hi);
+                }
+                strip_outer(acc[0], nt, a, q);
+            }
+        }
+        // data gradient: two terms of dz at t (the first two, transposed back) and at t + 1, 16 channels at a time
+        float ev[2][4] = {}, od[2][4] = {};
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+            unsigned r[2][2][2], r1[2][2][2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) r[h][e][i] = transpose8(a[2 * ks + h][e][i]);
+            {  // one row on: lane + 4's row, the last from memory (zero past the beam)
+                float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (g == 7 && t0 + 16 < Lout) v = *reinterpret_cast<const float4 *>(dr + 9 * kCh + 16 * ks);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    unsigned t[2];
+                    split<2>(h ? make_float2(v.z, v.w) : make_float2(v.x, v.y), t);
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const unsigned lo = __shfl_sync(kFull, r[h][0][i], lane + 4), hi = __shfl_sync(kFull, r[h][1][i], lane + 4);
+                        r1[h][0][i] = g == 7 ? hi : lo;
+                        r1[h][1][i] = g == 7 ? t[i] : hi;
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                unsigned bw[2][2];
+                ldsm_x4(smem_u32(sW + (k * kCh + ch + (lane & 7) + 8 * (lane >> 4)) * kTrPitch + ks * 16 + 8 * ((lane >> 3) & 1)),
+                        bw[0][0], bw[0][1], bw[1][0], bw[1][1]);
+                float(&d)[2][4] = k == 1 ? ev : od;
+                const unsigned(&s)[2][2][2] = k == 0 ? r1 : r;
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) mma_bf16(d[q], s[0][0][i], s[0][1][i], s[1][0][i], s[1][1][i], bw[q][0], bw[q][1]);
+            }
         }
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
+        for (int odd = 0; odd < 2; ++odd)
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const unsigned lo = __shfl_sync(kFull, p[nt][0][i], lane + 28), hi = __shfl_sync(kFull, p[nt][1][i], lane + 28);
-                p[nt][0][i] = transpose8(g == 0 ? first[nt][i] : lo);
-                p[nt][1][i] = transpose8(g == 0 ? lo : hi);
+            for (int e = 0; e < 2; ++e) {
+                float(&d)[2][4] = odd ? od : ev;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    float &v = d[k >> 1][2 * e + (k & 1)];
+                    v = mask >> (8 * odd + 4 * e + k) & 1u ? v : 0.0f;
+                }
+                if (!LAST)
+                    *reinterpret_cast<float4 *>(out + zo + (odd + 16 * e) * kCh) =
+                        make_float4(d[0][2 * e], d[0][2 * e + 1], d[1][2 * e], d[1][2 * e + 1]);
             }
-        strip_outer(acc[0], a, p);
         if (LAST) {
             // conv1: gW1[c][k][ci] = sum over positions p of dz1[p][c] x[2p + k - 1][ci], column 2k + ci of the
             // n8 tile (6 of 8 used; x is exact in BF16)
             const unsigned short *xr = reinterpret_cast<const unsigned short *>(x) + (size_t)n * kL * kCin;
+            float sum1[4] = {};
 #pragma unroll
             for (int odd = 0; odd < 2; ++odd) {  // p = 2t + odd
                 float(&d)[2][4] = odd ? od : ev;
-                unsigned t[2][2][2], bx[2];
+                unsigned t[2][2][3], bx[2];
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt) {
                     gb1[nt].x += d[nt][0] + d[nt][2];
                     gb1[nt].y += d[nt][1] + d[nt][3];
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) split<2>(make_float2(d[nt][2 * e], d[nt][2 * e + 1]), t[nt][e]);
+                    for (int e = 0; e < 2; ++e) split<3>(make_float2(d[nt][2 * e], d[nt][2 * e + 1]), t[nt][e]);
                 }
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
@@ -844,10 +865,12 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2)
                     bx[e] = lo | hi << 16;
                 }
 #pragma unroll
-                for (int i = 0; i < 2; ++i)
-                    mma_bf16(acc1, transpose8(t[0][0][i]), transpose8(t[1][0][i]), transpose8(t[0][1][i]),
+                for (int i = 2; i >= 0; --i)
+                    mma_bf16(sum1, transpose8(t[0][0][i]), transpose8(t[1][0][i]), transpose8(t[0][1][i]),
                              transpose8(t[1][1][i]), bx[0], bx[1]);
             }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc1[q] += sum1[q];
         }
     }
     // the columns' sums over the eight row groups, then the block's sums, pair by pair of warps (the two of a
