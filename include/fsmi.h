@@ -529,6 +529,17 @@ fsmi_status fsmi_gather_rows(const int32_t *src, long long nrows, int width, con
  * update counts), FSMI_QUEUE_BYTES for the other evaluations. */
 fsmi_status fsmi_workspace_size(int fn, long long nitems, const fsmi_params *prm, size_t *bytes);
 
+/* Bytes of device workspace that fsmi_eval_2d with these sizes and parameters would use on the current device under
+ * the calling thread's schedule, at most fsmi_workspace_size(FSMI_FN_EVAL_2D, W*H): 0 for a batch that has a
+ * warp for every beam (nothing for a queue to balance) and visits fewer cells than the map holds. */
+fsmi_status fsmi_eval_2d_workspace_size(int W, int H, int P, int B, const fsmi_params *prm, size_t *bytes);
+
+/* fsmi_eval_2d without a workspace, if it would use none (*need = 0); otherwise nothing is launched, *need is what
+ * fsmi_eval_2d_workspace_size reports and FSMI_ERR_WORKSPACE is returned. For callers that take workspaces from
+ * an allocator per call: one call where none is needed. */
+fsmi_status fsmi_eval_2d_no_workspace(const float *map, int W, int H, const int32_t *poses, int P, const int32_t *dirs,
+                                      int B, const fsmi_params *prm, float *out, size_t *need, fsmi_stream_t stream);
+
 /*
  * Native schedule tuning and CUDA-graph helpers (library conveniences; the paper has none).
  *

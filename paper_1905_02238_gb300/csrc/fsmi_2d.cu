@@ -1,4 +1,6 @@
 // 2D kernels and their launchers; the per-beam device code is in eval2d.cuh.
+#include <type_traits>
+
 #include "eval2d.cuh"
 
 namespace fsmi {
@@ -58,27 +60,61 @@ __global__ void k_gauss_tail(const float *__restrict__ s, float *__restrict__ ou
 }
 
 
+// Shape of one launch of k_eval_2d<VAR, SRC> under the thread's schedule.
+struct Launch2D {
+    int stride, wpb;
+    size_t smem;
+    WarpGrid g;
+};
+
+template <int VAR, int SRC>
+static cudaError_t shape_variant(const DevParams &p, long long nbeams, Launch2D &l)
+{
+    const Schedule &sc = current_schedule(FSMI_KIND_2D);
+    l.stride = stride_2d(p.nmax);
+    const size_t per_warp = (size_t)warp_floats_2d(l.stride) * sizeof(float);
+    l.wpb = fit_warps(sc.warps_per_block, per_warp, 0);
+    l.smem = (size_t)l.wpb * per_warp;
+    return warp_grid((const void *)k_eval_2d<VAR, SRC>, nbeams, l.wpb, l.smem, sc.blocks_per_sm, l.g);
+}
+
 template <int VAR, int SRC>
 static cudaError_t launch_variant(const Src2D &src, const DevParams &p, long long nbeams, float *out, int *status,
                                   unsigned long long *queue, cudaStream_t s)
 {
     const Schedule &sc = current_schedule(FSMI_KIND_2D);
-    const int stride = stride_2d(p.nmax);
-    const size_t per_warp = (size_t)warp_floats_2d(stride) * sizeof(float);
-    const int wpb = fit_warps(sc.warps_per_block, per_warp, 0);
-    const size_t smem = (size_t)wpb * per_warp;
-    auto kern = k_eval_2d<VAR, SRC>;
-    WarpGrid g;
-    cudaError_t e = warp_grid((const void *)kern, nbeams, wpb, smem, sc.blocks_per_sm, g);
+    Launch2D l;
+    cudaError_t e = shape_variant<VAR, SRC>(p, nbeams, l);
     if (e != cudaSuccess) return e;
-    if (g.one_each) queue = nullptr;  // nothing to balance: no counter to clear (one launch less)
+    if (l.g.one_each) queue = nullptr;  // nothing to balance: no counter to clear (one launch less)
     if (queue) {
         e = cudaMemsetAsync(queue, 0, sizeof(unsigned long long), s);
         if (e != cudaSuccess) return e;
     }
-    kern<<<g.grid, wpb * 32, smem, s>>>(src, p, nbeams, stride, out, status, queue,
-                                         sc.queue_chunk > 0 ? sc.queue_chunk : 1);
+    k_eval_2d<VAR, SRC><<<l.g.grid, l.wpb * 32, l.smem, s>>>(src, p, nbeams, l.stride, out, status, queue,
+                                                              sc.queue_chunk > 0 ? sc.queue_chunk : 1);
     return cudaGetLastError();
+}
+
+// f(the call's kernel variant as an integral constant)
+template <int SRC, class F>
+static cudaError_t with_variant(const DevParams &p, F &&f)
+{
+    int var = p.variant == FSMI_EXACT && (p.flags & FSMI_FLAG_FULL_SWEEP) ? kExactFullSweep : p.variant;
+    if constexpr (SRC != kSrcBeams) {
+        var = grid_variant(p);
+        switch (var) {
+            case kExactMass3: return f(std::integral_constant<int, kExactMass3>{});
+            case kExactMass4: return f(std::integral_constant<int, kExactMass4>{});
+            default: break;
+        }
+    }
+    switch (var) {
+        case FSMI_EXACT: return f(std::integral_constant<int, FSMI_EXACT>{});
+        case kExactFullSweep: return f(std::integral_constant<int, kExactFullSweep>{});
+        case FSMI_APPROX: return f(std::integral_constant<int, FSMI_APPROX>{});
+        default: return f(std::integral_constant<int, FSMI_UNIFORM>{});
+    }
 }
 
 template <int SRC>
@@ -86,21 +122,17 @@ static cudaError_t dispatch(const Src2D &src, const DevParams &p, long long nbea
                             unsigned long long *queue, cudaStream_t s)
 {
     if (nbeams <= 0) return cudaSuccess;
-    int var = p.variant == FSMI_EXACT && (p.flags & FSMI_FLAG_FULL_SWEEP) ? kExactFullSweep : p.variant;
-    if constexpr (SRC != kSrcBeams) {
-        var = grid_variant(p);
-        switch (var) {
-            case kExactMass3: return launch_variant<kExactMass3, SRC>(src, p, nbeams, out, status, queue, s);
-            case kExactMass4: return launch_variant<kExactMass4, SRC>(src, p, nbeams, out, status, queue, s);
-            default: break;
-        }
-    }
-    switch (var) {
-        case FSMI_EXACT: return launch_variant<FSMI_EXACT, SRC>(src, p, nbeams, out, status, queue, s);
-        case kExactFullSweep: return launch_variant<kExactFullSweep, SRC>(src, p, nbeams, out, status, queue, s);
-        case FSMI_APPROX: return launch_variant<FSMI_APPROX, SRC>(src, p, nbeams, out, status, queue, s);
-        default: return launch_variant<FSMI_UNIFORM, SRC>(src, p, nbeams, out, status, queue, s);
-    }
+    return with_variant<SRC>(
+        p, [&](auto var) { return launch_variant<decltype(var)::value, SRC>(src, p, nbeams, out, status, queue, s); });
+}
+
+cudaError_t eval_2d_one_each(const DevParams &p, long long nbeams, bool &one_each)
+{
+    Launch2D l;
+    const cudaError_t e =
+        with_variant<kSrcMap>(p, [&](auto var) { return shape_variant<decltype(var)::value, kSrcMap>(p, nbeams, l); });
+    one_each = e == cudaSuccess && l.g.one_each;
+    return e;
 }
 
 cudaError_t map_gains(const float *map, int W, int H, const DevParams &p, float4 *gains, cudaStream_t s)

@@ -230,12 +230,14 @@ unsigned long long *queue_of(int kind, void *ws, size_t ws_bytes)
     return (unsigned long long *)ws;
 }
 
-// Per-map-cell gains behind the queue counter, when the workspace fits them and the batch visits
-// more cells (up to nbeams * nmax, half that on average) than the map holds.
+// Whether a batch visits more cells (up to nbeams * nmax, half that on average) than the map holds.
+bool gains_pay(long long cells, long long nbeams, int nmax) { return nbeams * (nmax / 2) >= cells; }
+
+// Per-map-cell gains behind the queue counter, when the workspace fits them and they pay.
 float4 *gains_of(void *ws, size_t ws_bytes, long long cells, long long nbeams, int nmax)
 {
     if (!ws || !aligned16(ws) || ws_bytes < kQueueBytes + (size_t)cells * sizeof(float4)) return nullptr;
-    if (nbeams * (nmax / 2) < cells) return nullptr;
+    if (!gains_pay(cells, nbeams, nmax)) return nullptr;
     return (float4 *)((char *)ws + kQueueBytes);
 }
 
@@ -740,6 +742,35 @@ fsmi_status fsmi_workspace_size(int fn, long long nitems, const fsmi_params *prm
     else if (fn == FSMI_FN_UPDATE_MAP_2D) *bytes = (size_t)nitems * 2 * sizeof(uint32_t);
     else *bytes = kQueueBytes;
     return FSMI_OK;
+}
+
+fsmi_status fsmi_eval_2d_workspace_size(int W, int H, int P, int B, const fsmi_params *prm, size_t *bytes)
+{
+    if (!bytes) return FSMI_ERR_ARG;
+    *bytes = 0;
+    DevParams d;
+    const fsmi_status st = make_params(prm, kUse2D, d);
+    if (st != FSMI_OK) return st;
+    if (!grid_ok(W) || !grid_ok(H) || P < 0 || B < 0) return FSMI_ERR_ARG;
+    const long long cells = (long long)W * H, nbeams = (long long)P * B;
+    if (nbeams == 0) return FSMI_OK;
+    if (gains_pay(cells, nbeams, d.nmax)) {
+        *bytes = kQueueBytes + (size_t)cells * sizeof(float4);
+    } else if (g_schedule[FSMI_KIND_2D].queue_chunk > 0) {
+        bool one_each = false;
+        const cudaError_t e = eval_2d_one_each(d, nbeams, one_each);
+        if (e != cudaSuccess) return cuda_fail(e);
+        if (!one_each) *bytes = kQueueBytes;
+    }
+    return FSMI_OK;
+}
+
+fsmi_status fsmi_eval_2d_no_workspace(const float *map, int W, int H, const int32_t *poses, int P, const int32_t *dirs, int B,
+                                      const fsmi_params *prm, float *out, size_t *need, fsmi_stream_t stream)
+{
+    const fsmi_status st = fsmi_eval_2d_workspace_size(W, H, P, B, prm, need);
+    if (st != FSMI_OK) return st;
+    return *need ? FSMI_ERR_WORKSPACE : fsmi_eval_2d(map, W, H, poses, P, dirs, B, prm, out, nullptr, 0, stream);
 }
 
 fsmi_status fsmi_set_wait_limit(long long polls)

@@ -77,6 +77,8 @@ cudaError_t warp_grid(const void *kern, long long n, int wpb, size_t smem, int m
 constexpr size_t kQueueBytes = 256;
 
 // 2D (fsmi_2d.cu)
+// whether fsmi_eval_2d's launch has a warp for every beam, so that a work queue would not be used
+cudaError_t eval_2d_one_each(const DevParams &p, long long nbeams, bool &one_each);
 cudaError_t launch_eval_2d(const float *map, int W, int H, const int32_t *poses, int P, const int32_t *dirs, int B,
                            const DevParams &p, float *out, float4 *gains, unsigned long long *queue, int *status,
                            cudaStream_t s);

@@ -28,6 +28,7 @@ FLAG_FULL_SWEEP = 0x1
 FLAG_FULL_WINDOW = 0x2
 FN_EVAL_2D, FN_EVAL_BEAMS, FN_RLE_ENCODE_3D, FN_EVAL_RLE, FN_EVAL_3D, FN_UPDATE_MAP_2D = 0, 1, 2, 3, 4, 5
 QUEUE_BYTES = 256
+ERR_WORKSPACE = 5
 SURR_L, SURR_NPARAMS = 256, 269089
 KIND_2D, KIND_RLE = 0, 1
 STATUS_BEAM_OVERFLOW, STATUS_RUN_OVERFLOW, STATUS_BAD_BEAM, STATUS_TIMEOUT = 0x1, 0x2, 0x4, 0x10
@@ -157,6 +158,8 @@ def load():
             "fsmi_graph_launch": [p, p],
             "fsmi_graph_destroy": [p],
             "fsmi_workspace_size": [i, ll, P, ctypes.POINTER(ctypes.c_size_t)],
+            "fsmi_eval_2d_no_workspace": [p, i, i, p, i, p, i, P, p, ctypes.POINTER(ctypes.c_size_t), p],
+            "fsmi_eval_2d_workspace_size": [i, i, i, i, P, ctypes.POINTER(ctypes.c_size_t)],
             "fsmi_trajectory_workspace_size": [i, i, i, ctypes.POINTER(ctypes.c_size_t)],
             "fsmi_eval_trajectories_2d": [p, i, i, p, i, p, i, p, i, P, p, p, p, p, sz, p],
             "fsmi_best_trajectory": [p, p, i, p, i, p, p, p],
@@ -230,12 +233,6 @@ def _default_ws(nbytes: int, dev):
     return torch.empty(nbytes, dtype=torch.uint8, device=dev)
 
 
-def _small_2d(nbeams: int, cells: int, max_range: float) -> bool:
-    """Whether fsmi_eval_2d has no use for a workspace: fewer cell visits than map cells (no per-cell gains,
-    the library's own rule) and a warp for every beam (no queue; 1,216 warps fit at the longest range)."""
-    return nbeams <= 1024 and 0 < max_range <= MAX_RANGE_2D and nbeams * ((int(max_range * 1.41421357) + 3) // 2) < cells
-
-
 def _out(out, shape, m):
     if out is None or m.host:
         if _capturing():
@@ -274,8 +271,8 @@ def eval_2d(grid: torch.Tensor, poses: torch.Tensor, dirs: torch.Tensor, prm: Pa
             out: torch.Tensor | None = None, ws: torch.Tensor | None = None) -> torch.Tensor:
     """fsmi_eval_2d: grid float32 [H, W]; poses int32 [P, 4]; dirs int32 [B, 2] -> float32 [P, B].
     ws: optional device workspace (uint8, 16-byte aligned; workspace_size(FN_EVAL_2D, H*W) bytes
-    hold the work-queue counter and the per-cell gains); by default one is taken from torch's
-    allocator. Pass an empty tensor to use none."""
+    hold the work-queue counter and the per-cell gains); by default one of the size that the call can use
+    (fsmi_eval_2d_workspace_size) is taken from torch's allocator. Pass an empty tensor to use none."""
     lib = load()
     m = _Marshal(grid, poses, dirs)
     g = m.arg(grid, torch.float32, "grid", 2)
@@ -284,11 +281,16 @@ def eval_2d(grid: torch.Tensor, poses: torch.Tensor, dirs: torch.Tensor, prm: Pa
     P, B = ps.shape[0], ds.shape[0]
     out = _out(out, (P, B), m)
     cp = prm.c()
-    if ws is None and not _small_2d(P * B, g.numel(), cp.max_range):
-        ws = _default_ws(workspace_size(FN_EVAL_2D, g.numel()), m.dev)
+    args = _ptr(g), g.shape[1], g.shape[0], _ptr(ps), P, _ptr(ds), B, ctypes.byref(cp), _ptr(out)
+    if ws is None:
+        need = ctypes.c_size_t(0)
+        code = lib.fsmi_eval_2d_no_workspace(*args, ctypes.byref(need), _stream())
+        if code != ERR_WORKSPACE:
+            _raise(code, "fsmi_eval_2d")
+            return m.out(out)
+        ws = _default_ws(need.value, m.dev)
     wp, wb = _ws_args(ws)
-    _raise(lib.fsmi_eval_2d(_ptr(g), g.shape[1], g.shape[0], _ptr(ps), P, _ptr(ds), B, ctypes.byref(cp),
-                            _ptr(out), wp, wb, _stream()), "fsmi_eval_2d")
+    _raise(lib.fsmi_eval_2d(*args, wp, wb, _stream()), "fsmi_eval_2d")
     return m.out(out)
 
 
