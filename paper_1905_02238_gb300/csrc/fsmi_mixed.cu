@@ -207,7 +207,7 @@ static_assert(sizeof(ClassCache) <= kSetCacheFloats * sizeof(float), "class cach
 template <int VAR, int KIND>
 __global__ void __launch_bounds__(kMaxWarps * 32, 4)
     k_eval_mixed(MixedSrc src, DevParams p2, DevParams p3, const __grid_constant__ RleTable tbl, long long nitems,
-                 int stride2, int stride3, float *out,
+                 int stride2, float *out,
                  unsigned long long *times, int *status, unsigned long long *queue, int chunk,
                  const unsigned char *plan_raw, int bucket)
 {
@@ -387,7 +387,6 @@ cudaError_t launch_mixed_variant(const MixedSrc &src, const DevParams &p2, const
     // a 3D class runs under the RLE family's schedule, like fsmi_eval_3d; everything else the 2D one
     const Schedule &sc = current_schedule(KIND >= kMix3D ? FSMI_KIND_RLE : FSMI_KIND_2D);
     const int stride2 = stride_2d(p2.nmax);
-    const int stride3 = ((p3.nmax + 2 * p3.K + 4) + 3) & ~3;
     const size_t per_warp = ((size_t)max(warp_floats_2d(stride2), ray3d_warp_floats(p3)) + kSetCacheFloats) * sizeof(float);
     const size_t table = rle_table_bytes(table_spec(p3).K);
     const int wpb = fit_warps(sc.warps_per_block, per_warp, table);
@@ -406,7 +405,7 @@ cudaError_t launch_mixed_variant(const MixedSrc &src, const DevParams &p2, const
     }
     RleTable tbl{};
     if (src.has3d) fill_rle_table(p3, tbl);
-    return launch_kernel(early, kern, g.grid, wpb * 32, smem, s, src, p2, p3, tbl, nitems, stride2, stride3, out, times,
+    return launch_kernel(early, kern, g.grid, wpb * 32, smem, s, src, p2, p3, tbl, nitems, stride2, out, times,
                          status, queue, sc.queue_chunk > 0 ? sc.queue_chunk : 1, plan, bucket);
 }
 
