@@ -41,7 +41,8 @@ RCP_PER_SM_CLK = 16  # SFU rcp.approx results per SM per clock (measured 15.95)
 SFU_CLK_PER_TERM = 1.0 / EX2_PER_SM_CLK + 1.0 / RCP_PER_SM_CLK  # one ex2 and one rcp per tail term
 MASS_OPS_PER_TERM = 7  # FP32 FMA-pipe operations per cell-mass term of the exact kernel (csrc/cell_mass.cuh): distance,
 #                        square, weight, 3 Horner FMAs, accumulate (and one ex2)
-TAIL_CUT = 4.81  # scaled half-width of the exact kernel's default window (csrc/eval2d.cuh)
+MASS_CUT, MASS_CUT_BEFORE = 5.2, 4.81  # the exact kernel's default window after and before a first-hit cell, scaled,
+#                                       to which half the beam's widest cell is added (csrc/eval2d.cuh)
 
 # DRAM bytes (read + write) per launch of the 2D kernel on the benchmark workload (exact; the
 # Approx and Uniform legs by name), from an ncu capture of one full-size launch each
@@ -202,8 +203,8 @@ def band_terms(n, delta):
 
 
 def work_counts(fsmi, grid, p, d, chunk=32768):
-    """(cells, Theorem-1 boundary terms n(n+1), terms the exact kernel evaluates, Approx band
-    terms at Delta = 6) of one launch."""
+    """(cells, Theorem-1 boundary terms n(n+1), cell-mass terms within the exact kernel's window,
+    Approx band terms at Delta = 6) of one launch."""
     import torch
 
     cap = int(R_MAX * 1.5) + 4
@@ -218,8 +219,10 @@ def work_counts(fsmi, grid, p, d, chunk=32768):
         ll = torch.where(col[None, :] <= nn[:, None], ll, torch.full_like(ll, float("inf")))
         mu = 0.5 * (ll[:, :-1] + ll[:, 1:])
         valid = col[None, :-1] < nn[:, None]
-        lo = torch.searchsorted(ll, mu - TAIL_CUT)
-        hi = torch.searchsorted(ll, mu + TAIL_CUT)
+        # widest cell of the beam (the cells at its ends are cut off) and, per source cell, the first-hit cells in reach
+        wide = torch.where(valid, ll[:, 1:] - ll[:, :-1], torch.zeros_like(mu)).amax(1, keepdim=True)
+        lo = torch.searchsorted(mu, mu - (MASS_CUT + 0.5 * wide))
+        hi = torch.searchsorted(mu, mu + (MASS_CUT_BEFORE + 0.5 * wide))
         terms += float(torch.where(valid, hi - lo, torch.zeros_like(hi)).sum().item())
         n64 = nn.to(torch.float64)
         cells += float(n64.sum().item())
@@ -904,7 +907,7 @@ def run_fsmi(args):
     flush = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.float32, device=dev)
 
     # algorithmic work of one launch, from the (bit-exact) traversal: Theorem 1 has n(n+1)
-    # boundary terms per beam; the kernel evaluates those within its window
+    # terms per beam; the exact kernel evaluates the cell masses within its window
     cells, pairs, terms, band = work_counts(fsmi, grid, p, d)
 
     stream = torch.cuda.current_stream()

@@ -95,7 +95,7 @@ typedef struct {
  * FSMI_FLAG_FULL_WINDOW widens the window to every term whose Gaussian tail is non-zero in FP32
  * (about 13.3 sigma; the tail underflows to exactly 0 beyond), which gives the full sweep's result
  * bit for bit; FSMI_FLAG_FULL_SWEEP evaluates all n(n+1) terms (both for verification and timing
- * comparisons). */
+ * comparisons of the window: they use the same form of the Gaussian mass as the default). */
 #define FSMI_FLAG_FULL_SWEEP 0x1
 #define FSMI_FLAG_FULL_WINDOW 0x2
 

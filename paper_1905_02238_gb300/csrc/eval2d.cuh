@@ -8,7 +8,10 @@
 //   Approx (eq. fsmi_approx): the same with |k - j| <= Delta
 //   Uniform (Algorithm 4):    sum_j P(e_j) (D_{min(n,j+H)} - D_{max(0,j-H-1)}) / (2H + 1)
 //
-// The Gaussian pair sum is evaluated per first-hit cell j in boundary form (summation by parts):
+// The exact Gaussian sum of grid cells with sigma >= 1 cell takes the mass form (cell_mass.cuh, exact_mass_sum):
+// per source cell k its mass as a polynomial times one exponential, every term non-negative. Everything else
+// Gaussian (smaller sigma, explicit beams and cells wider than the form's table, Approx-FSMI) is evaluated per
+// first-hit cell j in boundary form (summation by parts):
 //   S_j = sum_k C_k (Phi(x_{k+1}) - Phi(x_k)) = C_j + sum_{m=1}^{n+1} (C_m - C_{m-1}) sgn(x_m) T(|x_m|)
 // with x_m = (l_m - mu_j) / sigma, C_0 = C_{n+1} = 0 and T the upper Gaussian tail. Every term is
 // a tail mass, so no difference of two values near 1 is formed in FP32, and each (j, m) pair costs
@@ -62,7 +65,8 @@ __host__ __device__ constexpr bool mass_variant(int v) { return v == kExactMass3
 // explicit beams, whose cells may be any width, the boundary form. Approx-FSMI stays in boundary form:
 // its band is too short to pay for the sources' polynomials (Delta = 3, 517 poses x 181 beams, R = 181.5:
 // 274 us in mass form, 250 us in boundary form). The exact sum of the 2048x2048 office batch (1024
-// poses x 360 beams, R = 256, sigma = 2) takes 1.69 ms in mass form, 1.86 ms in boundary form.
+// poses x 360 beams, R = 256, sigma = 2) took 1.69 ms in mass form, 1.86 ms in boundary form, both before the
+// traversal in closed form and with a cut of 4.58 for the masses (1.72 ms with both and the present cuts).
 inline int grid_variant(const DevParams &p)
 {
     if (p.variant != FSMI_EXACT) return p.variant;
@@ -99,7 +103,7 @@ struct Src2D {
 // Largest scaled distance whose tail is not flushed to zero: beyond |d| = 11.3 the factor
 // 2^(-d^2) <= 2^(-127.69) is subnormal and ex2.approx.ftz returns exactly 0, so the term is +-0.
 constexpr float kTailCut = 11.3f;
-// Default window of the exact sum: T(4.81) = 7.4e-9 < 2^-27. Boundaries come at most two per
+// Default window of the boundary form: T(4.81) = 7.4e-9 < 2^-27. Boundaries come at most two per
 // major-axis crossing interval (scaled length >= cs = sqrt(log2 e) / (sigma sqrt 2)), so the terms
 // skipped on one side weigh at most 2 T(4.81) / (1 - 2^(-9.62 cs)) times max |C_m - C_{m-1}|:
 // at most 2^-24 of it (one FP32 ulp) for sigma up to 19 cells (1.01 x 2^-24 at 20), below 2^-25
