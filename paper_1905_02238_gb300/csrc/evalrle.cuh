@@ -296,7 +296,7 @@ __device__ __forceinline__ void scan_block(const DevParams &p, const float (&o)[
     for (int t = 0; t < CPL; ++t) rle_gains(p, o[t], fo[t], fe[t]);
     float prod = (1.0f - o[0]) * (1.0f - o[1]), sum = fe[0] + fe[1];
     if (CPL == 4) {
-        prod *= (1.0f - o[CPL - 2]) * (1.0f - o[CPL - 1]);
+        prod = (prod * (1.0f - o[CPL - 2])) * (1.0f - o[CPL - 1]);  // cell by cell, see cell_prefixes
         sum += fe[CPL - 2] + fe[CPL - 1];
     }
     prod = warp_incl_mul(prod);
