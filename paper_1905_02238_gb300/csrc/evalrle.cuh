@@ -151,7 +151,8 @@ static __device__ void run_starts(const RunSmem &r, int nr, bool have_s)
 }
 
 // Run prefixes (Algorithms for P_E(u) and D_E(v)): P_E(u) = prod_{i<u} (1 - o_i)^{L_i},
-// D_E(u) = sum_{i<u} L_i f(delta_emp, r_i). On entry O, L and S are set.
+// D_E(u) = sum_{i<u} L_i f(delta_emp, r_i). On entry O, L and S are set. (A run's gains are formed once and wait in A
+// and F for the second pass.)
 static __device__ void run_prefixes(const RunSmem &r, int nr, const DevParams &p)
 {
     const int lane = lane_id();
@@ -163,6 +164,8 @@ static __device__ void run_prefixes(const RunSmem &r, int nr, const DevParams &p
         const int L = r.L[u];
         float fo, fe;
         rle_gains(p, o, fo, fe);
+        r.A[u] = fo;
+        r.F[u] = fe;
         prod *= ipowf(1.0f - o, L);
         sum = fmaf((float)L, fe, sum);
     }
@@ -177,12 +180,9 @@ static __device__ void run_prefixes(const RunSmem &r, int nr, const DevParams &p
     for (int u = lo; u < hi; ++u) {
         const float o = r.O[u];
         const int L = r.L[u];
-        const float x = 1.0f - o;
-        float fo, fe;
-        rle_gains(p, o, fo, fe);
+        const float x = 1.0f - o, fe = r.F[u];
         r.X[u] = x;
-        r.F[u] = fe;
-        r.A[u] = D + fo;
+        r.A[u] += D;
         r.O[u] = E * o;
         E *= ipowf(x, L);
         D = fmaf((float)L, fe, D);
@@ -501,6 +501,17 @@ __device__ __forceinline__ float window_conv_k(const float *CP, const float *CB,
     return v;
 }
 
+__host__ __device__ inline bool thm5_of(const DevParams &p) { return p.variant == FSMI_APPROX && p.approx_reading == 0; }
+// Which evaluation paths a 3D kernel is compiled with (each kernel holds as little as it can, for its registers and
+// the instruction cache): everything, with the variant and the ray's length read at run time; Theorem 5's sub-blocks;
+// the others (cell-level convolution and all run pairs) with a general or with a compiled-in radius
+// (conv_fixed).
+enum { kRay3dAny = 0, kRay3dThm5 = 1, kRay3dOther = 2, kRay3dFixed = 3 };
+__host__ __device__ inline int ray3d_mode(const DevParams &p)
+{
+    return thm5_of(p) ? kRay3dThm5 : conv_fixed(p.K) ? kRay3dFixed : kRay3dOther;
+}
+
 // The cells of a ray given as runs through scan_block: RI holds run u's index at its first cell and 0
 // elsewhere; with keep it receives every cell's run index.
 template <int CPL>
@@ -539,8 +550,9 @@ __device__ __forceinline__ void decompress(const DevParams &p, const float *O, i
 // (FSMI-RLE, Uniform-FSMI-RLE, strict-band Approx-FSMI-RLE), or for Theorem 5 the same sum over each
 // first-hit cell's window of kept pairs (window_conv). Each run's index is put at its first cell and
 // spread by a running maximum. Arrays: 0 run o, 3 P, 4 run starts S, 5 the cells' run indices, 6 C.
+template <int MODE, int CPL>
 static __device__ float ray_mi_cells(float *base, int stride, int nr, int n, const DevParams &p, const float *gtab,
-                                     const float *gz, const RleTable &t, int K, bool thm5)
+                                     const float *gz, const RleTable &t, int K)
 {
     const int lane = lane_id();
     const float *O = base;
@@ -551,16 +563,14 @@ static __device__ float ray_mi_cells(float *base, int stride, int nr, int n, con
     __syncwarp();
     for (int u = lane; u < nr; u += 32) RI[S[u]] = u;  // every run has a cell, so no two share one
     __syncwarp();
-    if (p.nmax > kShortRay)
-        decompress<4>(p, O, RI, n, CP, CB, thm5);
-    else
-        decompress<2>(p, O, RI, n, CP, CB, thm5);
+    decompress<CPL>(p, O, RI, n, CP, CB, MODE == kRay3dThm5);
     __syncwarp();
-    if (thm5) return window_conv(CP, CB, gtab, K, n, S, RI, p.trunc);
+    if (MODE == kRay3dThm5) return window_conv(CP, CB, gtab, K, n, S, RI, p.trunc);
     pad_conv(CB, K, n);
-    return band_conv<true, true>(CP, CB, gz, t, K, n);
+    return band_conv<MODE == kRay3dFixed, MODE == kRay3dOther>(CP, CB, gz, t, K, n);
 }
 
+template <int MODE, int CPL>
 __device__ __forceinline__ float ray_mi(float *base, int stride, int nr, const DevParams &p, const float2 *tab,
                                         const float *gtab, const float *gz, const RleTable &t, int K, bool have_s)
 {
@@ -568,13 +578,12 @@ __device__ __forceinline__ float ray_mi(float *base, int stride, int nr, const D
     const RunSmem r = run_smem(base, stride);
     run_starts(r, nr, have_s);
     const int n = r.S[nr];
-    const bool thm5 = p.variant == FSMI_APPROX && p.approx_reading == 0;
     float v;
     if (n < p.cell_runlen * nr) {
-        v = ray_mi_cells(base, stride, nr, n, p, gtab, gz, t, K, thm5);
+        v = ray_mi_cells<MODE, CPL>(base, stride, nr, n, p, gtab, gz, t, K);
     } else {
         run_prefixes(r, nr, p);
-        if (p.variant == FSMI_APPROX && p.approx_reading == 0)
+        if (MODE == kRay3dThm5)
             v = pairs_thm5(r, nr, tab, K, p.trunc);
         else
             v = pairs_all(r, nr, tab, K);
@@ -833,7 +842,6 @@ static __device__ int encode_cells(const float *CO, int n, int cap, float *O, in
 // run arrays sized for the runs the run-pair path can see: a ray takes that path only when
 // n >= cell_runlen * n_r, so n_r <= nmax / cell_runlen.
 
-__host__ __device__ inline bool thm5_of(const DevParams &p) { return p.variant == FSMI_APPROX && p.approx_reading == 0; }
 __host__ __device__ inline int ray3d_cell_stride(const DevParams &p) { return (p.nmax + conv_pad(p.K) + p.K + 12 + 3) & ~3; }
 __host__ __device__ inline int ray3d_nrcap(const DevParams &p)
 {
@@ -848,16 +856,6 @@ __host__ __device__ inline int ray3d_warp_floats(const DevParams &p)
 {
     return thm5_of(p) ? 2 * ray3d_run_stride(p) + 4 * ray3d_cell_stride(p)
                       : 3 * ray3d_cell_stride(p) + 6 * ray3d_run_stride(p);
-}
-
-// Which evaluation paths a fused-ray kernel is compiled with (each kernel holds as little as it can, for its
-// registers): everything, with the variant and the ray's length read at run time; Theorem 5's sub-blocks;
-// the others (cell-level convolution and all run pairs) with a general or with a compiled-in radius
-// (conv_fixed).
-enum { kRay3dAny = 0, kRay3dThm5 = 1, kRay3dOther = 2, kRay3dFixed = 3 };
-__host__ __device__ inline int ray3d_mode(const DevParams &p)
-{
-    return thm5_of(p) ? kRay3dThm5 : conv_fixed(p.K) ? kRay3dFixed : kRay3dOther;
 }
 
 // Samples and evaluates one ray in the warp's region `w` (ray3d_warp_floats floats); returns the MI
@@ -1036,7 +1034,8 @@ __device__ __forceinline__ void eval_ray_3d(const Vox3D &vx, const DevParams &p,
     __syncwarp();
 }
 
-// evaluation of one run-length-encoded ray given in CSR form
+// evaluation of one run-length-encoded ray given in CSR form (MODE, CPL as ray_mi_fused's, CPL by p.nmax)
+template <int MODE, int CPL>
 __device__ __forceinline__ void eval_ray_rle(const int32_t *__restrict__ off, const float *__restrict__ ro,
                                              const uint8_t *__restrict__ rl, const DevParams &p, const RleBlock &rb,
                                              const RleTable &t, int stride, long long ray, float *__restrict__ out, int *status)
@@ -1067,7 +1066,7 @@ __device__ __forceinline__ void eval_ray_rle(const int32_t *__restrict__ off, co
         __syncwarp();
         return;
     }
-    const float I = ray_mi(rb.base, stride, nr, p, rb.tab, rb.gtab, rb.gz, t, rb.ts.K, false);
+    const float I = ray_mi<MODE, CPL>(rb.base, stride, nr, p, rb.tab, rb.gtab, rb.gz, t, rb.ts.K, false);
     if (lane == 0) out[ray] = I;
     __syncwarp();
 }

@@ -28,6 +28,8 @@ static Eval3DKernel eval_3d_kernel(const DevParams &p, bool wide)
     return p.nmax > kShortRay ? k_eval_3d<MODE, 4, false> : k_eval_3d<MODE, 2, false>;
 }
 
+// As k_eval_3d for rays given as runs.
+template <int MODE, int CPL>
 __global__ void __launch_bounds__(kMaxWarps * 32)
     k_eval_rle(const int32_t *__restrict__ off, const float *__restrict__ ro, const uint8_t *__restrict__ rl,
                DevParams p, const __grid_constant__ RleTable tbl, long long nrays, int stride, float *__restrict__ out,
@@ -36,7 +38,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const RleBlock rb = rle_block(smem_raw, p, tbl, kArraysRLE * stride);
     for_each_item(nrays, queue, chunk,
-                  [&](long long ray) { eval_ray_rle(off, ro, rl, p, rb, tbl, stride, ray, out, status); });
+                  [&](long long ray) { eval_ray_rle<MODE, CPL>(off, ro, rl, p, rb, tbl, stride, ray, out, status); });
 }
 
 __global__ void __launch_bounds__(kWarpsRLE * 32)
@@ -256,19 +258,24 @@ cudaError_t launch_eval_rle(const int32_t *run_off, const float *run_o, const ui
 {
     if (nrays <= 0) return cudaSuccess;
     const Schedule &sc = current_schedule(FSMI_KIND_RLE);
+    const int mode = ray3d_mode(p);
+    const bool longer = p.nmax > kShortRay;
+    const auto kern = mode == kRay3dThm5    ? (longer ? k_eval_rle<kRay3dThm5, 4> : k_eval_rle<kRay3dThm5, 2>)
+                      : mode == kRay3dFixed ? (longer ? k_eval_rle<kRay3dFixed, 4> : k_eval_rle<kRay3dFixed, 2>)
+                                            : (longer ? k_eval_rle<kRay3dOther, 4> : k_eval_rle<kRay3dOther, 2>);
     const int stride = rle_stride(p.nmax, p.K);
     const size_t per_warp = (size_t)kArraysRLE * stride * sizeof(float);
     const int wpb = fit_warps(sc.warps_per_block, per_warp, rle_table_bytes(p.K));
     const size_t smem = rle_table_bytes(p.K) + (size_t)wpb * per_warp;
     WarpGrid g;
-    cudaError_t e = warp_grid((const void *)k_eval_rle, nrays, wpb, smem, sc.blocks_per_sm, g);
+    cudaError_t e = warp_grid((const void *)kern, nrays, wpb, smem, sc.blocks_per_sm, g);
     if (e == cudaSuccess && g.one_each) queue = nullptr;
     if (e == cudaSuccess) e = reset_queue(queue, s);
     if (e != cudaSuccess) return e;
     RleTable tbl;
     fill_rle_table(p, tbl);
-    k_eval_rle<<<g.grid, wpb * 32, smem, s>>>(run_off, run_o, run_len, p, tbl, nrays, stride, out, status,
-                                                      queue, sc.queue_chunk > 0 ? sc.queue_chunk : 1);
+    kern<<<g.grid, wpb * 32, smem, s>>>(run_off, run_o, run_len, p, tbl, nrays, stride, out, status, queue,
+                                        sc.queue_chunk > 0 ? sc.queue_chunk : 1);
     return cudaGetLastError();
 }
 
@@ -319,12 +326,14 @@ int32_t *g_scratch_ptr[64];
 cudaError_t encode_scratch_ptr(int32_t **ptr);
 
 template <int MODE>
-static cudaError_t prepare_eval_3d()
+static cudaError_t prepare_rays()
 {
     cudaFuncAttributes a;
     cudaError_t e = cudaFuncGetAttributes(&a, k_eval_3d<MODE, 4, false>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_3d<MODE, 2, false>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_3d<MODE, 0, true>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_rle<MODE, 4>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_rle<MODE, 2>);
     return e;
 }
 
@@ -332,10 +341,9 @@ static cudaError_t prepare_eval_3d()
 cudaError_t prepare_rle()
 {
     cudaFuncAttributes a;
-    cudaError_t e = prepare_eval_3d<kRay3dThm5>();
-    if (e == cudaSuccess) e = prepare_eval_3d<kRay3dFixed>();
-    if (e == cudaSuccess) e = prepare_eval_3d<kRay3dOther>();
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_rle);
+    cudaError_t e = prepare_rays<kRay3dThm5>();
+    if (e == cudaSuccess) e = prepare_rays<kRay3dFixed>();
+    if (e == cudaSuccess) e = prepare_rays<kRay3dOther>();
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_rle_count);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_rle_write);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_scan_tiles);
