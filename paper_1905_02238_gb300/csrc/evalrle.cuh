@@ -27,30 +27,31 @@
 
 namespace fsmi {
 
-// Gains f(delta_occ, o) and f(delta_emp, o) of one cell: the host-fitted polynomials of h(o) = f / (o (1 - o))
-// where they are accurate for these deltas (both together in packed FP32, Horner's rule), else the closed
-// forms.
-__device__ __forceinline__ void rle_gains(const DevParams &p, float o, float &fo, float &fe)
+// Gains f(delta_occ, o) and f(delta_emp, o) of one cell: the host-fitted polynomials of h(o) = f / (o (1 - o)),
+// both together in packed FP32, Horner's rule (TERMS agrees with p.gain_fit).
+template <int TERMS>
+__device__ __forceinline__ void poly_gains(const DevParams &p, float o, float &fo, float &fe)
 {
-    if (!p.gain_fit) {
-        fo = cell_gain(p.docc, o);
-        fe = cell_gain(p.demp, o);
-        return;
-    }
     const float x = __fmaf_rn(2.0f, o, -1.0f);
     const f32x2 X = pack2(x, x);
-    f32x2 h;
-    if (p.gain_fit == 2) {
-        h = pack2(p.gfit2[kGainShortTerms - 1][0], p.gfit2[kGainShortTerms - 1][1]);
+    f32x2 h = pack2(p.gfit2[TERMS - 1][0], p.gfit2[TERMS - 1][1]);
 #pragma unroll
-        for (int k = kGainShortTerms - 2; k >= 0; --k) h = fma2(h, X, pack2(p.gfit2[k][0], p.gfit2[k][1]));
-    } else {
-        h = pack2(p.gfit2[kGainFitTerms - 1][0], p.gfit2[kGainFitTerms - 1][1]);
-#pragma unroll
-        for (int k = kGainFitTerms - 2; k >= 0; --k) h = fma2(h, X, pack2(p.gfit2[k][0], p.gfit2[k][1]));
-    }
+    for (int k = TERMS - 2; k >= 0; --k) h = fma2(h, X, pack2(p.gfit2[k][0], p.gfit2[k][1]));
     const float w = __fmul_rn(o, __fsub_rn(1.0f, o));
     unpack2(mul2(pack2(w, w), h), fo, fe);
+}
+
+// The polynomials where they are accurate for these deltas, else the closed forms.
+__device__ __forceinline__ void rle_gains(const DevParams &p, float o, float &fo, float &fe)
+{
+    if (p.gain_fit == 2) {
+        poly_gains<kGainShortTerms>(p, o, fo, fe);
+    } else if (p.gain_fit) {
+        poly_gains<kGainFitTerms>(p, o, fo, fe);
+    } else {
+        fo = cell_gain(p.docc, o);
+        fe = cell_gain(p.demp, o);
+    }
 }
 
 // C keeps its first cell at a 16-byte boundary, conv_pad(K) >= K floats after its array's start; four outputs
@@ -285,15 +286,61 @@ struct CellScan {
 // cells per lane: rays of at most 64 samples go in one block of 64, so that half the lanes' work is not idle
 constexpr int kShortRay = 64;
 
-// One block of 32 CPL cells (CPL = 4, or 2 on short rays): o of this lane's cells i0 .. i0 + CPL - 1 (zero from
-// the ray's end on); stores P in CP and C in CB where i0 < n.
+// Closed-form gains of a block's cells, once per span of equal values: the spans' values are listed in the block's
+// part of CP, one lane evaluates each, and the cells read their span's pair back (CP, CB: scan_block writes there
+// next). Two logarithms and a division per gain cost too much to repeat per cell (256x256x64 voxels without noise,
+// 16 x 64x64 rays of 200 samples, delta 40 and 0.02: 196 us per cell, 159 us so; with noise 103 and 80 us).
 template <int CPL>
+__device__ __forceinline__ void closed_gains(const DevParams &p, const float (&o)[CPL], int i0, int n, float *CP, float *CB,
+                                             float (&fo)[CPL], float (&fe)[CPL])
+{
+    const int lane = lane_id(), b0 = i0 - CPL * lane;
+    const unsigned left = __shfl_up_sync(kFull, __float_as_uint(o[CPL - 1]), 1);
+    int id[CPL], cnt = 0;
+#pragma unroll
+    for (int t = 0; t < CPL; ++t) {
+        const unsigned before = t ? __float_as_uint(o[t > 0 ? t - 1 : 0]) : left;
+        id[t] = i0 + t < n && (__float_as_uint(o[t]) != before || (t == 0 && lane == 0));
+        cnt += id[t];
+    }
+    const int incl = warp_incl_add_int(cnt), total = __shfl_sync(kFull, incl, 31);
+    int k = incl - cnt - 1;
+#pragma unroll
+    for (int t = 0; t < CPL; ++t) {
+        if (id[t]) CP[b0 + ++k] = o[t];
+        id[t] = k;
+    }
+    __syncwarp();
+    for (int j = b0 + lane; j < b0 + total; j += 32) {
+        const float v = CP[j];
+        CP[j] = cell_gain(p.docc, v);
+        CB[j] = cell_gain(p.demp, v);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < CPL; ++t) {
+        fo[t] = i0 + t < n ? CP[b0 + id[t]] : 0.0f;
+        fe[t] = i0 + t < n ? CB[b0 + id[t]] : 0.0f;
+    }
+    __syncwarp();
+}
+
+// One block of 32 CPL cells (CPL = 4, or 2 on short rays): o of this lane's cells i0 .. i0 + CPL - 1 (zero from
+// the ray's end on); stores P in CP and C in CB where i0 < n. POLY: only for deltas with polynomial gains.
+template <int CPL, bool POLY>
 __device__ __forceinline__ void scan_block(const DevParams &p, const float (&o)[CPL], int i0, int n, CellScan &s, float *CP,
                                            float *CB)
 {
     float fo[CPL], fe[CPL];
+    if (p.gain_fit == 2) {
 #pragma unroll
-    for (int t = 0; t < CPL; ++t) rle_gains(p, o[t], fo[t], fe[t]);
+        for (int t = 0; t < CPL; ++t) poly_gains<kGainShortTerms>(p, o[t], fo[t], fe[t]);
+    } else if (POLY || p.gain_fit) {
+#pragma unroll
+        for (int t = 0; t < CPL; ++t) poly_gains<kGainFitTerms>(p, o[t], fo[t], fe[t]);
+    } else {
+        closed_gains<CPL>(p, o, i0, n, CP, CB, fo, fe);
+    }
     float prod = (1.0f - o[0]) * (1.0f - o[1]), sum = fe[0] + fe[1];
     if (CPL == 4) {
         prod = (prod * (1.0f - o[CPL - 2])) * (1.0f - o[CPL - 1]);  // cell by cell, see cell_prefixes
@@ -514,7 +561,7 @@ __host__ __device__ inline int ray3d_mode(const DevParams &p)
 
 // The cells of a ray given as runs through scan_block: RI holds run u's index at its first cell and 0
 // elsewhere; with keep it receives every cell's run index.
-template <int CPL>
+template <int CPL, bool POLY>
 __device__ __forceinline__ void decompress(const DevParams &p, const float *O, int *RI, int n, float *CP, float *CB, bool keep)
 {
     const int lane = lane_id();
@@ -541,7 +588,7 @@ __device__ __forceinline__ void decompress(const DevParams &p, const float *O, i
             o[t] = i0 + t < n ? O[u[t]] : 0.0f;
         }
         if (keep && i0 < n) store_cells(RI + i0, u);
-        scan_block<CPL>(p, o, i0, n, s, CP, CB);
+        scan_block<CPL, POLY>(p, o, i0, n, s, CP, CB);
     }
 }
 
@@ -563,7 +610,10 @@ static __device__ float ray_mi_cells(float *base, int stride, int nr, int n, con
     __syncwarp();
     for (int u = lane; u < nr; u += 32) RI[S[u]] = u;  // every run has a cell, so no two share one
     __syncwarp();
-    decompress<CPL>(p, O, RI, n, CP, CB, MODE == kRay3dThm5);
+    if (CPL == 4 || (CPL == 0 && p.nmax > kShortRay))
+        decompress<4, CPL != 0>(p, O, RI, n, CP, CB, MODE == kRay3dThm5);
+    else
+        decompress<2, CPL != 0>(p, O, RI, n, CP, CB, MODE == kRay3dThm5);
     __syncwarp();
     if (MODE == kRay3dThm5) return window_conv(CP, CB, gtab, K, n, S, RI, p.trunc);
     pad_conv(CB, K, n);
@@ -743,7 +793,7 @@ __device__ __forceinline__ void encode_block(const float (&o)[CPL], const bool (
 // instructions per ray and 1,690 to 1,136 us, with the convolution below (73 registers, 28 warps per SM; held
 // to 64: 1,152 - 1,172 us), then 1,103 us with a kernel per path and ray length (77 registers, 24 warps); Theorem 5
 // on 301x253x77 voxels, 23 x 80x61 rays: 162 to 150 us in all.
-template <int CPL, bool ENC>
+template <int CPL, bool ENC, bool POLY>
 __device__ __forceinline__ int sample_cells(const float *__restrict__ vox, int X, int Y, int Z, const int32_t *pose,
                                             const int32_t *u, int nsamp, const DevParams &p, float *CP, float *CB, float *CO,
                                             float *O, int *S, int nrcap, int *RI, int &count)
@@ -793,7 +843,7 @@ __device__ __forceinline__ int sample_cells(const float *__restrict__ vox, int X
             encode_block<CPL>(o, nw, i0, n, p.run_cap, inv_cap, rs, O, S, nrcap, RI);
         else if (i0 < n)
             store_cells(CO + i0, o);
-        scan_block<CPL>(p, o, i0, n, s, CP, CB);
+        scan_block<CPL, POLY>(p, o, i0, n, s, CP, CB);
         if (m != kFull) break;
     }
     if (ENC) {
@@ -862,7 +912,8 @@ __host__ __device__ inline int ray3d_warp_floats(const DevParams &p)
 // (warp-reduced) and, with nr_out, the run count. MODE must agree with ray3d_mode(p). Outside Theorem 5 the runs are
 // formed (from the sampled values in shared memory) only where they are needed: for a caller who asks for
 // their number, or on a ray whose spans of equal values do not already show that its mean run is short.
-// CPL: cells per lane of a block, 2 for rays of at most kShortRay samples, else 4 (0: read at run time).
+// CPL: cells per lane of a block, 2 for rays of at most kShortRay samples, else 4, both for polynomial gains only (the
+// closed forms' code takes registers from every ray); 0: ray length and gains read at run time.
 template <int MODE, int CPL>
 __device__ __forceinline__ float ray_mi_fused(const float *vox, int X, int Y, int Z, const int32_t *pose,
                                               const int32_t *u, int nsamp, const DevParams &p, const float2 *tab,
@@ -896,14 +947,14 @@ __device__ __forceinline__ float ray_mi_fused(const float *vox, int X, int Y, in
     bool cells;
     if (thm5) {
         n = CPL == 4 || (CPL == 0 && nsamp > kShortRay)
-                ? sample_cells<4, true>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, r.O, r.S, ray3d_nrcap(p), RI, nr)
-                : sample_cells<2, true>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, r.O, r.S, ray3d_nrcap(p), RI, nr);
+                ? sample_cells<4, true, CPL != 0>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, r.O, r.S, ray3d_nrcap(p), RI, nr)
+                : sample_cells<2, true, CPL != 0>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, r.O, r.S, ray3d_nrcap(p), RI, nr);
         cells = n < p.cell_runlen * nr;
     } else {
         int nspan;
         n = CPL == 4 || (CPL == 0 && nsamp > kShortRay)
-                ? sample_cells<4, false>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, nullptr, nullptr, 0, nullptr, nspan)
-                : sample_cells<2, false>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, nullptr, nullptr, 0, nullptr, nspan);
+                ? sample_cells<4, false, CPL != 0>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, nullptr, nullptr, 0, nullptr, nspan)
+                : sample_cells<2, false, CPL != 0>(vox, X, Y, Z, pose, u, nsamp, p, CP, CB, CO, nullptr, nullptr, 0, nullptr, nspan);
         cells = n < p.cell_runlen * nspan;  // at least one run per span
         if (n > 0 && (nr_out || !cells)) {
             nr = encode_cells(CO, n, p.run_cap, r.O, r.S, ray3d_nrcap(p));

@@ -25,8 +25,8 @@ static_assert(kMixBuckets <= 32, "the plan warp keeps one class per lane");
 static_assert(kMixBuckets * sizeof(unsigned long long) <= kQueueBytes, "a queue counter per class");
 // which kinds a launch of k_eval_mixed takes: both (the single launch), or one class's kind, 3D with
 // the evaluation path its variant uses (as fsmi_eval_3d compiles one kernel per path)
-enum { kMixAny = 0, kMix2D = 1, kMix3D = 2 };  // kMix3D + ray3d_mode: 3D on that path; + kMixShort: short rays
-constexpr int kMixShort = 16;
+enum { kMixAny = 0, kMix2D = 1, kMix3D = 2 };  // kMix3D + ray3d_mode: 3D on that path; + kMixShort: short rays,
+constexpr int kMixShort = 16, kMixClosed = 32;  // or + kMixClosed: any length, gains in closed form
 
 // the set holding item i (sets sorted by out_offset), or -1
 __device__ __forceinline__ int mixed_set_of(const fsmi_set *sets, int nsets, long long i)
@@ -319,8 +319,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4)
                     bad = FSMI_STATUS_BEAM_OVERFLOW;
                 }
             } else {
-                constexpr bool kShort = KIND >= kMixShort;
-                I = ray_mi_fused<KIND - kMix3D - (kShort ? kMixShort : 0), kShort ? 2 : 4>(cc->vox, cc->X, cc->Y, cc->Z, cc->pose + 12 * kp, cc->dir + 3 * kd, cc->nsamp, p3,
+                constexpr int kCells = KIND >= kMixClosed ? 0 : KIND >= kMixShort ? 2 : 4;
+                I = ray_mi_fused<KIND % kMixShort - kMix3D, kCells>(cc->vox, cc->X, cc->Y, cc->Z, cc->pose + 12 * kp, cc->dir + 3 * kd, cc->nsamp, p3,
                                         rb.tab, rb.gtab, rb.gz, tbl, rb.ts.K, base, nullptr);
             }
             __syncwarp();
@@ -457,6 +457,9 @@ cudaError_t launch_mixed_planned(const MixedSrc &src, const DevParams &d2, const
             // include kShortRay, so a class holds short rays only or none)
             auto go = [&](auto mode) {
                 constexpr int K3 = kMix3D + decltype(mode)::value;
+                if (!p.gain_fit)
+                    return launch_mixed_variant<FSMI_EXACT, K3 + kMixClosed>(sc3, n2, p, nitems, out, times, status, queue, s,
+                                                                           plan, kMixClasses + c, early);
                 return p.nmax > kShortRay ? launch_mixed_variant<FSMI_EXACT, K3>(sc3, n2, p, nitems, out, times, status,
                                                                                queue, s, plan, kMixClasses + c, early)
                                           : launch_mixed_variant<FSMI_EXACT, K3 + kMixShort>(
@@ -529,6 +532,7 @@ static cudaError_t prepare_mixed_3d()
     cudaFuncAttributes a;
     cudaError_t e = cudaFuncGetAttributes(&a, k_eval_mixed<FSMI_EXACT, kMix3D + MODE>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_mixed<FSMI_EXACT, kMix3D + MODE + kMixShort>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_mixed<FSMI_EXACT, kMix3D + MODE + kMixClosed>);
     return e;
 }
 

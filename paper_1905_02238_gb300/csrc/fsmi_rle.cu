@@ -8,9 +8,12 @@ namespace fsmi {
 
 // MODE, CPL: the paths of the call's variant and radius and its rays' length (the launcher picks them by
 // ray3d_mode(p) and kShortRay), so that each kernel holds only what it can take; WIDE for batches of more than
-// 2^31 - 1 rays (a 64-bit ray index division, which costs the others registers).
+// 2^31 - 1 rays (a 64-bit ray index division, which costs the others registers) and, with CPL = 0, for deltas
+// whose gains take the closed forms. The bound of 128 registers of the compiled-in radii's kernel is there for what the
+// compiler makes of it: 77 registers and 1,114 us for radius 15 on the 512x512x128 batch; 63 registers and 1,456 us
+// without a bound, 80 and 1,159 us with one of 80 (box of H = 4: 1,007 / 996 / 1,056 us).
 template <int MODE, int CPL, bool WIDE>
-__global__ void __launch_bounds__(kMaxWarps * 32)
+__global__ void __launch_bounds__(kMaxWarps * 32, MODE == kRay3dFixed && CPL == 4 ? 2 : 0)
     k_eval_3d(Vox3D vx, DevParams p, const __grid_constant__ RleTable tbl, long long nrays, int warp_floats,
               float *__restrict__ out, int32_t *__restrict__ nruns, unsigned long long *queue, int chunk)
 {
@@ -24,7 +27,7 @@ using Eval3DKernel = void (*)(Vox3D, DevParams, const RleTable, long long, int, 
 template <int MODE>
 static Eval3DKernel eval_3d_kernel(const DevParams &p, bool wide)
 {
-    if (wide) return k_eval_3d<MODE, 0, true>;
+    if (wide || !p.gain_fit) return k_eval_3d<MODE, 0, true>;
     return p.nmax > kShortRay ? k_eval_3d<MODE, 4, false> : k_eval_3d<MODE, 2, false>;
 }
 
@@ -39,6 +42,16 @@ __global__ void __launch_bounds__(kMaxWarps * 32)
     const RleBlock rb = rle_block(smem_raw, p, tbl, kArraysRLE * stride);
     for_each_item(nrays, queue, chunk,
                   [&](long long ray) { eval_ray_rle<MODE, CPL>(off, ro, rl, p, rb, tbl, stride, ray, out, status); });
+}
+
+using EvalRleKernel = void (*)(const int32_t *, const float *, const uint8_t *, DevParams, const RleTable, long long, int,
+                               float *, int *, unsigned long long *, int);
+
+template <int MODE>
+static EvalRleKernel eval_rle_kernel(const DevParams &p)
+{
+    if (!p.gain_fit) return k_eval_rle<MODE, 0>;
+    return p.nmax > kShortRay ? k_eval_rle<MODE, 4> : k_eval_rle<MODE, 2>;
 }
 
 __global__ void __launch_bounds__(kWarpsRLE * 32)
@@ -259,10 +272,9 @@ cudaError_t launch_eval_rle(const int32_t *run_off, const float *run_o, const ui
     if (nrays <= 0) return cudaSuccess;
     const Schedule &sc = current_schedule(FSMI_KIND_RLE);
     const int mode = ray3d_mode(p);
-    const bool longer = p.nmax > kShortRay;
-    const auto kern = mode == kRay3dThm5    ? (longer ? k_eval_rle<kRay3dThm5, 4> : k_eval_rle<kRay3dThm5, 2>)
-                      : mode == kRay3dFixed ? (longer ? k_eval_rle<kRay3dFixed, 4> : k_eval_rle<kRay3dFixed, 2>)
-                                            : (longer ? k_eval_rle<kRay3dOther, 4> : k_eval_rle<kRay3dOther, 2>);
+    const EvalRleKernel kern = mode == kRay3dThm5    ? eval_rle_kernel<kRay3dThm5>(p)
+                               : mode == kRay3dFixed ? eval_rle_kernel<kRay3dFixed>(p)
+                                                     : eval_rle_kernel<kRay3dOther>(p);
     const int stride = rle_stride(p.nmax, p.K);
     const size_t per_warp = (size_t)kArraysRLE * stride * sizeof(float);
     const int wpb = fit_warps(sc.warps_per_block, per_warp, rle_table_bytes(p.K));
@@ -334,6 +346,7 @@ static cudaError_t prepare_rays()
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_3d<MODE, 0, true>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_rle<MODE, 4>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_rle<MODE, 2>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_eval_rle<MODE, 0>);
     return e;
 }
 
