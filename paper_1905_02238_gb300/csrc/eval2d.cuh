@@ -67,6 +67,10 @@ __host__ __device__ constexpr bool mass_variant(int v) { return v == kExactMass3
 // 274 us in mass form, 250 us in boundary form). The exact sum of the 2048x2048 office batch (1024
 // poses x 360 beams, R = 256, sigma = 2) took 1.69 ms in mass form, 1.86 ms in boundary form, both before the
 // traversal in closed form and with a cut of 4.58 for the masses (1.72 ms with both and the present cuts).
+// From sigma = 1 to 1.5 the degree-4 form is kept for its error, not its time: 512 poses on the same map at sigma 1.0 /
+// 1.2 / 1.45 take 759 / 796 / 850 us, in boundary form 688 / 743 / 801 us, but on random cells at 1.49 its largest error is
+// 7.1e-7 against 1.8e-6. At sigma 1.5 and 2 the degree-3 form takes 777 and 875 us (boundary form 819 and 943, before the
+// traversal in closed form).
 inline int grid_variant(const DevParams &p)
 {
     if (p.variant != FSMI_EXACT) return p.variant;

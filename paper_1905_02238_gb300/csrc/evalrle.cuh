@@ -475,10 +475,10 @@ __device__ __forceinline__ float band_conv_any(const float *CP, const float *CB,
 }
 
 // radii with a compiled-in convolution: Gaussian kernels at sigma = 1.88 .. 2.01 cells, the strict band of Delta = 6,
-// the box of H = 4. A neighbouring radius in the general form costs 0 to 10 % more, 512x512x128 voxels, 64 x
-// 128x128 rays: sigma 1.0 / 1.5 / 1.9 / 2.0 / 2.1 / 3.0 in 1,113 / 1,170 / 1,119 / 1,121 / 1,219 / 1,330 us (one
+// the box of H = 4. A neighbouring radius in the general form costs 0 to 7 % more, 512x512x128 voxels, 64 x
+// 128x128 rays: sigma 1.0 / 1.5 / 1.9 / 2.0 / 2.1 / 3.0 in 1,066 / 1,126 / 1,114 / 1,114 / 1,189 / 1,307 us (one
 // output per lane and one load per tap, before: 1,700 / 1,811 / 1,701 / 1,703 / 1,941 / 2,245); box of H 3 / 4 / 5
-// in 1,018 / 1,010 / 1,110 us.
+// in 1,008 / 1,006 / 1,066 us.
 __host__ __device__ constexpr bool conv_fixed(int K) { return K == 15 || K == 6 || K == 4; }
 
 // FIXED / ANY: whether the kernel holds the compiled-in radii and the general form
@@ -791,7 +791,7 @@ __device__ __forceinline__ void encode_block(const float (&o)[CPL], const bool (
 // from the spans through shared memory, and six array accesses; a block of 128 pays the warp-wide steps
 // once and stores three 16-byte words. 512x512x128 voxels, 64 poses x 128x128 rays: 1,741 to 1,068 warp
 // instructions per ray and 1,690 to 1,136 us, with the convolution below (73 registers, 28 warps per SM; held
-// to 64: 1,152 - 1,172 us), then 1,103 us with a kernel per path and ray length (77 registers, 24 warps); Theorem 5
+// to 64: 1,152 - 1,172 us), then 1,103 us with a kernel per path and ray length (80 registers, 24 warps); Theorem 5
 // on 301x253x77 voxels, 23 x 80x61 rays: 162 to 150 us in all.
 template <int CPL, bool ENC, bool POLY>
 __device__ __forceinline__ int sample_cells(const float *__restrict__ vox, int X, int Y, int Z, const int32_t *pose,

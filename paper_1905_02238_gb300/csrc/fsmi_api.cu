@@ -286,7 +286,7 @@ int sm_count()
     return g_sms[dev];
 }
 
-cudaError_t resident_blocks(const void *kern, int threads, size_t smem, int &blocks)
+cudaError_t resident_blocks(const void *kern, int threads, size_t smem, int &blocks, int carveout)
 {
     struct Entry {
         const void *kern;
@@ -308,6 +308,8 @@ cudaError_t resident_blocks(const void *kern, int threads, size_t smem, int &blo
     // every caller sets the same limit, so that no thread lowers it under another's launch
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
+    if (e == cudaSuccess && carveout >= 0)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, threads, smem);
     if (e != cudaSuccess) return e;
     if (blocks < 1) return cudaErrorInvalidConfiguration;
@@ -315,10 +317,10 @@ cudaError_t resident_blocks(const void *kern, int threads, size_t smem, int &blo
     return cudaSuccess;
 }
 
-cudaError_t warp_grid(const void *kern, long long n, int wpb, size_t smem, int max_blocks_per_sm, WarpGrid &g)
+cudaError_t warp_grid(const void *kern, long long n, int wpb, size_t smem, int max_blocks_per_sm, WarpGrid &g, int carveout)
 {
     int occ = 0;
-    cudaError_t e = resident_blocks(kern, wpb * 32, smem, occ);
+    cudaError_t e = resident_blocks(kern, wpb * 32, smem, occ, carveout);
     if (e != cudaSuccess) return e;
     if (max_blocks_per_sm > 0 && max_blocks_per_sm < occ) occ = max_blocks_per_sm;
     const long long want = (n + wpb - 1) / wpb, fit = (long long)sm_count() * occ;

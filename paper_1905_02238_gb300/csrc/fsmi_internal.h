@@ -71,7 +71,8 @@ struct WarpGrid {
     unsigned grid;
     bool one_each;  // a warp for every item: static assignment gives each warp at most one, a queue nothing
 };
-cudaError_t warp_grid(const void *kern, long long n, int wpb, size_t smem, int max_blocks_per_sm, WarpGrid &g);
+cudaError_t warp_grid(const void *kern, long long n, int wpb, size_t smem, int max_blocks_per_sm, WarpGrid &g,
+                      int carveout = -1);
 
 // Bytes at the front of an evaluation workspace reserved for the work-queue counter.
 constexpr size_t kQueueBytes = 256;
@@ -146,8 +147,8 @@ cudaError_t launch_kernel(bool early, void (*kern)(P...), dim3 grid, unsigned th
 // Resident blocks per SM of `kern` with `threads` threads and `smem` bytes of dynamic shared memory on the
 // current device, its dynamic shared memory limit raised to the device's maximum. Looked up once per
 // kernel, block size and device and remembered per host thread (the attribute and occupancy calls were 4 of the
-// 10 us of a launch).
-cudaError_t resident_blocks(const void *kern, int threads, size_t smem, int &blocks);
+// 10 us of a launch). carveout >= 0: the share of shared memory, in percent, that the kernel prefers.
+cudaError_t resident_blocks(const void *kern, int threads, size_t smem, int &blocks, int carveout = -1);
 // records e as the calling thread's last CUDA error and returns FSMI_ERR_CUDA
 fsmi_status record_cuda_error(cudaError_t e);
 // poll limit of the surrogate fc kernel's epilogue wait for this host thread (< 0: the default)

@@ -9,9 +9,8 @@ namespace fsmi {
 // MODE, CPL: the paths of the call's variant and radius and its rays' length (the launcher picks them by
 // ray3d_mode(p) and kShortRay), so that each kernel holds only what it can take; WIDE for batches of more than
 // 2^31 - 1 rays (a 64-bit ray index division, which costs the others registers) and, with CPL = 0, for deltas
-// whose gains take the closed forms. The bound of 128 registers of the compiled-in radii's kernel is there for what the
-// compiler makes of it: 77 registers and 1,114 us for radius 15 on the 512x512x128 batch; 63 registers and 1,456 us
-// without a bound, 80 and 1,159 us with one of 80 (box of H = 4: 1,007 / 996 / 1,056 us).
+// whose gains take the closed forms. The compiled-in radii's kernel may use 128 registers (it takes 80): left to itself
+// the compiler stops at 63, which costs rays of long runs 5 % (256x256x64 voxels without noise, 143 against 137 us).
 template <int MODE, int CPL, bool WIDE>
 __global__ void __launch_bounds__(kMaxWarps * 32, MODE == kRay3dFixed && CPL == 4 ? 2 : 0)
     k_eval_3d(Vox3D vx, DevParams p, const __grid_constant__ RleTable tbl, long long nrays, int warp_floats,
@@ -21,6 +20,15 @@ __global__ void __launch_bounds__(kMaxWarps * 32, MODE == kRay3dFixed && CPL == 
     const RleBlock rb = rle_block(smem_raw, p, tbl, warp_floats);
     for_each_item(nrays, queue, chunk, [&](long long ray) { eval_ray_3d<MODE, CPL, WIDE>(vx, p, rb, tbl, ray, out, nruns); });
 }
+
+// Shared memory asked for k_eval_3d on rays longer than kShortRay, in percent of 228 KB (164 KB, which leaves the gathers
+// 92 KB of L1), by the kernels of at most 64 registers (all but the compiled-in radii's: 1,129 us with it, 1,114 without). Without a wish 32 warps of 64 registers get all of it once the convolution's radius reaches 15, 28 KB of
+// L1 stay, and the 512x512x128 batch takes 1,535 us at radius 16 and 1,613 at 23; so 1,191 and 1,308 us, at radius 8
+// and 12 (whose cells fitted 196 KB by themselves) 1,068 and 1,130. Kernels of 69 registers and fewer warps, as the
+// closed forms' code made them: 1,213, 1,326, 1,104 and 1,164 us. Short rays' cells are few: 645 us without the
+// wish (64 samples), 657 us with it.
+constexpr int kCarveout3D = 72;
+
 
 using Eval3DKernel = void (*)(Vox3D, DevParams, const RleTable, long long, int, float *, int32_t *, unsigned long long *, int);
 
@@ -255,7 +263,8 @@ cudaError_t launch_eval_3d(const Vox3D &v, const DevParams &p, float *out, int32
     const Eval3DKernel kern = mode == kRay3dThm5    ? eval_3d_kernel<kRay3dThm5>(p, wide)
                               : mode == kRay3dFixed ? eval_3d_kernel<kRay3dFixed>(p, wide)
                                                     : eval_3d_kernel<kRay3dOther>(p, wide);
-    cudaError_t e = warp_grid((const void *)kern, nrays, wpb, smem, sc.blocks_per_sm, g);
+    cudaError_t e = warp_grid((const void *)kern, nrays, wpb, smem, sc.blocks_per_sm, g,
+                              p.nmax > kShortRay && mode != kRay3dFixed ? kCarveout3D : -1);
     if (e == cudaSuccess && g.one_each) queue = nullptr;  // nothing to balance
     if (e == cudaSuccess) e = reset_queue(queue, s);
     if (e != cudaSuccess) return e;
